@@ -480,7 +480,8 @@ cudaError_t launch_attention(const AttnParams &p0, cudaStream_t s) {
     const int Tg = p.nw > 1 ? (p.grid_side / p.nw) * (p.grid_side / p.nw) : p.T;
     if (p.B == 0 || Tg == 0) return cudaSuccess;
     if (attention_tc_enabled()) {
-        const cudaError_t e = launch_attention_tc(p, s);
+        cudaError_t e = launch_attention_res(p, s);
+        if (e == cudaErrorNotSupported) e = launch_attention_tc(p, s);
         if (e != cudaErrorNotSupported) return e;
     }
     dim3 grid((Tg + QT - 1) / QT, p.H, p.B * G2);

@@ -43,11 +43,9 @@
 // Every mbarrier wait is bounded (about one second); on expiry the kernel latches the device status
 // word, every role stops, the loaders drain their copies and the TMEM is freed after every MMA
 // issued has completed.
-#include <cuda.h>
-
 #include <cstdint>
-#include <mutex>
 
+#include "attn_ptx.cuh"
 #include "ilw_kernels.h"
 
 namespace ilw {
@@ -85,7 +83,6 @@ static_assert(NS * TKB <= kTmemCols && TKB + 128 <= kTmemCols, "TMEM columns");
 constexpr int NLOAD = 96;        // q loader threads (warps 1-3)
 constexpr int NSMX = 128 * NCQ;  // softmax threads (warps 4 ..)
 constexpr int kThreadsTc = 128 + NSMX;
-constexpr long long kWaitTc = 2000000000ll;  // ~1 s at 2 GHz
 
 struct TcSmem {  // offsets from the 1024-aligned base
     static constexpr int kQ = 0;
@@ -104,126 +101,6 @@ struct TcSmem {  // offsets from the 1024-aligned base
     static constexpr int kSlot = kBar + 8 * kNBar;  // TMEM address, abort flag
     static constexpr int kBytes = kSlot + 16;
 };
-
-__device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void bar_init(uint32_t b, uint32_t n) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(b), "r"(n) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(uint32_t b) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
-}
-__device__ __forceinline__ bool bar_try(uint32_t b, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred P;\n mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2, %3;\n selp.b32 %0, 1, 0, P;\n}\n"
-        : "=r"(ok)
-        : "r"(b), "r"(parity), "r"(20000)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait: false (after latching `code` and raising the abort flag) when it ran out, or when
-// another role already aborted.
-__device__ __forceinline__ bool bar_wait(uint32_t b, uint32_t parity, volatile int *abort, int *status, int code) {
-    if (bar_try(b, parity)) return true;
-    const long long t0 = clock64();
-    for (uint32_t i = 0;; ++i) {
-        if (bar_try(b, parity)) return true;
-        if ((i & 63) == 63) {
-            if (*abort) return false;
-            if (clock64() - t0 > kWaitTc) {
-                if (status) atomicExch(status, code);
-                *abort = 1;
-                return false;
-            }
-        }
-    }
-}
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void commit(uint32_t b) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(b) : "memory");
-}
-// 128-byte swizzled operand: 8-row groups 1024 bytes apart (K-major rows of 128 B, or, for the
-// N-major V operand, rows of 128 B along N with 8-row groups along K)
-__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-// 32-byte swizzled K-major operand of K = 16: rows of 32 bytes, 8-row groups 256 bytes apart
-__device__ __forceinline__ uint64_t desc_sw32(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(256 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)6 << 61;
-    return d;
-}
-__device__ __forceinline__ void mma(uint32_t dt, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-// TMEM load of N = 16 or 32 consecutive 32-bit columns of this thread's lane.
-template <int N>
-__device__ __forceinline__ void tld(uint32_t taddr, uint32_t (&v)[N]) {
-    if constexpr (N == 32) {
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-              "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-              "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-              "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-            : "r"(taddr));
-    } else {
-        static_assert(N == 16, "16 or 32 columns");
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-              "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-            : "r"(taddr));
-    }
-}
-// Waits for this thread's TMEM loads; the destination registers are marked as written by the
-// wait so that no use is scheduled before it.
-template <int N>
-__device__ __forceinline__ void twait(uint32_t (&a)[N]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
-                   "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])
-                 :
-                 : "memory");
-    if constexpr (N == 32)
-        asm volatile(""
-                     : "+r"(a[16]), "+r"(a[17]), "+r"(a[18]), "+r"(a[19]), "+r"(a[20]), "+r"(a[21]), "+r"(a[22]),
-                       "+r"(a[23]), "+r"(a[24]), "+r"(a[25]), "+r"(a[26]), "+r"(a[27]), "+r"(a[28]), "+r"(a[29]),
-                       "+r"(a[30]), "+r"(a[31])::"memory");
-}
-__device__ __forceinline__ void cpa16(uint32_t dst, const void *src, uint32_t n) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void bar_expect_tx(uint32_t b, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void tma_2d(uint32_t dst, const CUtensorMap *m, int32_t x, int32_t y, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_3d(uint32_t dst, const CUtensorMap *m, int32_t x, int32_t y, int32_t z, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
-        "l"((uint64_t)m), "r"(x), "r"(y), "r"(z), "r"(bar)
-        : "memory");
-}
 
 // Kernel arguments: the attention problem and the tensor maps of its k and v columns.
 struct TcArgs {
@@ -837,22 +714,6 @@ __global__ void __launch_bounds__(kThreadsTc, kMinBlocks) attn_tc_kernel(const _
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
     }
-}
-
-typedef CUresult (*EncodeTiledTc)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledTc encode_tc() {
-    static std::once_flag once;
-    static EncodeTiledTc fn = nullptr;
-    std::call_once(once, [] {
-        void *f = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledTc)f;
-    });
-    return fn;
 }
 
 // Tensor map over the 64 H fp16 columns of k (or v) starting at `base`: 2-D {64 H, B T} with

@@ -152,6 +152,9 @@ cudaError_t launch_attention(const AttnParams &p, cudaStream_t s);
 // The tensor-memory (tcgen05) form for dh = 64 with fp16-carried q|k|v, 16-byte aligned rows and
 // windows of side <= 128; cudaErrorNotSupported when the problem is outside that.
 cudaError_t launch_attention_tc(const AttnParams &p, cudaStream_t s);
+// The form whose scores stay in tensor memory (groups of at most 2048 keys, per-row s_d; any q|k|v
+// carrier, dh 32 or 64); cudaErrorNotSupported when the problem is outside that.
+cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s);
 
 // ---------------------------------------------------------------- deformable sampling
 struct DeformParams {

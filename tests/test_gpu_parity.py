@@ -280,6 +280,44 @@ def test_attention_extreme_scores(ilw, orc):
     assert_same(host(got), orc.attention(qkv, B, T, H, dh, 0, smx, 1 << 30, 33), "attn extreme")
 
 
+@pytest.mark.parametrize("B,T,H,dh,win,form", [
+    (1, 1, 1, 64, 0, "f16"), (1, 16, 1, 64, 0, "f16"), (1, 33, 2, 32, 0, "f16"),  # one unit of 16 keys, a partial one
+    (2, 257, 1, 64, 0, "f16"), (1, 448, 1, 64, 0, "f16"),  # past one MMA's 256 keys, a CTA's 448
+    (1, 449, 1, 64, 0, "i8"), (1, 897, 1, 64, 0, "f16"), (1, 1793, 1, 64, 0, "f16"),  # clusters of 2, 4 and 8 CTAs
+    (1, 3585, 1, 64, 0, "f16"),                            # past a cluster of 8: the streaming kernel
+    (90, 40, 2, 32, 0, "i8"), (41, 130, 2, 64, 0, "f16"),  # several jobs per CTA, units changing
+    (12, 600, 2, 64, 0, "f16"), (5, 900, 3, 32, 0, "i8"),  # the same in clusters
+    (2, 900, 2, 64, 2, "i8"), (1, 5329, 1, 64, 1, "f16"), (1, 441, 2, 64, 21, "f16"), (2, 1764, 1, 32, 2, "f16")])
+def test_attention_resident_shapes(ilw, orc, B, T, H, dh, win, form):
+    """The kernel whose scores stay in tensor memory, at the edges of its tiles and of its split over
+    a cluster; images beyond the first few repeat them, and every repeat is compared."""
+    d, n = H * dh, min(B, 3)
+    qkv = synth.uniform_int(16, f"qkvr{T}{H}{dh}", (n * T, 3 * d), -90, 90, np.int8)
+    full = np.concatenate([qkv.reshape(n, -1)] * (B // n + 1))[:B].reshape(B * T, 3 * d)
+    smx = {"I0": 4000, "k_inter": 16, "k_out": 8, "s_d": -1, "m_p": 4, "M_hw": 31}
+    got = host(ilw.shiftmax_attn(dev(full if form == "i8" else full.astype(np.float16)), B, T, H, dh, win, smx, 3 << 29, 36))
+    want = orc.attention(qkv, n, T, H, dh, win, smx, 3 << 29, 36).reshape(n, -1)
+    for b in range(B):
+        assert_same(got.reshape(B, -1)[b], want[b % n], f"resident T={T} win={win} image {b}")
+
+
+@pytest.mark.parametrize("I0,k_inter,k_out,m_p", [(1, 16, 8, 4), (3, 10, 4, 0), (700, 0, 8, 4), (16384, 16, 8, 4),
+                                                  (32767, 15, 7, 4), (32767, 16, 8, 16), (9000, 16, 1, 31)])
+def test_attention_resident_parameters(ilw, orc, I0, k_inter, k_out, m_p):
+    """Its Shiftmax parameters over their range: sums of four and of two values in 32 bits, every form
+    of the output (one and two outputs per word, the 64-bit product), and shifts of the output
+    requantisation on both sides of 33; int8 outputs with rows that no vector store fits."""
+    B, T, H = 1, 210, 1
+    qkv = synth.uniform_int(17, f"qkvp{I0}{k_inter}", (B * T, 192), -60, 60, np.int8)
+    smx = {"I0": I0, "k_inter": k_inter, "k_out": k_out, "s_d": -1, "m_p": m_p, "M_hw": 31}
+    out = torch.zeros((B * T, 70), dtype=torch.int8, device="cuda")
+    for s_o in (30, 36):
+        ilw.shiftmax_attn(dev(qkv.astype(np.float16)), B, T, H, 64, 0, smx, 3 << 28, s_o, out=out[:, 3:67])
+        want = orc.attention(qkv, B, T, H, 64, 0, smx, 3 << 28, s_o)
+        assert_same(host(out[:, 3:67]), want, f"resident I0={I0} k={k_inter} s_o={s_o}")
+        assert not bool(out[:, :3].any()) and not bool(out[:, 67:].any())
+
+
 # ------------------------------------------------------------------------------ split conv
 def test_split_conv(ilw, orc):
     M, N, Ks = 333, 256, (384, 384, 384, 384)

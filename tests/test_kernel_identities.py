@@ -31,6 +31,33 @@ def test_invariant_divisor_reciprocal(I0):
     assert np.array_equal(q, n // np.uint64(I0))
 
 
+@pytest.mark.parametrize("I0,k", [(1, 16), (2, 3), (3, 16), (7, 0), (255, 16), (4097, 16), (6000, 16), (11586, 9),
+                                  (16384, 16), (32767, 16)])
+def test_shiftexp_in_fp32(I0, k):
+    """Attention's ShiftExp on fp32 integers: with M = 1.5 2^23, M + 3a/2 rounded up and -M - a/16
+    rounded down add up to n = a + ceil(a/2) - ceil(a/16) (both stay below 2^24, where the last place
+    is 1); 2^23 + n rcp rounded down, rcp the float next above 1 / I0, holds q = floor(n / I0); and
+    2^23 + I0 - r/2 rounded down holds Ib, so (Ib << 16) >> q is ShiftExp 2^(16 - k)."""
+    a = np.arange(0, (1 << 21) + 1, dtype=np.int64)
+    M = 3 << 22
+    up, dn = M + (3 * a + 1) // 2, M + (a + 15) // 16
+    assert up.max() < 1 << 24 and dn.max() < 1 << 24
+    n = np.minimum(up - dn, k * I0)
+    assert np.array_equal(up - dn, a + ((a + 1) >> 1) - ((a + 15) >> 4))
+    rcp = np.float32(1.0) / np.float32(I0)
+    if float(rcp) * I0 < 1.0:
+        rcp = np.nextafter(rcp, np.float32(2.0))
+    m, e = np.frexp(np.float64(rcp))
+    mant, sh = int(m * (1 << 24)), 24 - int(e)  # rcp = mant 2^-sh, exactly
+    assert mant * 2.0 ** -sh == float(rcp) and mant * I0 >= 1 << sh
+    q = (n * mant) >> sh  # floor of the exact product, as the fused multiply-add rounds it
+    assert np.array_equal(q, n // I0) and q.max() <= 16
+    Ib = I0 + ((-(n - q * I0)) >> 1)
+    assert Ib.min() >= 0 and Ib.max() <= I0
+    literal = (I0 - (n % I0 + 1) // 2) << (k - n // I0)
+    assert np.array_equal((Ib << 16) >> q, literal << (16 - k))
+
+
 def test_sigmoid_uses_one_shiftexp():
     """SD-ShiftGELU: with I_shift = ReLU(I_p), I_delta = I_p - I_shift, exactly one of I_delta
     and -I_shift is 0 (both when I_p = 0), so {I_delta, -I_shift} = {0, -|I_p|}."""
