@@ -440,6 +440,10 @@ int ilwdetr_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, int32_t
  * ilwdetr_device_status. */
 int ilwdetr_gather_rows(const void *src, int64_t src_ld, int64_t src_rows, const int32_t *idx, int64_t n,
                         int64_t row_bytes, void *dst, int64_t dst_ld, ilw_stream_t stream);
+/* The same for `batches` sources of src_rows rows one after the other (one per image): dst row b n + i =
+ * row idx[b n + i] of source b, i < n; idx int32 [batches, n]. */
+int ilwdetr_gather_rows_batched(const void *src, int64_t src_ld, int64_t src_rows, const int32_t *idx, int64_t n,
+                                int64_t batches, int64_t row_bytes, void *dst, int64_t dst_ld, ilw_stream_t stream);
 
 #ifdef __cplusplus
 }

@@ -16,7 +16,7 @@ __all__ = [
     "BlockWeights", "block_forward", "block_workspace_bytes", "device_status",
     "patch_embed", "patch_embed_workspace_bytes", "Backbone", "Graphed",
     "requant", "resample_nearest", "DecoderWeights", "decoder_workspace_bytes", "decoder_layer_forward",
-    "Projector", "Detector", "int_sigmoid", "relu_i8", "topk", "gather_rows", "DetectionHead", "TwoStage",
+    "Projector", "Detector", "int_sigmoid", "relu_i8", "topk", "gather_rows", "gather_rows_batched", "DetectionHead", "TwoStage",
     "QueryPos", "BoxRefine", "ivit_shiftgelu",
 ]
 
@@ -153,6 +153,7 @@ SIGNATURES = {
     "ilwdetr_ivit_shiftgelu": ([_VP, _I64, _I64, _I32, _VP, _I64, C.POINTER(GeluT), _VP], C.c_int),
     "ilwdetr_topk": ([_VP, _I64, _I32, _I32, _I32, _VP, _VP, _VP], C.c_int),
     "ilwdetr_gather_rows": ([_VP, _I64, _I64, _VP, _I64, _I64, _VP, _I64, _VP], C.c_int),
+    "ilwdetr_gather_rows_batched": ([_VP, _I64, _I64, _VP, _I64, _I64, _I64, _VP, _I64, _VP], C.c_int),
     "ilwdetr_decoder_workspace_bytes": ([_I32, _I32, _I64, _I32, _I32, _I32, _I32, _I32], C.c_size_t),
     "ilwdetr_decoder_layer_forward": ([C.POINTER(DecoderParamsT), _VP, _VP, _VP, C.POINTER(_I32), _I32, _VP,
                                        _I32, _I32, _VP, _VP, C.c_size_t, _VP], C.c_int),
@@ -755,6 +756,21 @@ def gather_rows(X, idx, out=None):
     return out
 
 
+def gather_rows_batched(X, idx, out=None):
+    """ilwdetr_gather_rows_batched: X [batches * rows, C] holds one source of equal size per row of idx
+    (int32 [batches, n]); row b n + i of the result is row idx[b, i] of source b."""
+    import torch
+
+    B, n = idx.shape
+    rb = X.shape[1] * X.element_size()
+    if out is None:
+        out = torch.empty((B * n, X.shape[1]), dtype=X.dtype, device=X.device)
+    _check(lib().ilwdetr_gather_rows_batched(_ptr(X), X.stride(0) * X.element_size(), X.shape[0] // B, _ptr(idx), n, B, rb,
+                                             _ptr(out), out.stride(0) * out.element_size(), _stream()),
+           "gather_rows_batched")
+    return out
+
+
 class DetectionHead:
     """The detection head on the decoder output (``synth.head_params``): class scores by the integer
     sigmoid of a linear layer's raw logits; box logits from a 3-layer integer MLP (ReLU on the int8
@@ -841,18 +857,14 @@ class TwoStage:
     def forward(self, memory, B, S, K):
         """memory int8 [B*S, d] -> (values [B, K], token indices [B, K], ref16 int16 [B*K, 4],
         boxes int32 [B*K, 4])."""
-        import torch
-
         tp, t = self.tp, self.t
         d = memory.shape[1]
         Cn = tp["w_enc"].shape[0]
         enc = gemm_requant(memory, t["w_enc_p"], Cn, t["b_enc"], None, None, 32)
         best, _ = topk(enc, 1)
         vals, idx = topk(best.view(B, S), K)
-        # the selected tokens' memory rows and anchors, image by image (views of the batch)
-        sel = torch.empty((B * K, d), dtype=torch.int8, device=memory.device)
-        for b in range(B):
-            gather_rows(memory[b * S:(b + 1) * S], idx[b], out=sel[b * K:(b + 1) * K])
+        # the selected tokens' memory rows (each image its own) and anchors
+        sel = gather_rows_batched(memory, idx)
         anc = gather_rows(t["anchor16"], idx.view(-1))
         h1 = gemm_requant(sel, t["w_p1_p"], d, t["b_p1"], t["m_p1"], t["s_p1"], 8)
         relu_i8(h1, out=h1)

@@ -698,17 +698,28 @@ int ilwdetr_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, int32_t
     return cuda_status(ilw::launch_topk(S, lds, rows, N, K, vals, idx, (cudaStream_t)stream), "topk");
 }
 
+static int gather_impl(const void *src, int64_t src_ld, int64_t src_rows, const int32_t *idx, int64_t n, int64_t batches,
+                       int64_t row_bytes, void *dst, int64_t dst_ld, ilw_stream_t stream, const char *what) {
+    if (n < 0 || batches < 0 || row_bytes < 0 || src_rows < 0 || row_bytes % 4 || src_ld % 4 || dst_ld % 4 ||
+        src_ld < row_bytes || dst_ld < row_bytes)
+        return fail(ILW_ERR_INVALID_ARG, "%s: bad sizes (row bytes and strides multiples of 4)", what);
+    if (n == 0 || batches == 0 || row_bytes == 0) return ILW_OK;
+    if (!src || !idx || !dst || !aligned(src, 4) || !aligned(dst, 4) || !aligned(idx, 4))
+        return fail(ILW_ERR_INVALID_ARG, "%s: NULL or misaligned", what);
+    if (g_check_only) return ILW_OK;
+    return cuda_status(ilw::launch_gather_rows(src, src_ld, src_rows, idx, n, batches, row_bytes, dst, dst_ld,
+                                               (cudaStream_t)stream),
+                       what);
+}
+
 int ilwdetr_gather_rows(const void *src, int64_t src_ld, int64_t src_rows, const int32_t *idx, int64_t n,
                         int64_t row_bytes, void *dst, int64_t dst_ld, ilw_stream_t stream) {
-    if (n < 0 || row_bytes < 0 || src_rows < 0 || row_bytes % 4 || src_ld % 4 || dst_ld % 4 || src_ld < row_bytes ||
-        dst_ld < row_bytes)
-        return fail(ILW_ERR_INVALID_ARG, "gather_rows: bad sizes (row bytes and strides multiples of 4)");
-    if (n == 0 || row_bytes == 0) return ILW_OK;
-    if (!src || !idx || !dst || !aligned(src, 4) || !aligned(dst, 4) || !aligned(idx, 4))
-        return fail(ILW_ERR_INVALID_ARG, "gather_rows: NULL or misaligned");
-    if (g_check_only) return ILW_OK;
-    return cuda_status(ilw::launch_gather_rows(src, src_ld, src_rows, idx, n, row_bytes, dst, dst_ld, (cudaStream_t)stream),
-                       "gather_rows");
+    return gather_impl(src, src_ld, src_rows, idx, n, 1, row_bytes, dst, dst_ld, stream, "gather_rows");
+}
+
+int ilwdetr_gather_rows_batched(const void *src, int64_t src_ld, int64_t src_rows, const int32_t *idx, int64_t n,
+                                int64_t batches, int64_t row_bytes, void *dst, int64_t dst_ld, ilw_stream_t stream) {
+    return gather_impl(src, src_ld, src_rows, idx, n, batches, row_bytes, dst, dst_ld, stream, "gather_rows_batched");
 }
 
 int ilwdetr_ivit_shiftgelu(const int32_t *X, int64_t ldx, int64_t rows, int32_t L, int32_t *Y, int64_t ldy,

@@ -18,7 +18,7 @@
 //               carried in fp16, the fp16 128 x 64 tile in the MMA's 128-byte swizzled layout) and
 //               the fp16 weight tile (BN x 64, 128-byte swizzle); with resident weights the CTA's
 //               BN rows of W are loaded once, before its first tile; TMEM allocation
-//   warp 1      MMA issuer (one thread): 4 x (128 x BN x 16) MMAs per 64-wide K stage
+//   warp 1      MMA issuer: 4 x (128 x BN x 16) MMAs per 64-wide K stage
 //   warps 2-5   operand converters (int8 A only): int8 activation rows (smem) -> fp16 rows in the
 //               same 128-byte swizzled K-major layout TMA produces for the weights
 //   warps 6-13  epilogue: TMEM -> registers -> integer epilogue -> HBM, one row per thread and
@@ -162,6 +162,12 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
     return d;
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred P;\n elect.sync _|P, 0xffffffff;\n selp.b32 %0, 1, 0, P;\n}\n" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
@@ -634,51 +640,61 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        // The whole warp runs the loop and one elected lane issues: the operands then stay in uniform
+        // registers.  One thread on its own (`if (lane == 0)`) moves every operand of every MMA over and
+        // needs 113 clocks per MMA, above the 64 (N = 128) and 96 (N = 192) the MMA itself takes; this
+        // form needs 60 and 86.
+        {
+            const bool issue = elect_lane();
+            auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
+                return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, p.status, code, p.wait_cycles));
+            };
             const uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
             // operand descriptors from two precomputed bases: a 16-byte step of the address is 1 in
             // the descriptor's low word (shared-memory offsets stay below 256 KB, so nothing carries)
             const uint64_t a_desc0 = sw128_desc(smem_u32(smem)), w_desc0 = sw128_desc(smem_u32(wres));
-            int it = 0, tl = 0, s = 0;
+            int tl = 0, s = 0;
             uint32_t ph = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < p.tiles && ok; t += gridDim.x, ++tl) {
-                const int b = tl % p.nbuf;
-                const uint32_t use = (uint32_t)(tl / p.nbuf);
-                if (!mbar_wait(acc_empty(b), (use & 1) ^ 1, abort, p.status, kStatusTimeoutMma, p.wait_cycles)) break;
+                const int b = p.nbuf == 2 ? tl & 1 : 0;
+                const uint32_t use = (uint32_t)(p.nbuf == 2 ? tl >> 1 : tl);
+                if (!wait(acc_empty(b), (use & 1) ^ 1, kStatusTimeoutMma)) break;
                 tc_fence_after();
                 for (int sg = 0; sg < p.nseg && ok; ++sg) {
-                    const Seg &S = p.seg[sg];
-                    const int nk = (S.klen + BK - 1) / BK;
+                    const int nk = (p.seg[sg].klen + BK - 1) / BK;
                     const uint32_t dt = tmem + (uint32_t)(b * acc_cols + sg * BN);
-                    for (int kk = 0; kk < nk; ++kk, ++it) {
-                        if (!mbar_wait(AF16 ? full(s) : a_ready(s), ph, abort, p.status,
-                                       AF16 ? kStatusTimeoutTma : kStatusTimeoutOperand, p.wait_cycles) ||
-                            (WRES && tl == 0 && !mbar_wait(wfull(kk), 0, abort, p.status, kStatusTimeoutTma, p.wait_cycles))) {
-                            ok = false;
-                            break;
-                        }
+#pragma unroll 1
+                    for (int kk = 0; kk < nk; ++kk) {
+                        ok = wait(AF16 ? full(s) : a_ready(s), ph, AF16 ? kStatusTimeoutTma : kStatusTimeoutOperand);
+                        if (WRES && ok && tl == 0) ok = wait(wfull(kk), 0, kStatusTimeoutTma);
+                        if (!ok) break;
                         tc_fence_after();
                         const uint64_t da = a_desc0 + (uint64_t)((s * kStage) >> 4);
                         const uint64_t dw = WRES ? w_desc0 + (uint64_t)((kk * SM::kWtile) >> 4) : da + (uint64_t)(SM::kA16 >> 4);
+                        if (issue) {
 #pragma unroll
-                        for (int k16 = 0; k16 < BK / 16; ++k16)
-                            tc_mma(dt, da + 2 * k16, dw + 2 * k16, idesc, (kk > 0 || k16 > 0) ? 1u : 0u);
-                        tc_commit(empty(s));
+                            for (int k16 = 0; k16 < BK / 16; ++k16)
+                                tc_mma(dt, da + 2 * k16, dw + 2 * k16, idesc, (kk > 0 || k16 > 0) ? 1u : 0u);
+                            tc_commit(empty(s));
+                        }
+                        __syncwarp();
                         if (++s == STAGES) {
                             s = 0;
                             ph ^= 1u;
                         }
                     }
                 }
-                tc_commit(acc_full(b));  // arrives once every MMA of this tile has completed
+                if (issue) tc_commit(acc_full(b));  // arrives once every MMA of this tile has completed
+                __syncwarp();
             }
             // every MMA issued has completed before the CTA can reach the TMEM release (also after an
             // abort, when the epilogue no longer waits for the accumulators)
-            tc_commit(drain);
+            if (issue) tc_commit(drain);
             const long long t0 = clock64();
             while (!mbar_try(drain, 0) && clock64() - t0 < p.wait_cycles) {
             }
+            __syncwarp();
         }
     } else if (warp < EPI0) {
         // ---------------------------------------------------------------- operand converters

@@ -47,19 +47,117 @@ __global__ void __launch_bounds__(256) relu_i8_kernel(const int8_t *__restrict__
         Y[i] = X[i] < 0 ? (int8_t)0 : X[i];
 }
 
-// Per-row top-K by a bitonic sort of (value, index) keys in shared memory: key = (value biased to
-// unsigned) << 32 | (2^32 - 1 - index), so one descending order puts larger values first and, for
-// equal values, smaller indices first.  Padding keys are 0, below every real key.
-__global__ void topk_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t N, int32_t npad, int32_t K,
-                            int32_t *__restrict__ vals, int32_t *__restrict__ idx) {
-    extern __shared__ unsigned long long keys[];
+// Per-row top-K, one CTA per row, ties to the lower index.  Bound by latency (a row's 33 KB at 8400
+// values are nothing): sorting the whole padded row took 105 steps over 16384 keys, 211 us; selecting
+// first leaves K keys to order.  Thread t holds values t VPT .. (VPT of them) in registers.
+//   1. the K-th largest value, found bit by bit below the row's maximum: every step counts the values at
+//      or above a candidate over the CTA;
+//   2. a scan over the threads gives every value above it its place among the selected, and the values
+//      equal to it, in index order, the places left;
+//   3. the selected keys (value, lower index first) are ordered by counting the larger ones for
+//      K <= kRankMax, else by a bitonic sort of the K keys.
+// Keys: (value biased to unsigned) << 32 | (2^32 - 1 - index), so one descending order puts larger
+// values first and, for equal values, smaller indices first.  Padding keys are 0, below every real key.
+constexpr int kTopkThreads = 1024;
+constexpr int kRankMax = 512;
+template <int VPT>
+__global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t N,
+                                                            int32_t kpad, int32_t K, int32_t *__restrict__ vals,
+                                                            int32_t *__restrict__ idx) {
+    extern __shared__ unsigned long long keys[];  // kpad
+    __shared__ uint32_t part[2][32];
     const int32_t *s = S + (int64_t)blockIdx.x * lds;
-    for (int i = threadIdx.x; i < npad; i += blockDim.x)
-        keys[i] = i < N ? ((unsigned long long)((uint32_t)s[i] ^ 0x80000000u) << 32) | (0xFFFFFFFFu - (uint32_t)i) : 0ull;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, i0 = tid * VPT;
+    // biased values; past the row 0, which step 2 never selects (it is told apart by its index)
+    uint32_t v[VPT];
+#pragma unroll
+    for (int j = 0; j < VPT; ++j) v[j] = i0 + j < N ? (uint32_t)s[i0 + j] ^ 0x80000000u : 0u;
+    // the CTA's sum of one value per thread (alternating buffers: one barrier per call)
+    int buf = 0;
+    auto cta_sum = [&](uint32_t x) -> uint32_t {
+        x = __reduce_add_sync(0xffffffffu, x);
+        if (lane == 0) part[buf][warp] = x;
+        __syncthreads();
+        x = __reduce_add_sync(0xffffffffu, part[buf][lane]);
+        buf ^= 1;
+        return x;
+    };
+    // bits above the highest in which the row's values differ are the maximum's
+    uint32_t hi = 0, lo = 0xffffffffu;
+#pragma unroll
+    for (int j = 0; j < VPT; ++j)
+        if (i0 + j < N) {
+            hi = max(hi, v[j]);
+            lo = min(lo, v[j]);
+        }
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    if (lane == 0) {
+        part[0][warp] = hi;
+        part[1][warp] = lo;
+    }
     __syncthreads();
-    for (int k = 2; k <= npad; k <<= 1)
+    hi = __reduce_max_sync(0xffffffffu, part[0][lane]);
+    lo = __reduce_min_sync(0xffffffffu, part[1][lane]);
+    __syncthreads();
+    // thr: the largest value with at least K values at or above it (that many are at or above `lo`)
+    const int top = 32 - __clz(hi ^ lo);
+    uint32_t thr = top == 32 ? 0u : hi >> top << top;
+    for (int bit = top - 1; bit >= 0; --bit) {
+        const uint32_t cand = thr | (1u << bit);
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < VPT; ++j) c += (i0 + j < N && v[j] >= cand) ? 1u : 0u;
+        if (cta_sum(c) >= (uint32_t)K) thr = cand;
+    }
+    // places: (values above thr) << 16 | (values equal to it), summed over the threads before this one
+    uint32_t c = 0;
+#pragma unroll
+    for (int j = 0; j < VPT; ++j)
+        if (i0 + j < N) c += v[j] > thr ? 1u << 16 : (v[j] == thr ? 1u : 0u);
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    __syncthreads();
+    if (lane == 31) part[0][warp] = incl;
+    for (int i = K + tid; i < kpad; i += kTopkThreads) keys[i] = 0ull;
+    __syncthreads();
+    const uint32_t w = part[0][lane];
+    const uint32_t total = __reduce_add_sync(0xffffffffu, w);
+    uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + incl - c;
+    const uint32_t above = total >> 16;
+    uint32_t pg = before >> 16, pe = above + (before & 0xffffu);
+#pragma unroll
+    for (int j = 0; j < VPT; ++j) {
+        if (i0 + j >= N || v[j] < thr) continue;
+        const uint32_t pos = v[j] > thr ? pg++ : pe++;
+        if (pos < (uint32_t)K) keys[pos] = ((unsigned long long)v[j] << 32) | (0xFFFFFFFFu - (uint32_t)(i0 + j));
+    }
+    __syncthreads();
+    auto put = [&](int at, unsigned long long key) {
+        vals[(int64_t)blockIdx.x * K + at] = (int32_t)((uint32_t)(key >> 32) ^ 0x80000000u);
+        idx[(int64_t)blockIdx.x * K + at] = (int32_t)(0xFFFFFFFFu - (uint32_t)key);
+    };
+    if (K <= kRankMax) {
+        // 2 threads (adjacent lanes) per key, each over half of the keys: its place is the number of larger ones
+        const int e = tid >> 1, h = tid & 1;
+        if (e - (lane >> 1) < K) {  // the warp has a key
+            const unsigned long long key = e < K ? keys[e] : ~0ull;
+            const int half = (K + 1) >> 1, b = h * half, n = h ? K - half : half;
+            int rank = 0;
+#pragma unroll 8
+            for (int i = 0; i < n; ++i) rank += keys[b + i] > key ? 1 : 0;
+            rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+            if (e < K && h == 0) put(rank, key);
+        }
+        return;
+    }
+    for (int k = 2; k <= kpad; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < npad; i += blockDim.x) {
+            for (int i = tid; i < kpad; i += kTopkThreads) {
                 const int ixj = i ^ j;
                 if (ixj > i) {
                     const unsigned long long a = keys[i], b = keys[ixj];
@@ -71,11 +169,7 @@ __global__ void topk_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t 
             }
             __syncthreads();
         }
-    for (int i = threadIdx.x; i < K; i += blockDim.x) {
-        const unsigned long long key = keys[i];
-        vals[(int64_t)blockIdx.x * K + i] = (int32_t)((uint32_t)(key >> 32) ^ 0x80000000u);
-        idx[(int64_t)blockIdx.x * K + i] = (int32_t)(0xFFFFFFFFu - (uint32_t)key);
-    }
+    for (int i = tid; i < K; i += kTopkThreads) put(i, keys[i]);
 }
 
 // K = 1: one warp per row keeps the largest value with the smallest index among its columns, and
@@ -109,13 +203,13 @@ __global__ void __launch_bounds__(256) top1_kernel(const int32_t *__restrict__ S
     }
 }
 
-// Row gather in 4-byte words: dst row i = src row idx[i].  An index outside [0, src_rows) gives a
-// zero row and latches kStatusBadIndex in the device status word.
+// Row gather in 4-byte words: dst row i = row idx[i] of source i / n (src_rows rows each).  An index
+// outside [0, src_rows) gives a zero row and latches kStatusBadIndex in the device status word.
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint32_t *__restrict__ src, int64_t src_ldw,
                                                           int64_t src_rows, const int32_t *__restrict__ idx, int64_t n,
-                                                          int64_t roww, uint32_t *__restrict__ dst, int64_t dst_ldw,
-                                                          int *status) {
-    const int64_t total = n * roww;
+                                                          int64_t batches, int64_t roww, uint32_t *__restrict__ dst,
+                                                          int64_t dst_ldw, int *status) {
+    const int64_t total = n * batches * roww;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = t / roww, w = t - i * roww;
         const int64_t r = idx[i];
@@ -124,7 +218,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint32_t *__rest
             if (w == 0 && status) atomicExch(status, kStatusBadIndex);
             continue;
         }
-        dst[i * dst_ldw + w] = src[r * src_ldw + w];
+        dst[i * dst_ldw + w] = src[((i / n) * src_rows + r) * src_ldw + w];
     }
 }
 
@@ -193,25 +287,27 @@ cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, 
         top1_kernel<<<grid_for(((int64_t)rows + 7) / 8, 1), 256, 0, s>>>(S, lds, rows, N, vals, idx);
         return cudaGetLastError();
     }
-    int npad = 2;
-    while (npad < N) npad <<= 1;
-    const size_t smem = (size_t)npad * 8;
-    const int threads = npad / 2 < 1024 ? (npad / 2 < 32 ? 32 : npad / 2) : 1024;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int kpad = 2;
+    while (kpad < K) kpad <<= 1;
+    const size_t smem = (size_t)kpad * 8;
+    auto go = [&](auto kern, SmemLimit &limit) -> cudaError_t {
+        const cudaError_t e = raise_smem_limit(limit, (const void *)kern, 16384 * 8);
         if (e != cudaSuccess) return e;
-    }
-    topk_kernel<<<(unsigned)rows, threads, smem, s>>>(S, lds, N, npad, K, vals, idx);
-    return cudaGetLastError();
+        kern<<<(unsigned)rows, kTopkThreads, smem, s>>>(S, lds, N, kpad, K, vals, idx);
+        return cudaGetLastError();
+    };
+    static SmemLimit l2, l9, l16;
+    if (N <= 2 * kTopkThreads) return go(topk_kernel<2>, l2);
+    if (N <= 9 * kTopkThreads) return go(topk_kernel<9>, l9);  // the detector's 8400 memory tokens
+    return go(topk_kernel<16>, l16);
 }
 
 cudaError_t launch_gather_rows(const void *src, int64_t src_ld_bytes, int64_t src_rows, const int32_t *idx, int64_t n,
-                               int64_t row_bytes, void *dst, int64_t dst_ld_bytes, cudaStream_t s) {
-    if (n == 0 || row_bytes == 0) return cudaSuccess;
-    gather_rows_kernel<<<grid_for(n * (row_bytes / 4), 256), 256, 0, s>>>((const uint32_t *)src, src_ld_bytes / 4,
-                                                                           src_rows, idx, n, row_bytes / 4,
-                                                                           (uint32_t *)dst, dst_ld_bytes / 4,
-                                                                           status_word_ptr());
+                               int64_t batches, int64_t row_bytes, void *dst, int64_t dst_ld_bytes, cudaStream_t s) {
+    if (n == 0 || batches == 0 || row_bytes == 0) return cudaSuccess;
+    gather_rows_kernel<<<grid_for(n * batches * (row_bytes / 4), 256), 256, 0, s>>>(
+        (const uint32_t *)src, src_ld_bytes / 4, src_rows, idx, n, batches, row_bytes / 4, (uint32_t *)dst,
+        dst_ld_bytes / 4, status_word_ptr());
     return cudaGetLastError();
 }
 

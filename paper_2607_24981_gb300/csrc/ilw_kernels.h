@@ -186,7 +186,7 @@ cudaError_t launch_ivit_shiftgelu(const int32_t *X, int64_t ldx, int64_t rows, i
 cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, int32_t K, int32_t *vals,
                         int32_t *idx, cudaStream_t s);
 cudaError_t launch_gather_rows(const void *src, int64_t src_ld_bytes, int64_t src_rows, const int32_t *idx, int64_t n,
-                               int64_t row_bytes, void *dst, int64_t dst_ld_bytes, cudaStream_t s);
+                               int64_t batches, int64_t row_bytes, void *dst, int64_t dst_ld_bytes, cudaStream_t s);
 
 // ---------------------------------------------------------------- detector: requantisation, resampling
 struct RequantParams {

@@ -70,6 +70,26 @@ def test_topk(ilw, orc, rows, N, K, lo, hi):
     same(host(v), wv, f"topk values {rows}x{N} K={K}")
 
 
+@pytest.mark.parametrize("rows,N,K,lo,hi", [(2, 9216, 512, -(1 << 20), 1 << 20), (1, 9217, 513, -50, 50),
+                                            (3, 2048, 300, -1, 1), (2, 2049, 1000, -(1 << 31), (1 << 31) - 1),
+                                            (1, 16384, 2, 0, 0), (4, 33, 32, -9, 9), (300, 8400, 300, -3000, 3000)])
+def test_topk_selection(ilw, orc, rows, N, K, lo, hi):
+    """The selection's edges: values per thread (2, 9, 16), K at the end of the counting order (512)
+    and past it, ties that span threads and rows of one value."""
+    S = synth.uniform_int(76, f"topks{rows}.{N}", (rows, N), lo, hi)
+    v, i = ilw.topk(dev(S), K)
+    wv, wi = orc.topk(S, K)
+    same(host(i), wi, f"topk idx {rows}x{N} K={K}")
+    same(host(v), wv, f"topk values {rows}x{N} K={K}")
+
+
+def test_gather_rows_batched(ilw, orc):
+    X = synth.uniform_int(77, "gatherb", (3 * 50, 8), -128, 127, np.int8)
+    idx = synth.uniform_int(78, "gatherb.i", (3, 21), 0, 49)
+    want = np.concatenate([orc.gather_rows(X[b * 50:(b + 1) * 50], idx[b]) for b in range(3)])
+    same(host(ilw.gather_rows_batched(dev(X), dev(idx))), want, "batched gather")
+
+
 def test_gather_rows(ilw, orc):
     X = synth.uniform_int(74, "gather", (1000, 6), -(1 << 30), 1 << 30)
     idx = synth.uniform_int(75, "gather.i", (777,), 0, 999)
