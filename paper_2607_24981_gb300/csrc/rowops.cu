@@ -317,6 +317,28 @@ __device__ __forceinline__ void ln_store4(TOut *y, const int32_t (&o)[4]) {
     }
 }
 
+// The same from u = value + 127 (8-bit outputs, in [0, 254]) or value + 32767 (16-bit, in [0, 65534]):
+// clamping to u is one add-min-relu, and one add and one exclusive or per word undo the bias (u + 1 never
+// carries into the next lane, and flipping the top bit takes 128 or 32768 off).
+template <typename TOut> struct LnBias { static constexpr int one = LnOut<TOut>::bits == 8 ? 127 : 32767; };
+template <typename TOut>
+__device__ __forceinline__ void ln_store4_biased(TOut *y, const int32_t (&u)[4]) {
+    const uint32_t a = __byte_perm(u[0], u[1], sizeof(TOut) == 1 ? 0x0040 : 0x5410);
+    const uint32_t b = __byte_perm(u[2], u[3], sizeof(TOut) == 1 ? 0x0040 : 0x5410);
+    if constexpr (sizeof(TOut) == 1) {
+        *(uint32_t *)y = (__byte_perm(a, b, 0x5410) + 0x01010101u) ^ 0x80808080u;
+    } else if constexpr (LnOut<TOut>::bits == 16) {
+        *(uint2 *)y = make_uint2((a + 0x00010001u) ^ 0x80008000u, (b + 0x00010001u) ^ 0x80008000u);
+    } else {
+        // the fp16 bits of 1024 + u are 0x6400 + u; one half2 subtract of 1151 leaves the value
+        const __half2 k1151 = __half2half2(__ushort_as_half((unsigned short)0x647f));
+        uint32_t wa = a | 0x64006400u, wb = b | 0x64006400u;
+        __half2 ha = __hsub2(*reinterpret_cast<__half2 *>(&wa), k1151);
+        __half2 hb = __hsub2(*reinterpret_cast<__half2 *>(&wb), k1151);
+        *(uint2 *)y = make_uint2(*reinterpret_cast<uint32_t *>(&ha), *reinterpret_cast<uint32_t *>(&hb));
+    }
+}
+
 // acc += a * b with a 64-bit accumulator in one wide multiply-add
 __device__ __forceinline__ void madw(int64_t &acc, int32_t a, int32_t b) {
     asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
@@ -335,28 +357,100 @@ __device__ __noinline__ void ln_norm4_exact(const int32_t (&x)[4], int64_t mu, i
     }
 }
 
-// I-LayerNorm by row groups (Sec. 3.3; mean, variance, Newton's integer square root,
+// What the host works out once per launch: the range of V whose Newton root needs no steps, 1 / (2 C).
+struct LnConst {
+    uint64_t lo, hi;
+    float inv2c;
+};
+// isqrt(V) for 4 <= V < 2^48, and rem = V - s^2 in [0, 2 s].  The float root is below 2^-21 relative and 1
+// absolute off, 9 at most, so V - s^2 fits 32 bits (and is formed there); one step from it leaves s within 1,
+// which the remainder tells.
+__device__ __forceinline__ uint32_t isqrt_u48(uint64_t V, uint32_t &rem_out) {
+    const float vf = u64_to_float(V), rs = rsqrtf(vf);
+    uint32_t s = __float2uint_rz(vf * rs);
+    int32_t rem = (int32_t)((uint32_t)V - s * s);
+    s += __float2int_rd(__int2float_rn(rem) * (0.5f * rs));
+    rem = (int32_t)((uint32_t)V - s * s);
+    if (rem < 0) {
+        --s;
+        rem += 2 * (int32_t)s + 1;
+    } else if (rem > 2 * (int32_t)s) {
+        rem -= 2 * (int32_t)s + 1;
+        ++s;
+    }
+    rem_out = (uint32_t)rem;
+    return s;
+}
+// floor((2^31 - 1) / s) for 2 <= s < 2^25: the float quotient is below 2^-21 relative and 1 absolute
+// off, so the remainder is below 2^10 + s in magnitude and one step from it leaves 1 at most.
+__device__ __forceinline__ uint32_t div_int31_u24(uint32_t s) {
+    const float rc = __fdividef(1.0f, __uint2float_rn(s));
+    uint32_t q = __float2uint_rz(2147483648.0f * rc);
+    int32_t rem = (int32_t)(kInt31Max - q * s);
+    const int32_t dq = __float2int_rd(__int2float_rn(rem) * rc);
+    q += dq;
+    rem -= dq * (int32_t)s;
+    if (rem < 0) --q;
+    else if (rem >= (int32_t)s) ++q;
+    return q;
+}
+// A row's mean, F and whether y F fits 32 bits, from its sums, in full generality.
+struct LnRow {
+    int64_t mu, F;
+    bool fits;
+};
+__device__ __noinline__ LnRow ln_row_general(int64_t S, int64_t Q, int32_t C, int32_t iters) {
+    // mu = floor((2S + C) / (2C)); V = Q - 2 mu S + C mu^2 (= sum (x - mu)^2)
+    const int64_t num = 2 * S + C, den = 2 * (int64_t)C;
+    int64_t mu = num / den;
+    if ((num % den) != 0 && num < 0) mu -= 1;
+    const uint64_t V = (uint64_t)(Q - 2 * mu * S + (int64_t)C * mu * mu);
+    const uint64_t R = V < (1ull << 48) ? newton_isqrt_fast(V, iters) : newton_isqrt_early(V, iters);
+    return {mu, R < (1ull << 32) ? (int64_t)div_int31((uint32_t)R) : 0, iters >= 1 || V < (1ull << 32)};
+}
+
+// I-LayerNorm by rows (Sec. 3.3; mean, variance, Newton's integer square root,
 // F = floor((2^31 - 1) / R), n = (y F) >> 1, out = sat(rq(n + beta; m, s))).  LPR lanes own one row,
-// 32 / LPR rows per warp, 256 / LPR rows per CTA and step (persistent grid).  A lane reads 16-byte
-// chunks sub, sub + LPR, ... of its row (CPL at most; the LPR lanes of a row read adjacent chunks, so
-// a warp's load covers 32 / LPR row segments of LPR * 16 bytes) and keeps them in registers, sums x
-// and x^2 (int64), and the LPR lanes combine them with shuffles; the row's sums go to shared memory.
-// The per-row scalar work (mean, variance, Newton, F) then runs once per row, one row per thread of
-// the first 256 / LPR threads, instead of on every lane of the row: it is most of the instructions
-// when each of the LPR lanes repeats it.  Every lane reads its row's mean and F back and normalises
-// its own chunks with the per-column parameters from shared memory.
+// 32 / LPR rows per warp and step (persistent grid).  A lane reads 16-byte chunks sub, sub + LPR, ... of
+// its row (CPL at most, exactly when FULL; the LPR lanes of a row read adjacent chunks, so a warp's load
+// covers 32 / LPR row segments of LPR * 16 bytes) and keeps them in registers, sums x and x^2, the LPR lanes
+// combine the sums with shuffles, and each works out the row's mean, root and F.  The warps run apart, no
+// barrier after the parameters are staged, and a warp's first rows are loaded before that.
+// Long inputs are bound by instructions beside the loads, short ones by the chain of one row; so the
+// per-row part is kept short: for 16-bit values (a warp's, as almost always) the sums of two products and
+// the mean are 32-bit, and the Newton root is taken without its steps.  The iteration, for V in
+// [lo, hi], has reached {isqrt(V), isqrt(V) + 1} a step before its last, and from there it stays at
+// s = isqrt(V), unless V = s^2 + 2 s, where it alternates between the two.  Those V, V outside the range
+// and wider values take the general form.
+// 2^20 rows of 384 int32 to int8: 302 us, 6.66 TB/s (461 us with the per-row part on one thread per row
+// behind two barriers and stepped); with half the values per lane (more lanes repeating the per-row part)
+// 10 % slower.
 // 32-bit normalisation: after at least one Newton step R >= isqrt(V) >= |y| for every y = x - mu of
 // the row (a floored Newton step from any positive start lands at or above isqrt(V)), so
 // |y F| <= |y| (2^31 - 1) / R < 2^31 and y F fits int32; with one shift s >= 33 for every column and
 // |beta| <= 2^30 the requantisation is the high-word form with a scalar rounding constant; otherwise
 // (or for rows with iters = 0 and V >= 2^32) the 64-bit formulas run.
-template <typename TIn, typename TOut, int LPR, int CPL>
-__global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p) {
-    extern __shared__ __align__(16) int32_t ln_par[];  // beta[C], mult[C], shift[C]
+template <typename TIn, typename TOut, int LPR, int CPL, bool FULL>
+__global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const LnConst lc) {
+    extern __shared__ __align__(16) int32_t ln_par[];  // beta, mult, shift of CP columns
     constexpr int EB = sizeof(TIn), EPC = 16 / EB;      // elements per 16-byte chunk
-    constexpr int RPW = 32 / LPR;
-    const int C = p.C, nch = C / EPC;
-    int32_t *s_beta = ln_par, *s_mult = ln_par + C, *s_shift = ln_par + 2 * C;
+    constexpr int RPW = 32 / LPR, CP = LPR * CPL * EPC;
+    const int C = p.C;
+    int32_t *s_beta = ln_par, *s_mult = ln_par + CP, *s_shift = ln_par + 2 * CP;
+    const int lane = threadIdx.x & 31, sub = lane % LPR, rr = lane / LPR;
+    const int64_t step = (int64_t)gridDim.x * 8 * RPW;
+    int64_t row = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * RPW + rr;
+    // the chunks that the lane has of its row: none past the end (every lane stays for the shuffles)
+    auto chunks = [&]() { return row < p.rows ? C / EPC - sub : 0; };
+    int4 v[CPL];
+    auto load = [&]() {
+        const int nc = chunks();
+        const int4 *xr = (const int4 *)((const uint8_t *)p.X + row * p.ldx * EB) + sub;
+#pragma unroll
+        for (int i = 0; i < CPL; ++i)
+            v[i] = (FULL ? nc > 0 : LPR * i < nc) ? __ldg(xr + LPR * i) : make_int4(0, 0, 0, 0);
+    };
+    load();
     for (int i = threadIdx.x; i < C / 4; i += blockDim.x) {
         ((int4 *)s_beta)[i] = __ldg((const int4 *)p.beta + i);
         ((int4 *)s_mult)[i] = __ldg((const int4 *)p.mult + i);
@@ -370,128 +464,128 @@ __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p) {
     const bool cols_fast = __syncthreads_and(col_fast) != 0 && uniform_shift >= 33;
     const int32_t rnd = cols_fast ? 1 << (uniform_shift - 33) : 0, sh = uniform_shift - 32;
 
-    constexpr int RPC = 8 * RPW;  // rows per CTA and step (256 threads)
-    __shared__ int64_t s_S[RPC], s_Q[RPC], s_mu[RPC], s_F[RPC];
-    __shared__ int32_t s_ok[RPC];
-    const int lane = threadIdx.x & 31, sub = lane % LPR, rr = lane / LPR;
-    const int lrow = (threadIdx.x >> 5) * RPW + rr;  // the lane's row within the CTA's rows
-    for (int64_t r0 = (int64_t)blockIdx.x * RPC; r0 < p.rows; r0 += (int64_t)gridDim.x * RPC) {
-        const int64_t row = r0 + lrow;
-        const bool live = row < p.rows;  // every lane stays for the shuffles and the barriers
-        const uint8_t *xr = (const uint8_t *)p.X + (live ? row : 0) * p.ldx * EB;
-        int4 v[CPL];
+    for (; __any_sync(0xffffffffu, row < p.rows); row += step, load()) {
+        bool small = true;
+        if constexpr (EB == 4) {
+            int32_t mx = 0, mn = 0;
 #pragma unroll
-        for (int i = 0; i < CPL; ++i) {
-            const int j = sub + LPR * i;
-            v[i] = (live && j < nch) ? __ldg((const int4 *)xr + j) : make_int4(0, 0, 0, 0);
+            for (int i = 0; i < CPL; ++i) {
+                mx = __vimax3_s32(mx, v[i].x, v[i].y);
+                mn = __vimin3_s32(mn, v[i].x, v[i].y);
+                mx = __vimax3_s32(mx, v[i].z, v[i].w);
+                mn = __vimin3_s32(mn, v[i].z, v[i].w);
+            }
+            small = __all_sync(0xffffffffu, mx < 32768 && mn >= -32768);
         }
-        // sum x and sum x^2 of the lane's chunks
-        int64_t S = 0, Q = 0;
+        int64_t mu, F;
+        bool fits;
+        if (small) {
+            // |S| <= 2^25, Q <= 2^40: C <= 1024 16-bit values
+            int32_t S = 0;
+            uint64_t Q = 0;
 #pragma unroll
-        for (int i = 0; i < CPL; ++i) {
-            if constexpr (EB == 2) {
-                const uint32_t w[4] = {(uint32_t)v[i].x, (uint32_t)v[i].y, (uint32_t)v[i].z, (uint32_t)v[i].w};
-                int32_t s32 = 0;
+            for (int i = 0; i < CPL; ++i) {
+                const int32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int32_t lo = (int32_t)(w[u] << 16) >> 16, hi = (int32_t)w[u] >> 16;
-                    s32 += lo + hi;
-                    Q += (int64_t)((uint32_t)(lo * lo) + (uint32_t)(hi * hi));  // <= 2^31
-                }
-                S += s32;
-            } else {
-                const int32_t e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    madw(S, e[u], 1);
-                    madw(Q, e[u], e[u]);
+                for (int u = 0; u < 4; u += EB / 2) {
+                    const int32_t lo = EB == 2 ? (w[u] << 16) >> 16 : w[u], hi = EB == 2 ? w[u] >> 16 : w[(u + 1) & 3];
+                    S += lo + hi;
+                    Q += (uint32_t)(lo * lo) + (uint32_t)(hi * hi);  // <= 2^31
                 }
             }
-        }
 #pragma unroll
-        for (int o = LPR / 2; o; o >>= 1) {
-            S += __shfl_xor_sync(0xffffffffu, S, o, LPR);
-            Q += __shfl_xor_sync(0xffffffffu, Q, o, LPR);
-        }
-        if (sub == 0) {
-            s_S[lrow] = S;
-            s_Q[lrow] = Q;
-        }
-        __syncthreads();
-        if (threadIdx.x < RPC) {
-            // one row per thread: mu = floor((2S + C) / (2C)); V = Q - 2 mu S + C mu^2 (= sum (x - mu)^2)
-            const int64_t S1 = s_S[threadIdx.x], Q1 = s_Q[threadIdx.x];
-            const int64_t num = 2 * S1 + C, den = 2 * (int64_t)C;
-            int64_t mu;
-            if (num >= -(1ll << 31) && num < (1ll << 31)) {
-                const int32_t n32 = (int32_t)num, d32 = (int32_t)den;
-                const int32_t qt = n32 / d32;
-                mu = qt - ((n32 % d32 != 0 && n32 < 0) ? 1 : 0);
-            } else {
-                mu = num / den;
-                if ((num % den) != 0 && num < 0) mu -= 1;
+            for (int o = LPR / 2; o; o >>= 1) {
+                S += __shfl_xor_sync(0xffffffffu, S, o, LPR);
+                Q += __shfl_xor_sync(0xffffffffu, Q, o, LPR);
             }
-            const uint64_t V = (uint64_t)(Q1 - 2 * mu * S1 + (int64_t)C * mu * mu);
-            const uint64_t R = V < (1ull << 48) ? newton_isqrt_fast(V, p.iters) : newton_isqrt_early(V, p.iters);
-            s_mu[threadIdx.x] = mu;
-            s_F[threadIdx.x] = R < (1ull << 32) ? (int64_t)div_int31((uint32_t)R) : 0;
-            s_ok[threadIdx.x] = p.iters >= 1 || V < (1ull << 32);
-        }
-        __syncthreads();
-        const int64_t mu = s_mu[lrow], F = s_F[lrow];
-        const bool fast = cols_fast && __all_sync(0xffffffffu, s_ok[lrow] != 0);
-        const int32_t F32 = (int32_t)F, mF = (int32_t)(0u - (uint32_t)mu * (uint32_t)F);
-        TOut *yr = (TOut *)p.Y + (live ? row : 0) * p.ldy;
+            const int32_t num = 2 * S + C;  // mu = floor((2S + C) / (2C)): a float quotient, at most 1 off
+            int32_t m32 = __float2int_rd(__int2float_rn(num) * lc.inv2c);
+            const int32_t r = num - 2 * C * m32;
+            m32 += r < 0 ? -1 : (r >= 2 * C ? 1 : 0);
+            const uint64_t V = Q - (uint64_t)((int64_t)m32 * (2 * S - C * m32));
+            bool direct = V >= lc.lo && V <= lc.hi;
+            if (direct) {
+                uint32_t rem;
+                const uint32_t s = isqrt_u48(V, rem);
+                direct = rem != 2 * s;
+                mu = m32;
+                F = div_int31_u24(s);
+                fits = true;
+            }
+            if (!direct) {
+                const LnRow lr = ln_row_general(S, (int64_t)Q, C, p.iters);
+                mu = lr.mu, F = lr.F, fits = lr.fits;
+            }
+        } else {
+            int64_t S = 0, Q = 0;
+            if constexpr (EB == 4) {
 #pragma unroll
-        for (int i = 0; i < CPL; ++i) {
-            const int j = sub + LPR * i;
-            if (!live || j >= nch) continue;
-            int32_t x[EPC];
-            if constexpr (EB == 2) {
-                const uint32_t w[4] = {(uint32_t)v[i].x, (uint32_t)v[i].y, (uint32_t)v[i].z, (uint32_t)v[i].w};
+                for (int i = 0; i < CPL; ++i) {
+                    const int32_t e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    x[2 * u] = (int32_t)(w[u] << 16) >> 16;
-                    x[2 * u + 1] = (int32_t)w[u] >> 16;
+                    for (int u = 0; u < 4; ++u) {
+                        madw(S, e[u], 1);
+                        madw(Q, e[u], e[u]);
+                    }
                 }
-            } else {
-                x[0] = v[i].x; x[1] = v[i].y; x[2] = v[i].z; x[3] = v[i].w;
             }
-            const int c0 = j * EPC;
-            int32_t o[EPC];
-            if (fast) {
+#pragma unroll
+            for (int o = LPR / 2; o; o >>= 1) {
+                S += __shfl_xor_sync(0xffffffffu, S, o, LPR);
+                Q += __shfl_xor_sync(0xffffffffu, Q, o, LPR);
+            }
+            const LnRow lr = ln_row_general(S, Q, C, p.iters);
+            mu = lr.mu, F = lr.F, fits = lr.fits;
+        }
+        const int nc = chunks();
+        TOut *yr = (TOut *)p.Y + row * p.ldy + sub * EPC;
+        // one chunk's values (4 of them at u4)
+        auto values = [&](int i, int u4, int32_t (&x)[4]) {
+            const int32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                x[u] = EB == 4 ? w[u] : ((u & 1) ? w[(u4 + u) / 2] >> 16 : (w[(u4 + u) / 2] << 16) >> 16);
+        };
+        if (cols_fast && __all_sync(0xffffffffu, fits)) {
+            const int32_t F32 = (int32_t)F, mF = (int32_t)(0u - (uint32_t)mu * (uint32_t)F);
+#pragma unroll
+            for (int i = 0; i < CPL; ++i) {
+                if (!FULL && LPR * i >= C / EPC) break;
+                const int c0 = (sub + LPR * i) * EPC;
 #pragma unroll
                 for (int u4 = 0; u4 < EPC; u4 += 4) {
+                    int32_t x[4], o[4];
+                    values(i, u4, x);
                     const int4 b4 = *(const int4 *)(s_beta + c0 + u4), m4 = *(const int4 *)(s_mult + c0 + u4);
                     const int32_t be[4] = {b4.x, b4.y, b4.z, b4.w}, mm[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         // (x - mu) F = x F + mF in wrapping 32-bit arithmetic (the product fits int32)
-                        const int32_t n = (int32_t)((uint32_t)x[u4 + u] * (uint32_t)F32 + (uint32_t)mF) >> 1;
-                        const int32_t tq = rq_hi(n + be[u], mm[u], rnd, sh);
-                        o[u4 + u] = LnOut<TOut>::bits == 8 ? clamp8(tq) : clamp16(tq);
+                        const int32_t n = (int32_t)((uint32_t)x[u] * (uint32_t)F32 + (uint32_t)mF) >> 1;
+                        o[u] = __viaddmin_s32_relu(rq_hi(n + be[u], mm[u], rnd, sh), LnBias<TOut>::one,
+                                                   2 * LnBias<TOut>::one);
                     }
+                    if (FULL ? nc > 0 : LPR * i < nc) ln_store4_biased<TOut>(yr + LPR * i * EPC + u4, o);
                 }
-            } else {
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < CPL; ++i) {
+                if (LPR * i >= nc) break;
+                const int c0 = (sub + LPR * i) * EPC;
 #pragma unroll
                 for (int u4 = 0; u4 < EPC; u4 += 4) {
-                    int32_t xx[4], be[4], mm[4], ss[4], oo[4];
+                    int32_t x[4], be[4], mm[4], ss[4], o[4];
+                    values(i, u4, x);
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        xx[u] = x[u4 + u];
                         be[u] = s_beta[c0 + u4 + u];
                         mm[u] = s_mult[c0 + u4 + u];
                         ss[u] = s_shift[c0 + u4 + u];
                     }
-                    ln_norm4_exact(xx, mu, F, be, mm, ss, LnOut<TOut>::bits, oo);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) o[u4 + u] = oo[u];
+                    ln_norm4_exact(x, mu, F, be, mm, ss, LnOut<TOut>::bits, o);
+                    ln_store4<TOut>(yr + LPR * i * EPC + u4, o);
                 }
-            }
-#pragma unroll
-            for (int u4 = 0; u4 < EPC; u4 += 4) {
-                const int32_t oo[4] = {o[u4], o[u4 + 1], o[u4 + 2], o[u4 + 3]};
-                ln_store4<TOut>(yr + c0 + u4, oo);
             }
         }
     }
@@ -545,6 +639,33 @@ __global__ void __launch_bounds__(256) layernorm_kernel(const LnParams p) {
     }
 }
 
+// The V for which `iters` Newton steps from 2^16 end at isqrt(V) (or its alternation): from above, the
+// integer iteration never exceeds the real one r <- (r + V / r) / 2, so once the latter is within 1 of
+// sqrt(V) the former is at isqrt(V) or one above, and one more step settles it.  More steps are needed the
+// farther sqrt(V) lies from 2^16 on either side.  (Half of the 1 is left to the rounding of the doubles.)
+LnConst ln_const(int iters, int C) {
+    auto settled = [&](double x) {
+        double r = 65536.0;
+        for (int j = 1; j < iters; ++j) r = (r + x * x / r) / 2;
+        return r - x < 0.5;
+    };
+    const float inv2c = 1.0f / (2.0f * (float)C);
+    if (iters < 2) return {1, 0, inv2c};
+    double a = 1.0, b = 65536.0;  // the smallest root in reach: settled(b) holds
+    if (!settled(a)) {
+        for (int i = 0; i < 40; ++i) (settled((a + b) / 2) ? b : a) = (a + b) / 2;
+        a = b;
+    }
+    const double lo = a + 1.0;
+    double c = 65536.0, d = 16777215.0;  // the largest
+    if (!settled(d)) {
+        for (int i = 0; i < 40; ++i) (settled((c + d) / 2) ? c : d) = (c + d) / 2;
+        d = c;
+    }
+    const double hi = d - 1.0;
+    return {(uint64_t)(lo * lo), (uint64_t)(hi * hi), inv2c};
+}
+
 template <typename TIn, typename TOut>
 cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
     const int eb = sizeof(TIn), ob = sizeof(TOut);
@@ -552,9 +673,10 @@ cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
                        ((uintptr_t)p.X % 16) == 0 && ((uintptr_t)p.Y % (4 * ob)) == 0 &&
                        (((uintptr_t)p.beta | (uintptr_t)p.mult | (uintptr_t)p.shift) % 16) == 0 && p.C * eb <= 2048;
     if (tiled) {
+        const LnConst lc = ln_const(p.iters, p.C);
         const int nch = p.C * eb / 16;
-        const size_t smem = (size_t)3 * p.C * sizeof(int32_t);
-        auto go = [&](auto kern, int lpr) -> cudaError_t {
+        auto go = [&](auto kern, int lpr, int cpl) -> cudaError_t {
+            const size_t smem = (size_t)3 * lpr * cpl * (16 / eb) * sizeof(int32_t);
             int dev = 0, sms = 0, per_sm = 0;
             cudaError_t e = cudaGetDevice(&dev);
             if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -564,16 +686,19 @@ cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
             const int64_t rpc = 256 / lpr;
             const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(per_sm, 1) * sms,
                                                                         (p.rows + rpc - 1) / rpc));
-            kern<<<(unsigned)grid, 256, smem, s>>>(p);
+            kern<<<(unsigned)grid, 256, smem, s>>>(p, lc);
             return cudaGetLastError();
         };
         // chunks per lane: 6 for int16 rows (8 values each), 12 for int32 rows (4 values each), so a
         // lane holds at most 48 values; lanes per row from the row's chunk count
         constexpr int CPL = sizeof(TIn) == 2 ? 6 : 12;
-        if (nch <= 4 * CPL) return go(layernorm_rows<TIn, TOut, 4, CPL>, 4);
-        if (nch <= 8 * CPL) return go(layernorm_rows<TIn, TOut, 8, CPL>, 8);
-        if (nch <= 16 * CPL) return go(layernorm_rows<TIn, TOut, 16, CPL>, 16);
-        if (nch <= 32 * CPL) return go(layernorm_rows<TIn, TOut, 32, CPL>, 32);
+        // (rows of 192 and 384 fill their lanes and need no test of a chunk against the row's end)
+        if (nch == 4 * CPL) return go(layernorm_rows<TIn, TOut, 4, CPL, true>, 4, CPL);
+        if (nch == 8 * CPL) return go(layernorm_rows<TIn, TOut, 8, CPL, true>, 8, CPL);
+        if (nch <= 4 * CPL) return go(layernorm_rows<TIn, TOut, 4, CPL, false>, 4, CPL);
+        if (nch <= 8 * CPL) return go(layernorm_rows<TIn, TOut, 8, CPL, false>, 8, CPL);
+        if (nch <= 16 * CPL) return go(layernorm_rows<TIn, TOut, 16, CPL, false>, 16, CPL);
+        if (nch <= 32 * CPL) return go(layernorm_rows<TIn, TOut, 32, CPL, false>, 32, CPL);
     }
     const int rows_per_block = 8;
     dim3 grid((unsigned)((p.rows + rows_per_block - 1) / rows_per_block));

@@ -196,6 +196,27 @@ def test_int_layernorm(ilw, orc, C, in_bits, out_bits, iters):
     assert_same(host(got), want, f"ln C={C}")
 
 
+@pytest.mark.parametrize("rows,C,in_bits,out_bits,iters", [
+    (1, 192, 16, 8, 10), (33, 384, 32, 8, 10), (1030, 256, 32, 16, 4), (70, 384, 16, 16, 3), (65, 768, 16, 8, 16),
+    (130, 512, 32, 8, 12)])
+def test_int_layernorm_row_forms(ilw, orc, rows, C, in_bits, out_bits, iters):
+    """Neighbouring rows inside and outside the range of V whose root needs no Newton steps, rows with
+    V = s^2 + 2 s (the iteration alternates), rows of wide values, full and partly filled lanes."""
+    rng = np.random.default_rng(rows + C)
+    lim = (1 << (in_bits - 1)) - 1
+    amp = np.exp(rng.uniform(0, np.log(lim if in_bits == 16 else 1 << 20), size=(rows, 1)))
+    X = np.clip(np.rint(rng.standard_normal((rows, C)) * amp + rng.uniform(-1, 1, (rows, 1)) * amp), -lim, lim).astype(np.int32)
+    X[::7] = 0
+    X[::7, :8] = rng.integers(-1, 2, size=(len(X[::7]), 8))  # V = 0, 3, 8 = s^2 + 2 s among them
+    X[3::11, 0] = -lim - 1  # the type's lowest value
+    X = X.astype(np.int16 if in_bits == 16 else np.int32)
+    beta, mult, shift = synth.ln_params(7, f"lnr{C}", C)
+    if out_bits == 16:
+        shift = shift - 7
+    got = ilw.int_layernorm(dev(X), dev(beta), dev(mult), dev(shift), iters, out_bits)
+    assert_same(host(got), orc.int_layernorm(X, beta, mult, shift, iters, out_bits), f"ln rows {rows} x {C}")
+
+
 @pytest.mark.parametrize("C,in_bits", [(384, 16), (192, 32), (100, 16), (1000, 32)])
 def test_int_layernorm_f16_out(ilw, orc, C, in_bits):
     """out_bits ILW_I8_IN_F16: the int8 outputs carried in float16 (the encoder's form)."""

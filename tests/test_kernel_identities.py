@@ -150,6 +150,87 @@ def test_newton_early_exit_matches_fixed_iteration_count():
             assert _newton_early(V, iters) == _newton_fixed(V, iters), (V, iters)
 
 
+def _newton_range(iters):
+    """The V for which I-LayerNorm takes the root without the steps (the launch's own search)."""
+
+    def settled(x):
+        r = 65536.0
+        for _ in range(1, iters):
+            r = (r + x * x / r) / 2
+        return r - x < 0.5
+
+    def edge(out, inn):
+        for _ in range(40):
+            m = (out + inn) / 2
+            out, inn = (out, m) if settled(m) else (m, inn)
+        return inn
+
+    if iters < 2:
+        return 1, 0
+    lo = (1.0 if settled(1.0) else edge(1.0, 65536.0)) + 1.0
+    hi = (16777215.0 if settled(16777215.0) else edge(16777215.0, 65536.0)) - 1.0
+    return int(lo * lo), int(hi * hi)
+
+
+def _isqrt_u48(V, ulp):
+    """The kernels' integer square root: float32 reciprocal root (`ulp` units off), one step on the 32-bit
+    remainder, +-1."""
+    f32 = np.float32
+    vf = f32(float(f32(V >> 32)) * 4294967296.0 + float(f32(V & 0xFFFFFFFF)))
+    rs = f32(1.0 / np.sqrt(float(vf)))
+    rs = f32(rs + f32(ulp) * np.spacing(rs))
+    s = int(vf * rs)
+    rem = V - s * s
+    assert abs(rem) < 2**31
+    s += int(np.floor(f32(rem) * (f32(0.5) * rs)))
+    rem = V - s * s
+    assert abs(rem) < 2**31
+    if rem < 0:
+        s -= 1
+    elif rem > 2 * s:
+        s += 1
+    return s
+
+
+def _div_int31_u24(s, ulp):
+    """The kernels' floor((2^31 - 1) / s): float32 reciprocal (`ulp` units off), one step, +-1."""
+    f32 = np.float32
+    rc = f32(1.0 / s)
+    rc = f32(rc + f32(ulp) * np.spacing(rc))
+    q = int(f32(2147483648.0) * rc)
+    rem = 2**31 - 1 - q * s
+    assert abs(rem) < 2**31
+    dq = int(np.floor(f32(rem) * rc))
+    q, rem = q + dq, rem - dq * s
+    return q - 1 if rem < 0 else q + (rem >= s)
+
+
+@pytest.mark.parametrize("iters", [1, 2, 3, 4, 6, 10, 14, 16, 20])
+def test_newton_root_without_its_steps(iters):
+    """Inside the range of V that the launch works out from the step count, the fixed number of Newton
+    steps ends at isqrt(V) unless V = s^2 + 2 s: at the range's edges, at squares and at random."""
+    import math
+
+    rng = np.random.default_rng(iters)
+    lo, hi = _newton_range(iters)
+    if iters < 2:
+        assert lo > hi
+        return
+    a, b = math.isqrt(lo), math.isqrt(hi)
+    assert lo <= 2**32 <= hi < 2**48
+    roots = {a + d for d in range(40)} | {b - d for d in range(40)} | {65536 + d for d in range(-20, 21)}
+    roots |= {int(v) for v in np.exp(rng.uniform(np.log(a + 1), np.log(b), size=1500))}
+    Vs = {r * r + d for r in roots for d in (-1, 0, 1, r, 2 * r - 1, 2 * r, 2 * r + 1)}
+    Vs |= {int(v) for v in np.exp(rng.uniform(np.log(lo + 1), np.log(hi), size=3000))}
+    for V in Vs:
+        if lo <= V <= hi:
+            s = math.isqrt(V)
+            assert all(_isqrt_u48(V, u) == s for u in (-2, 0, 2)), V
+            assert all(_div_int31_u24(s, u) == (2**31 - 1) // s for u in (-2, 0, 2)), s
+            if V - s * s != 2 * s:
+                assert _newton_fixed(V, iters) == s, (V, iters)
+
+
 def test_shiftmax_output_from_shiftexp_parts():
     """Attention forms the Constrained Shiftmax output (I_exp F) >> sh from ShiftExp's parts: with
     I_exp = I_b << (k - q) and sh = 31 - k_out + 1 + s_d >= k, floor(I_exp F / 2^sh) equals
