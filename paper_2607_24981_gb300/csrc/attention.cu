@@ -118,6 +118,7 @@ struct Group {
 // are; otherwise they arrive as int8 and are converted on the way in.
 template <int DH, bool FASTQ, bool QF16, bool DIRECT>
 __global__ void __launch_bounds__(THREADS, 4) attn_kernel(const AttnParams p) {
+    grid_wait();
     constexpr int LDH = DH * 2 + 16;  // padded fp16 row (bytes): conflict-free ldmatrix
     constexpr int KS = DH / 16;       // k16 steps of q k^T
     constexpr int NT = DH / 8;        // n-tiles of P V
@@ -490,10 +491,10 @@ cudaError_t launch_attention(const AttnParams &p0, cudaStream_t s) {
     const bool direct = p.smx.s_d < 0 && p.smx.m_p + 15 <= p.smx.M_hw && 32 - p.smx.k_out >= p.smx.se.k;
 #define ILW_ATTN(DH, QF)                                                                          \
     do {                                                                                          \
-        if (fastq && direct) attn_kernel<DH, true, QF, true><<<grid, THREADS, 0, s>>>(p);         \
-        else if (fastq) attn_kernel<DH, true, QF, false><<<grid, THREADS, 0, s>>>(p);             \
-        else if (direct) attn_kernel<DH, false, QF, true><<<grid, THREADS, 0, s>>>(p);            \
-        else attn_kernel<DH, false, QF, false><<<grid, THREADS, 0, s>>>(p);                       \
+        if (fastq && direct) launch_after(attn_kernel<DH, true, QF, true>, grid, THREADS, 0, s, p);         \
+        else if (fastq) launch_after(attn_kernel<DH, true, QF, false>, grid, THREADS, 0, s, p);             \
+        else if (direct) launch_after(attn_kernel<DH, false, QF, true>, grid, THREADS, 0, s, p);            \
+        else launch_after(attn_kernel<DH, false, QF, false>, grid, THREADS, 0, s, p);                       \
     } while (0)
     if (p.qkv_f16) {
         if (p.dh == 64) ILW_ATTN(64, true);

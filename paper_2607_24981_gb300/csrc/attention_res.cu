@@ -367,6 +367,7 @@ __global__ void __launch_bounds__(kResThreads, 1) attn_res_kernel(const __grid_c
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     fence_before();
     __syncthreads();
     fence_after();
@@ -955,12 +956,14 @@ cudaError_t launch_res(const ResArgs &a, int clusters, cudaStream_t s) {
     cfg.blockDim = dim3(kResThreads);
     cfg.dynamicSmemBytes = (size_t)res_smem(a.nkp, CS);
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = CS;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, attn_res_kernel<CS>, a);
 }
 

@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(kThreadsTc, kMinBlocks) attn_tc_kernel(const _
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     fence_before();
     __syncthreads();
     fence_after();
@@ -749,7 +750,7 @@ cudaError_t launch_tc_one(const TcArgs &a, dim3 grid, size_t smem, cudaStream_t 
     const cudaError_t attr =
         raise_smem_limit(limit, (const void *)attn_tc_kernel<FASTQ, DIRECT, SUM4, MAYPAIR, MAYFULL>, (int)smem);
     if (attr != cudaSuccess) return attr;
-    attn_tc_kernel<FASTQ, DIRECT, SUM4, MAYPAIR, MAYFULL><<<grid, kThreadsTc, smem, s>>>(a);
+    launch_after(attn_tc_kernel<FASTQ, DIRECT, SUM4, MAYPAIR, MAYFULL>, grid, kThreadsTc, smem, s, a);
     return cudaGetLastError();
 }
 // windows: one form; global attention: full blocks compiled apart, and paired last tiles when the

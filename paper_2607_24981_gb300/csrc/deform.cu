@@ -12,6 +12,7 @@ namespace ilw {
 namespace {
 
 __global__ void __launch_bounds__(256) deform_kernel(const DeformParams p, int64_t total) {
+    grid_wait();
     int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= total) return;
     const int quads = p.dh >> 2;
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(256) deform_kernel(const DeformParams p, int64
 cudaError_t launch_deform(const DeformParams &p, cudaStream_t s) {
     int64_t total = (int64_t)p.B * p.Q * p.H * (p.dh / 4);
     if (total == 0) return cudaSuccess;
-    deform_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(p, total);
+    launch_after(deform_kernel, (unsigned)((total + 255) / 256), 256, 0, s, p, total);
     return cudaGetLastError();
 }
 

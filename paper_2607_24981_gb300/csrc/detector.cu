@@ -26,6 +26,7 @@ __device__ __forceinline__ void load4<int32_t>(const int32_t *p, int64_t (&v)[4]
 // One thread per 4 consecutive elements of a row (C % 4 == 0, rows 8/16-byte aligned).
 template <typename TIn, typename TOut>
 __global__ void __launch_bounds__(256) requant_kernel(const RequantParams p) {
+    grid_wait();
     const int32_t cq = p.C >> 2;
     const int64_t total = p.rows * cq;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -58,6 +59,7 @@ __global__ void __launch_bounds__(256) requant_kernel(const RequantParams p) {
 __global__ void __launch_bounds__(256) resample_kernel(const int8_t *__restrict__ X, int64_t x_bstride, int32_t B,
                                                        int32_t Hi, int32_t Wi, int32_t C, int8_t *__restrict__ Y,
                                                        int64_t y_bstride, int32_t Ho, int32_t Wo) {
+    grid_wait();
     const int32_t c16 = C >> 4;
     const int64_t total = (int64_t)B * Ho * Wo * c16;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
@@ -77,6 +79,7 @@ __global__ void __launch_bounds__(256) resample_kernel(const int8_t *__restrict_
 // outputs (16 bytes) per item.
 __global__ void head_pad64_kernel(const int8_t *__restrict__ X, int64_t ldx, int64_t M, int32_t nh, int32_t dh,
                                   __half *__restrict__ Y) {
+    grid_wait();
     const int64_t per_row = (int64_t)nh * 8;  // 16-byte chunks of a padded row
     const int64_t items = M * per_row;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
@@ -100,6 +103,7 @@ __global__ void head_pad64_kernel(const int8_t *__restrict__ X, int64_t ldx, int
 // The inverse for int8 rows: O[m, h dh + c] = Y[m, h 64 + c] for c < dh.
 __global__ void head_compact_kernel(const int8_t *__restrict__ Y, int64_t ldy, int64_t M, int32_t H, int32_t dh,
                                     int8_t *__restrict__ O, int64_t ldo) {
+    grid_wait();
     const int64_t per_row = (int64_t)H * dh;
     const int64_t items = M * per_row;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += (int64_t)gridDim.x * blockDim.x) {
@@ -122,13 +126,13 @@ cudaError_t launch_requant(const RequantParams &p, cudaStream_t s) {
     if (items == 0) return cudaSuccess;
     const unsigned g = grid_for(items);
     if (p.in_bits == 16) {
-        if (p.out_bits == 8) requant_kernel<int16_t, int8_t><<<g, 256, 0, s>>>(p);
-        else if (p.out_bits == 16) requant_kernel<int16_t, int16_t><<<g, 256, 0, s>>>(p);
-        else requant_kernel<int16_t, int32_t><<<g, 256, 0, s>>>(p);
+        if (p.out_bits == 8) launch_after(requant_kernel<int16_t, int8_t>, g, 256, 0, s, p);
+        else if (p.out_bits == 16) launch_after(requant_kernel<int16_t, int16_t>, g, 256, 0, s, p);
+        else launch_after(requant_kernel<int16_t, int32_t>, g, 256, 0, s, p);
     } else {
-        if (p.out_bits == 8) requant_kernel<int32_t, int8_t><<<g, 256, 0, s>>>(p);
-        else if (p.out_bits == 16) requant_kernel<int32_t, int16_t><<<g, 256, 0, s>>>(p);
-        else requant_kernel<int32_t, int32_t><<<g, 256, 0, s>>>(p);
+        if (p.out_bits == 8) launch_after(requant_kernel<int32_t, int8_t>, g, 256, 0, s, p);
+        else if (p.out_bits == 16) launch_after(requant_kernel<int32_t, int16_t>, g, 256, 0, s, p);
+        else launch_after(requant_kernel<int32_t, int32_t>, g, 256, 0, s, p);
     }
     return cudaGetLastError();
 }
@@ -136,13 +140,13 @@ cudaError_t launch_requant(const RequantParams &p, cudaStream_t s) {
 cudaError_t launch_head_pad64(const int8_t *X, int64_t ldx, int64_t M, int32_t nh, int32_t dh, __half *Y,
                               cudaStream_t s) {
     if (M == 0 || nh == 0) return cudaSuccess;
-    head_pad64_kernel<<<grid_for(M * nh * 8), 256, 0, s>>>(X, ldx, M, nh, dh, Y);
+    launch_after(head_pad64_kernel, grid_for(M * nh * 8), 256, 0, s, X, ldx, M, nh, dh, Y);
     return cudaGetLastError();
 }
 cudaError_t launch_head_compact(const int8_t *Y, int64_t ldy, int64_t M, int32_t H, int32_t dh, int8_t *O, int64_t ldo,
                                 cudaStream_t s) {
     if (M == 0 || H == 0) return cudaSuccess;
-    head_compact_kernel<<<grid_for(M * H * dh), 256, 0, s>>>(Y, ldy, M, H, dh, O, ldo);
+    launch_after(head_compact_kernel, grid_for(M * H * dh), 256, 0, s, Y, ldy, M, H, dh, O, ldo);
     return cudaGetLastError();
 }
 
@@ -150,7 +154,7 @@ cudaError_t launch_resample(const int8_t *X, int64_t x_bstride, int32_t B, int32
                             int8_t *Y, int64_t y_bstride, int32_t Ho, int32_t Wo, cudaStream_t s) {
     const int64_t items = (int64_t)B * Ho * Wo * (C / 16);
     if (items == 0) return cudaSuccess;
-    resample_kernel<<<grid_for(items), 256, 0, s>>>(X, x_bstride, B, Hi, Wi, C, Y, y_bstride, Ho, Wo);
+    launch_after(resample_kernel, grid_for(items), 256, 0, s, X, x_bstride, B, Hi, Wi, C, Y, y_bstride, Ho, Wo);
     return cudaGetLastError();
 }
 

@@ -18,6 +18,7 @@ constexpr int kGeluTabBytes = 65536;  // 65535 entries, padded to 16 bytes
 __device__ __align__(16) int8_t g_gelu_tab[kGeluSlots][kGeluTabBytes];
 
 __global__ void gelu_table_kernel(int8_t *tab, GeluC c, int32_t m_g, int32_t s_g) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < kGeluTabBytes) {
         const int32_t g = min(i, 65534) - 32767;
@@ -71,7 +72,7 @@ const int8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStre
     }
     int8_t *tab = base[dev] + (size_t)slot * kGeluTabBytes;
     if (!built[dev][slot]) {
-        gelu_table_kernel<<<kGeluTabBytes / 256, 256, 0, s>>>(tab, c, m_g, s_g);
+        launch_after(gelu_table_kernel, kGeluTabBytes / 256, 256, 0, s, tab, c, m_g, s_g);
         if ((*err = cudaGetLastError()) != cudaSuccess) return nullptr;
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if ((*err = cudaStreamIsCapturing(s, &cs)) != cudaSuccess) return nullptr;
@@ -85,6 +86,7 @@ const int8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStre
 
 // int8 weight -> fp16 operand copy (|w| <= 127: exact)
 __global__ void pack_weight_kernel(const int8_t *W, int64_t n, __half *w16) {
+    grid_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) w16[i] = __int2half_rn((int)W[i]);
 }
@@ -179,7 +181,7 @@ void gemm_set_debug_wait(int32_t skip, long long cycles) {
 
 cudaError_t launch_pack_weight(const int8_t *W, int32_t N, int32_t K, void *packed, cudaStream_t s) {
     const int64_t n = (int64_t)N * K;
-    pack_weight_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(W, n, (__half *)packed);
+    launch_after(pack_weight_kernel, (unsigned)((n + 255) / 256), 256, 0, s, W, n, (__half *)packed);
     return cudaGetLastError();
 }
 

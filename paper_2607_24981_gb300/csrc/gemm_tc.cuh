@@ -570,6 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1013,7 +1014,7 @@ cudaError_t launch_tc(TcParams<NB> &tp, cudaStream_t s) {
         per_n = per_n < 1 ? 1 : (per_n > tiles_m ? tiles_m : per_n);
         grid = per_n * tp.tiles_n;
     }
-    gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES><<<grid, kThreads, smem, s>>>(tp);
+    launch_after(gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES>, grid, kThreads, smem, s, tp);
     return cudaGetLastError();
 }
 

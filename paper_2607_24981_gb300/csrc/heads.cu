@@ -24,6 +24,7 @@ __device__ __forceinline__ int32_t int_sigmoid1(int32_t x, const ShiftExpC &se, 
 
 __global__ void __launch_bounds__(256) int_sigmoid_kernel(const int32_t *__restrict__ X, int32_t *__restrict__ Y,
                                                           int64_t n, ShiftExpC se, int32_t out_sh) {
+    grid_wait();
     const int64_t n4 = n / 4;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
         const int4 v = ((const int4 *)X)[i];
@@ -36,6 +37,7 @@ __global__ void __launch_bounds__(256) int_sigmoid_kernel(const int32_t *__restr
 
 // ReLU of int8 values, four per thread step (n4 words), then the tail
 __global__ void __launch_bounds__(256) relu_i8_kernel(const int8_t *__restrict__ X, int8_t *__restrict__ Y, int64_t n) {
+    grid_wait();
     const int64_t n4 = n / 4;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t w = ((const uint32_t *)X)[i];
@@ -64,6 +66,7 @@ template <int VPT>
 __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t N,
                                                             int32_t kpad, int32_t K, int32_t *__restrict__ vals,
                                                             int32_t *__restrict__ idx) {
+    grid_wait();
     extern __shared__ unsigned long long keys[];  // kpad
     __shared__ uint32_t part[2][32];
     const int32_t *s = S + (int64_t)blockIdx.x * lds;
@@ -176,6 +179,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__res
 // the warp combines the lanes' candidates (larger value, or equal value and smaller index, wins).
 __global__ void __launch_bounds__(256) top1_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t rows, int32_t N,
                                                    int32_t *__restrict__ vals, int32_t *__restrict__ idx) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t wpr = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += wpr) {
@@ -209,6 +213,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint32_t *__rest
                                                           int64_t src_rows, const int32_t *__restrict__ idx, int64_t n,
                                                           int64_t batches, int64_t roww, uint32_t *__restrict__ dst,
                                                           int64_t dst_ldw, int *status) {
+    grid_wait();
     const int64_t total = n * batches * roww;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = t / roww, w = t - i * roww;
@@ -233,6 +238,7 @@ __device__ __forceinline__ int64_t ip1702(int32_t x) {
 __global__ void __launch_bounds__(256) ivit_shiftgelu_kernel(const int32_t *__restrict__ X, int64_t ldx, int64_t rows,
                                                              int32_t L, int32_t *__restrict__ Y, int64_t ldy,
                                                              ShiftExpC se, int32_t out_sh) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t wpr = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t r = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); r < rows; r += wpr) {
@@ -263,20 +269,20 @@ unsigned grid_for(int64_t work, int per_block) {
 cudaError_t launch_int_sigmoid(const int32_t *X, int32_t *Y, int64_t n, const ShiftExpC &se, int32_t k_out,
                                cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    int_sigmoid_kernel<<<grid_for((n + 3) / 4, 256), 256, 0, s>>>(X, Y, n, se, 32 - k_out);
+    launch_after(int_sigmoid_kernel, grid_for((n + 3) / 4, 256), 256, 0, s, X, Y, n, se, 32 - k_out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_ivit_shiftgelu(const int32_t *X, int64_t ldx, int64_t rows, int32_t L, int32_t *Y, int64_t ldy,
                                   const GeluC &c, cudaStream_t s) {
     if (rows == 0) return cudaSuccess;
-    ivit_shiftgelu_kernel<<<grid_for((rows + 7) / 8, 1), 256, 0, s>>>(X, ldx, rows, L, Y, ldy, c.se, c.out_sh);
+    launch_after(ivit_shiftgelu_kernel, grid_for((rows + 7) / 8, 1), 256, 0, s, X, ldx, rows, L, Y, ldy, c.se, c.out_sh);
     return cudaGetLastError();
 }
 
 cudaError_t launch_relu_i8(const int8_t *X, int8_t *Y, int64_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    relu_i8_kernel<<<grid_for((n + 3) / 4, 256), 256, 0, s>>>(X, Y, n);
+    launch_after(relu_i8_kernel, grid_for((n + 3) / 4, 256), 256, 0, s, X, Y, n);
     return cudaGetLastError();
 }
 
@@ -284,7 +290,7 @@ cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, 
                         int32_t *idx, cudaStream_t s) {
     if (rows == 0) return cudaSuccess;
     if (K == 1) {
-        top1_kernel<<<grid_for(((int64_t)rows + 7) / 8, 1), 256, 0, s>>>(S, lds, rows, N, vals, idx);
+        launch_after(top1_kernel, grid_for(((int64_t)rows + 7) / 8, 1), 256, 0, s, S, lds, rows, N, vals, idx);
         return cudaGetLastError();
     }
     int kpad = 2;
@@ -293,7 +299,7 @@ cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, 
     auto go = [&](auto kern, SmemLimit &limit) -> cudaError_t {
         const cudaError_t e = raise_smem_limit(limit, (const void *)kern, 16384 * 8);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)rows, kTopkThreads, smem, s>>>(S, lds, N, kpad, K, vals, idx);
+        launch_after(kern, (unsigned)rows, kTopkThreads, smem, s, S, lds, N, kpad, K, vals, idx);
         return cudaGetLastError();
     };
     static SmemLimit l2, l9, l16;
@@ -305,8 +311,7 @@ cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, 
 cudaError_t launch_gather_rows(const void *src, int64_t src_ld_bytes, int64_t src_rows, const int32_t *idx, int64_t n,
                                int64_t batches, int64_t row_bytes, void *dst, int64_t dst_ld_bytes, cudaStream_t s) {
     if (n == 0 || batches == 0 || row_bytes == 0) return cudaSuccess;
-    gather_rows_kernel<<<grid_for(n * batches * (row_bytes / 4), 256), 256, 0, s>>>(
-        (const uint32_t *)src, src_ld_bytes / 4, src_rows, idx, n, batches, row_bytes / 4, (uint32_t *)dst,
+    launch_after(gather_rows_kernel, grid_for(n * batches * (row_bytes / 4), 256), 256, 0, s, (const uint32_t *)src, src_ld_bytes / 4, src_rows, idx, n, batches, row_bytes / 4, (uint32_t *)dst,
         dst_ld_bytes / 4, status_word_ptr());
     return cudaGetLastError();
 }

@@ -13,6 +13,7 @@ namespace {
 __global__ void __launch_bounds__(256) patchify_kernel(const int8_t *__restrict__ img, int32_t Cin, int32_t Hh,
                                                        int32_t Ww, int32_t p, int64_t total,
                                                        int8_t *__restrict__ A) {
+    grid_wait();
     int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= total) return;
     const int segs = p >> 4;  // 16-byte segments per patch row
@@ -40,6 +41,7 @@ __device__ __forceinline__ uint32_t i8x2_f16(uint32_t w) {
 __global__ void __launch_bounds__(256) patchify_f16_kernel(const int8_t *__restrict__ img, int32_t Cin, int32_t Hh,
                                                            int32_t Ww, int32_t p, int64_t total,
                                                            __half *__restrict__ A) {
+    grid_wait();
     int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (id >= total) return;
     const int segs = p >> 4;
@@ -68,7 +70,7 @@ cudaError_t launch_patchify_f16(const int8_t *img, int32_t B, int32_t Cin, int32
                                 __half *A, cudaStream_t s) {
     int64_t total = (int64_t)B * (Hh / p) * (Ww / p) * Cin * p * (p / 16);
     if (total == 0) return cudaSuccess;
-    patchify_f16_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(img, Cin, Hh, Ww, p, total, A);
+    launch_after(patchify_f16_kernel, (unsigned)((total + 255) / 256), 256, 0, s, img, Cin, Hh, Ww, p, total, A);
     return cudaGetLastError();
 }
 
@@ -76,7 +78,7 @@ cudaError_t launch_patchify(const int8_t *img, int32_t B, int32_t Cin, int32_t H
                             int8_t *A, cudaStream_t s) {
     int64_t total = (int64_t)B * (Hh / p) * (Ww / p) * Cin * p * (p / 16);
     if (total == 0) return cudaSuccess;
-    patchify_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(img, Cin, Hh, Ww, p, total, A);
+    launch_after(patchify_kernel, (unsigned)((total + 255) / 256), 256, 0, s, img, Cin, Hh, Ww, p, total, A);
     return cudaGetLastError();
 }
 

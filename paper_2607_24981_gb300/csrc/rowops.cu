@@ -76,6 +76,7 @@ template <int NCH, int LANES, bool FASTQ, bool SUM4>
 __global__ void __launch_bounds__(256) shiftmax_rows_vec(const int32_t *__restrict__ X, int64_t ldx,
                                                           int64_t rows, int32_t len, const ShiftmaxC c,
                                                           uint8_t *__restrict__ P, int64_t ldp) {
+    grid_wait();
     constexpr int RPW = 32 / LANES;
     const int lane = threadIdx.x & 31, sub = lane % LANES;
     const int64_t row = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * RPW + lane / LANES;
@@ -156,6 +157,7 @@ __global__ void __launch_bounds__(256) shiftmax_rows_vec(const int32_t *__restri
 __global__ void __launch_bounds__(256) shiftmax_rows_generic(const int32_t *__restrict__ X, int64_t ldx,
                                                               int64_t rows, int32_t len, const ShiftmaxC c,
                                                               uint8_t *__restrict__ P, int64_t ldp) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
@@ -185,6 +187,7 @@ __device__ __forceinline__ int32_t gelu_one(int32_t x, const GeluC &c) {
 
 __global__ void __launch_bounds__(256) sdshiftgelu_vec(const int4 *__restrict__ X, int4 *__restrict__ Y,
                                                         int64_t n4, const GeluC c) {
+    grid_wait();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
         int4 v = __ldcs(X + i);
         int4 o;
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(256) sdshiftgelu_vec(const int4 *__restrict__ 
 // function (exact by construction) and streams the data through lookups.
 __global__ void __launch_bounds__(256) sdshiftgelu_table(const int4 *__restrict__ X, int4 *__restrict__ Y, int64_t n4,
                                                           const GeluC c, int32_t T) {
+    grid_wait();
     extern __shared__ uint8_t tab[];
     for (int i = threadIdx.x; i <= 2 * T; i += blockDim.x) tab[i] = (uint8_t)gelu_idiv(i - T, c);
     __syncthreads();
@@ -223,6 +227,7 @@ __global__ void __launch_bounds__(256) sdshiftgelu_table(const int4 *__restrict_
 }
 
 __global__ void sdshiftgelu_tail(const int32_t *X, int32_t *Y, int64_t start, int64_t n, const GeluC c) {
+    grid_wait();
     int64_t i = start + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) Y[i] = gelu_one(X[i], c);
 }
@@ -432,6 +437,7 @@ __device__ __noinline__ LnRow ln_row_general(int64_t S, int64_t Q, int32_t C, in
 // (or for rows with iters = 0 and V >= 2^32) the 64-bit formulas run.
 template <typename TIn, typename TOut, int LPR, int CPL, bool FULL>
 __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const LnConst lc) {
+    grid_wait();
     extern __shared__ __align__(16) int32_t ln_par[];  // beta, mult, shift of CP columns
     constexpr int EB = sizeof(TIn), EPC = 16 / EB;      // elements per 16-byte chunk
     constexpr int RPW = 32 / LPR, CP = LPR * CPL * EPC;
@@ -593,6 +599,7 @@ __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const
 
 template <typename TIn, typename TOut, int EPL>
 __global__ void __launch_bounds__(256) layernorm_kernel(const LnParams p) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= p.rows) return;
@@ -686,7 +693,7 @@ cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
             const int64_t rpc = 256 / lpr;
             const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(per_sm, 1) * sms,
                                                                         (p.rows + rpc - 1) / rpc));
-            kern<<<(unsigned)grid, 256, smem, s>>>(p, lc);
+            launch_after(kern, (unsigned)grid, 256, smem, s, p, lc);
             return cudaGetLastError();
         };
         // chunks per lane: 6 for int16 rows (8 values each), 12 for int32 rows (4 values each), so a
@@ -702,13 +709,13 @@ cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
     }
     const int rows_per_block = 8;
     dim3 grid((unsigned)((p.rows + rows_per_block - 1) / rows_per_block));
-    if (p.C <= 128) layernorm_kernel<TIn, TOut, 4><<<grid, 256, 0, s>>>(p);
-    else if (p.C <= 256) layernorm_kernel<TIn, TOut, 8><<<grid, 256, 0, s>>>(p);
-    else if (p.C <= 384) layernorm_kernel<TIn, TOut, 12><<<grid, 256, 0, s>>>(p);
-    else if (p.C <= 512) layernorm_kernel<TIn, TOut, 16><<<grid, 256, 0, s>>>(p);
-    else if (p.C <= 1024) layernorm_kernel<TIn, TOut, 32><<<grid, 256, 0, s>>>(p);
-    else if (p.C <= 2048) layernorm_kernel<TIn, TOut, 64><<<grid, 256, 0, s>>>(p);
-    else layernorm_kernel<TIn, TOut, 128><<<grid, 256, 0, s>>>(p);
+    if (p.C <= 128) launch_after(layernorm_kernel<TIn, TOut, 4>, grid, 256, 0, s, p);
+    else if (p.C <= 256) launch_after(layernorm_kernel<TIn, TOut, 8>, grid, 256, 0, s, p);
+    else if (p.C <= 384) launch_after(layernorm_kernel<TIn, TOut, 12>, grid, 256, 0, s, p);
+    else if (p.C <= 512) launch_after(layernorm_kernel<TIn, TOut, 16>, grid, 256, 0, s, p);
+    else if (p.C <= 1024) launch_after(layernorm_kernel<TIn, TOut, 32>, grid, 256, 0, s, p);
+    else if (p.C <= 2048) launch_after(layernorm_kernel<TIn, TOut, 64>, grid, 256, 0, s, p);
+    else launch_after(layernorm_kernel<TIn, TOut, 128>, grid, 256, 0, s, p);
     return cudaGetLastError();
 }
 
@@ -726,10 +733,10 @@ cudaError_t launch_shiftmax_rows(const int32_t *X, int64_t ldx, int64_t rows, in
     auto g = [&](int lanes) { return dim3((unsigned)((rows + 8 * (32 / lanes) - 1) / (8 * (32 / lanes)))); };
     const bool s4 = ((int64_t)c.se.I0 << c.se.k) < ((int64_t)1 << 30);
 #define ILW_SMX(NCH, LANES)                                                                                         \
-    (fq ? (s4 ? (shiftmax_rows_vec<NCH, LANES, true, true><<<g(LANES), 256, 0, s>>>(X, ldx, rows, len, c, P, ldp), 0)  \
-              : (shiftmax_rows_vec<NCH, LANES, true, false><<<g(LANES), 256, 0, s>>>(X, ldx, rows, len, c, P, ldp), 0)) \
-        : (s4 ? (shiftmax_rows_vec<NCH, LANES, false, true><<<g(LANES), 256, 0, s>>>(X, ldx, rows, len, c, P, ldp), 0) \
-              : (shiftmax_rows_vec<NCH, LANES, false, false><<<g(LANES), 256, 0, s>>>(X, ldx, rows, len, c, P, ldp), 0)))
+    (fq ? (s4 ? (launch_after(shiftmax_rows_vec<NCH, LANES, true, true>, g(LANES), 256, 0, s, X, ldx, rows, len, c, P, ldp), 0)  \
+              : (launch_after(shiftmax_rows_vec<NCH, LANES, true, false>, g(LANES), 256, 0, s, X, ldx, rows, len, c, P, ldp), 0)) \
+        : (s4 ? (launch_after(shiftmax_rows_vec<NCH, LANES, false, true>, g(LANES), 256, 0, s, X, ldx, rows, len, c, P, ldp), 0) \
+              : (launch_after(shiftmax_rows_vec<NCH, LANES, false, false>, g(LANES), 256, 0, s, X, ldx, rows, len, c, P, ldp), 0)))
     if (vec && len <= 64) ILW_SMX(4, 4);
     else if (vec && len <= 128) ILW_SMX(4, 8);
     else if (vec && len <= 416) ILW_SMX(13, 8);
@@ -737,7 +744,7 @@ cudaError_t launch_shiftmax_rows(const int32_t *X, int64_t ldx, int64_t rows, in
     else if (vec && len <= 1664) ILW_SMX(13, 32);
     else if (vec && len <= 2048) ILW_SMX(16, 32);
 #undef ILW_SMX
-    else shiftmax_rows_generic<<<grid, 256, 0, s>>>(X, ldx, rows, len, c, P, ldp);
+    else launch_after(shiftmax_rows_generic, grid, 256, 0, s, X, ldx, rows, len, c, P, ldp);
     return cudaGetLastError();
 }
 
@@ -756,15 +763,15 @@ cudaError_t launch_sdshiftgelu(const int32_t *X, int32_t *Y, int64_t n, const Ge
             if (e != cudaSuccess) return e;
             int64_t blocks = (n4 + 255) / 256;
             if (blocks > 6 * (int64_t)sm_count()) blocks = 6 * (int64_t)sm_count();
-            sdshiftgelu_table<<<(unsigned)blocks, 256, smem, s>>>((const int4 *)X, (int4 *)Y, n4, c, T);
+            launch_after(sdshiftgelu_table, (unsigned)blocks, 256, smem, s, (const int4 *)X, (int4 *)Y, n4, c, T);
         } else if (n4) {
             int64_t blocks = (n4 + 255) / 256;
             if (blocks > 16 * (int64_t)sm_count()) blocks = 16 * (int64_t)sm_count();
-            sdshiftgelu_vec<<<(unsigned)blocks, 256, 0, s>>>((const int4 *)X, (int4 *)Y, n4, c);
+            launch_after(sdshiftgelu_vec, (unsigned)blocks, 256, 0, s, (const int4 *)X, (int4 *)Y, n4, c);
         }
     }
     int64_t start = n4 * 4;
-    if (start < n) sdshiftgelu_tail<<<(unsigned)((n - start + 255) / 256), 256, 0, s>>>(X, Y, start, n, c);
+    if (start < n) launch_after(sdshiftgelu_tail, (unsigned)((n - start + 255) / 256), 256, 0, s, X, Y, start, n, c);
     return cudaGetLastError();
 }
 

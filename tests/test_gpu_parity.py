@@ -404,3 +404,49 @@ def test_block_forward(ilw, orc, cfg):
                           m_r=bp["m_r2"], s_r=bp["s_r2"])
     assert_same(host(y2), y_ref, "y via ops")
     ilw.device_status()
+
+
+# ------------------------------------------------------------- launches that overlap the one before
+@pytest.mark.parametrize("M", [40, 3000])
+def test_launches_follow_one_another(ilw, M):
+    """A kernel may start before the one ahead of it on the stream has written its results: chains in which
+    every launch reads what the last one wrote, buffers are rewritten in place and reused, and copies and
+    a forked stream come between, back to back, and recorded as a graph and replayed, against the same
+    chain with a synchronisation after every call."""
+    N = 192
+    x0 = dev(synth.uniform_int(11, f"chain{M}", (M, N), -3000, 3000, np.int16))
+    W, b, m, s = synth.gemm_params(11, "chainW", N, N, 73.0, 3000.0, "literal")
+    Wp, b, m, s = ilw.pack_weight(dev(W)), dev(b), dev(m), dev(s)
+    ln = [dev(a) for a in synth.ln_params(11, "chainln", N)]
+    x, x8, r8, y, c = (torch.empty((M, N), dtype=t, device="cuda")
+                       for t in (torch.int16, torch.int8, torch.int8, torch.int16, torch.int16))
+    side = torch.cuda.Stream()
+
+    def chain(sync=lambda: None):
+        x.copy_(x0), sync()
+        for i in range(6):
+            ilw.int_layernorm(x, *ln, out=x8), sync()
+            main = torch.cuda.current_stream()
+            side.wait_stream(main)
+            with torch.cuda.stream(side):  # the fork reads x8 while the main stream does
+                ilw.relu_i8(x8, out=r8), sync()
+            ilw.gemm_requant(x8, Wp, N, b, m, s, 16, res=x, m_r=3 << 28, s_r=30, out=x), sync()
+            main.wait_stream(side)
+            ilw.gemm_requant(r8, Wp, N, b, m, s, 16, out=y), sync()
+            c.copy_(y), sync()
+            ilw.requant(x, 1 << 30, 31, Z=c, m2=1 << 30, s2=31, out_bits=16, out=x), sync()
+        return x.clone()
+
+    want = chain(torch.cuda.synchronize)
+    assert len(torch.unique(want)) > 100
+    for _ in range(20):
+        got = chain()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = chain()
+    for _ in range(20):
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
