@@ -9,20 +9,20 @@ namespace ilw {
 namespace {
 
 // SD-ShiftGELU output tables, one slot per parameter set (I0, k_inter, k_out, m_g, s_g): entry
-// g + 32767 is sat8(rq(g * I_div(g); m_g, s_g)) for every int16 value g (Algorithm 1 followed by the
+// g + 32767 is sat8(rq(g * I_div(g); m_g, s_g)) + 128 for every int16 value g (Algorithm 1 followed by the
 // output requantisation), a pure function of g.  A slot, once given to a parameter set, keeps it
 // for the life of the process: kernels in flight on other streams and captured graphs hold its
 // address, so it is never rebuilt for another set.  A parameter set beyond the last slot is refused.
 constexpr int kGeluSlots = 256;  // 16 MiB per device
 constexpr int kGeluTabBytes = 65536;  // 65535 entries, padded to 16 bytes
-__device__ __align__(16) int8_t g_gelu_tab[kGeluSlots][kGeluTabBytes];
+__device__ __align__(16) uint8_t g_gelu_tab[kGeluSlots][kGeluTabBytes];
 
-__global__ void gelu_table_kernel(int8_t *tab, GeluC c, int32_t m_g, int32_t s_g) {
+__global__ void gelu_table_kernel(uint8_t *tab, GeluC c, int32_t m_g, int32_t s_g) {
     grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < kGeluTabBytes) {
         const int32_t g = min(i, 65534) - 32767;
-        tab[i] = (int8_t)sat8(rq((int64_t)g * gelu_idiv(g, c), m_g, s_g));
+        tab[i] = (uint8_t)(sat8(rq((int64_t)g * gelu_idiv(g, c), m_g, s_g)) + 128);
     }
 }
 
@@ -31,7 +31,7 @@ __global__ void gelu_table_kernel(int8_t *tab, GeluC c, int32_t m_g, int32_t s_g
 // every stream; a build recorded into a graph is repeated by each replay until an eager call builds it
 // (every replay writes the same bytes, since the slot never changes hands).  With every slot taken,
 // a new parameter set gets cudaErrorMemoryAllocation and nothing is launched.
-const int8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStream_t s, cudaError_t *err) {
+const uint8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStream_t s, cudaError_t *err) {
     struct Key {
         int dev;
         int32_t I0, k, out_sh, m_g, s_g;
@@ -43,7 +43,7 @@ const int8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStre
     static Key keys[64][kGeluSlots];
     static bool built[64][kGeluSlots] = {};
     static int nused[64] = {};
-    static int8_t *base[64] = {};
+    static uint8_t *base[64] = {};
     *err = cudaSuccess;
     int dev = 0;
     if ((*err = cudaGetDevice(&dev)) != cudaSuccess) return nullptr;
@@ -55,7 +55,7 @@ const int8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStre
     if (!base[dev]) {
         void *b = nullptr;
         if ((*err = cudaGetSymbolAddress(&b, g_gelu_tab)) != cudaSuccess) return nullptr;
-        base[dev] = (int8_t *)b;
+        base[dev] = (uint8_t *)b;
     }
     const Key key{dev, c.se.I0, c.se.k, c.out_sh, m_g, s_g};
     int slot = -1;
@@ -70,7 +70,7 @@ const int8_t *gelu_table_impl(const GeluC &c, int32_t m_g, int32_t s_g, cudaStre
         keys[dev][slot] = key;
         built[dev][slot] = false;
     }
-    int8_t *tab = base[dev] + (size_t)slot * kGeluTabBytes;
+    uint8_t *tab = base[dev] + (size_t)slot * kGeluTabBytes;
     if (!built[dev][slot]) {
         launch_after(gelu_table_kernel, kGeluTabBytes / 256, 256, 0, s, tab, c, m_g, s_g);
         if ((*err = cudaGetLastError()) != cudaSuccess) return nullptr;
@@ -161,7 +161,7 @@ bool gemm_make_map(CUtensorMap *m, const void *base, CUtensorMapDataType dt, int
                    int64_t ld, int box_cols, int box_rows, CUtensorMapSwizzle sw) {
     return make_map_impl(m, base, dt, esize, rows, cols, ld, box_cols, box_rows, sw);
 }
-const int8_t *gemm_gelu_table(const GeluC &c, int32_t m_g, int32_t s_g, cudaStream_t s, cudaError_t *err) {
+const uint8_t *gemm_gelu_table(const GeluC &c, int32_t m_g, int32_t s_g, cudaStream_t s, cudaError_t *err) {
     return gelu_table_impl(c, m_g, s_g, s, err);
 }
 
@@ -213,19 +213,19 @@ cudaError_t launch_gemm(const GemmProblem &gp, const EpiParams &ep, cudaStream_t
         };
         if (gelu) {  // 192-wide measured faster inside the encoder step even at 6 vs 8 rounds (FC1)
             if (n192) return run<192, 3, 1, true, false, true>(gp, ep, s);
-            if (K <= kSegK && smem_bytes<128, 3, KIND_GELU8, true, true>(nkb * 128 * 128) <= kSmemMax)
-                return run<128, 3, 1, true, true, true>(gp, ep, s);
+            if (K <= kSegK && smem_bytes<128, 6, KIND_GELU8, true, true>(nkb * 128 * 128, 0, 3) <= kSmemMax)
+                return run<128, 6, 1, true, true, true>(gp, ep, s);
             return run<128, 3, 1, true, false, true>(gp, ep, s);
         }
         if (K <= kSegK) {
-            const bool w192 = n192 && smem_bytes<192, 3, KIND_RQ8, true, true>(nkb * 192 * 128) <= kSmemMax;
-            const bool w128 = smem_bytes<128, 3, KIND_RQ8, true, true>(nkb * 128 * 128) <= kSmemMax;
+            const bool w192 = n192 && smem_bytes<192, 6, KIND_RQ8, true, true>(nkb * 192 * 128, 0, 3) <= kSmemMax;
+            const bool w128 = smem_bytes<128, 6, KIND_RQ8, true, true>(nkb * 128 * 128, 0, 3) <= kSmemMax;
             const int64_t c192w = w192 ? cost(192, true) : INT64_MAX, c128w = w128 ? cost(128, true) : INT64_MAX,
                           c192 = n192 ? cost(192, false) : INT64_MAX, c128 = cost(128, false);
             const int64_t best = std::min(std::min(c192w, c128w), std::min(c192, c128));
-            if (c192w == best) return run<192, 3, 1, true, true, false>(gp, ep, s);
+            if (c192w == best) return run<192, 6, 1, true, true, false>(gp, ep, s);
             if (c192 == best) return run<192, 4, 1, true, false, false>(gp, ep, s);
-            if (c128w == best) return run<128, 3, 1, true, true, false>(gp, ep, s);
+            if (c128w == best) return run<128, 6, 1, true, true, false>(gp, ep, s);
             return run<128, 5, 1, true, false, false>(gp, ep, s);
         }
         return run<128, 5, 1, true, false, false>(gp, ep, s);

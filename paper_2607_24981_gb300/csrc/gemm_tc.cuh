@@ -44,7 +44,7 @@ namespace ilw {
 // Host helpers of the tensor-core GEMM shared by its translation units (defined in gemm_tc.cu).
 bool gemm_make_map(CUtensorMap *m, const void *base, CUtensorMapDataType dt, int esize, int64_t rows, int64_t cols,
                    int64_t ld, int box_cols, int box_rows, CUtensorMapSwizzle sw);
-const int8_t *gemm_gelu_table(const GeluC &c, int32_t m_g, int32_t s_g, cudaStream_t s, cudaError_t *err);
+const uint8_t *gemm_gelu_table(const GeluC &c, int32_t m_g, int32_t s_g, cudaStream_t s, cudaError_t *err);
 // The wait bound of the next GEMM launches and the K block whose load the producer skips (-1: none),
 // as set by ilwdetr_debug_gemm_wait (defaults: about one second, none).
 void gemm_debug_wait(int32_t *skip, long long *cycles);
@@ -56,11 +56,9 @@ cudaError_t run_i8(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s);
 namespace {
 
 constexpr int BM = 128, BK = 64;
-constexpr int kThreads = 448;
 constexpr int kMaxSeg = 8;
 constexpr int kSegK = 1024;  // max K per accumulator for exact fp32 accumulation
 constexpr int kMaxWk = kSegK / 64;  // K blocks of resident weights (one barrier each)
-constexpr int kStageBytes = 1024;   // per epilogue warp: the 32 x 16 output box of the TMA store
 constexpr long long kWaitCycles = 2000000000ll;  // ~1 s at 2 GHz: the default bound of every wait
 
 struct Seg {
@@ -81,11 +79,14 @@ struct TcParams {  // CUtensorMap members keep the 64-byte alignment TMA needs
     int32_t nbuf;       // TMEM accumulator sets (1 or 2)
     int32_t wres_bytes; // resident weight bytes (WRES), a multiple of 1024
     int32_t tmem_cols;
-    int32_t tma_store;  // 1: outputs go out by TMA tensor stores of 32 x 16 boxes through shared memory
+    int32_t tma_store;  // boxes per epilogue warp (2 or 1) of the outputs' TMA stores through shared memory; 0: plain stores
     int32_t dbg_skip;   // test hook: the producer issues no load for this K-block counter value (-1: none)
     long long wait_cycles;  // the bound of every wait (about one second, shorter for the test hook)
     CUtensorMap cmap;   // C [M, N] with 16 x 32 boxes (2-byte outputs: 32-byte swizzle)
-    const int8_t *gelu_tab;  // SD-ShiftGELU output table in global memory (16-byte aligned, 65536 bytes)
+    CUtensorMap rmap;   // the int16 residual in 32 x 32 boxes (res_tma)
+    int32_t res_tma;    // 1: each epilogue warp loads its residual box by TMA and writes its results over it
+    int32_t stages;     // pipeline stages in use (STAGES at most)
+    const uint8_t *gelu_tab;  // SD-ShiftGELU output table in global memory (16-byte aligned, 65536 bytes)
     int *status;
     EpiParams ep;
 };
@@ -139,14 +140,23 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)map) : "memory");
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"((uint64_t)src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, int32_t x, int32_t y, uint32_t src) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"((uint64_t)map),
                  "r"(x), "r"(y), "r"(src)
                  : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
 __device__ __forceinline__ void fence_async_smem_g() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -168,14 +178,20 @@ __device__ __forceinline__ bool elect_lane() {
     asm volatile("{\n .reg .pred P;\n elect.sync _|P, 0xffffffff;\n selp.b32 %0, 1, 0, P;\n}\n" : "=r"(p));
     return p != 0;
 }
-__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+// One MMA / commit by the lanes with `issue` set (one of the warp): a predicate, not a branch, so that the
+// operands stay in uniform registers.
+__device__ __forceinline__ void tc_mma(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc, uint32_t issue) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(issue)
         : "memory");
 }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void tc_commit(uint32_t bar, uint32_t issue) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar), "r"(issue)
+        : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
@@ -243,6 +259,10 @@ struct Smem {
     static constexpr int kWtile = BN * 128;  // one K block of W
 };
 
+// Epilogue parameters in shared memory: four arrays of a column part, per warp or (WRES) per part.
+template <int BN, bool WRES>
+constexpr int prm_words() { return (WRES ? 4 : 16) * BN; }
+
 // Output kinds: one compact epilogue per kernel instantiation.
 // F16OUT: RQ8 values as fp16; GELU_F16: GELU8 values as fp16
 enum { KIND_RQ8 = 0, KIND_RQ16 = 1, KIND_RAW32 = 2, KIND_GELU8 = 3, KIND_F16OUT = 4, KIND_GELU_F16 = 5 };
@@ -258,6 +278,22 @@ __device__ __forceinline__ void lds16(const int32_t *p, int32_t (&o)[16]) {
                      : "r"(a + 16 * j));
 }
 
+__device__ __forceinline__ void lds8(const int32_t *p, int32_t (&o)[8]) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(o[4 * j]), "=r"(o[4 * j + 1]), "=r"(o[4 * j + 2]), "=r"(o[4 * j + 3])
+                     : "r"(a + 16 * j));
+}
+
+enum { FORM_GENERAL = 0, FORM_UNI = 1, FORM_VAR = 2, FORM_FLT = 3 };
+// rq(acc + bias; m, s) in 64 bits, clamped to +-2^30, which saturates the same.
+__device__ __forceinline__ int32_t rq_clamped(int32_t acc, int32_t bias, int32_t m, int32_t s) {
+    const int64_t t = rq((int64_t)acc + bias, m, s);
+    return (int32_t)(t < -(1 << 30) ? -(1 << 30) : (t > (1 << 30) ? (1 << 30) : t));
+}
+
 // The fused epilogue of 16 consecutive columns of one row, computed stage by stage so that the
 // 16 independent elements overlap.  FAST (uniform across the warp, decided per tile) says every
 // shift of the warp's columns is >= 33; ss then holds s - 32 and sr 2^(s-33) (rq_hi), else ss
@@ -266,7 +302,7 @@ template <int KIND, bool FAST, bool RFAST>
 __device__ __forceinline__ void epi_chunk(const EpiParams &ep, bool has_res, const uint32_t (&rp)[8],
                                           const int32_t (&acc)[16], const int32_t (&sb)[16],
                                           const int32_t (&sm)[16], const int32_t (&ss)[16],
-                                          const int32_t (&sr)[16], const int8_t *gtab, int32_t (&out)[16]) {
+                                          const int32_t (&sr)[16], const uint8_t *gtab, int32_t (&out)[16]) {
     if (KIND == KIND_RAW32) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) out[i] = acc[i] + sb[i];
@@ -279,14 +315,15 @@ __device__ __forceinline__ void epi_chunk(const EpiParams &ep, bool has_res, con
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
-            const int64_t t = rq((int64_t)acc[i] + sb[i], sm[i], ss[i]);
-            r[i] = (int32_t)(t < -(1 << 30) ? -(1 << 30) : (t > (1 << 30) ? (1 << 30) : t));  // saturates the same
+            r[i] = rq_clamped(acc[i], sb[i], sm[i], ss[i]);
         }
     }
     if (KIND == KIND_GELU8 || KIND == KIND_GELU_F16) {
         // g = sat16(r); the table holds sat8(rq(g * I_div(g); m_g, s_g)) for every int16 g
 #pragma unroll
-        for (int i = 0; i < 16; ++i) out[i] = gtab[clamp16(r[i])];
+        for (int i = 0; i < 16; ++i) {
+            out[i] = (int32_t)gtab[clamp16(r[i])] - 128;
+        }
         return;
     }
     if (has_res) {
@@ -302,100 +339,105 @@ __device__ __forceinline__ void epi_chunk(const EpiParams &ep, bool has_res, con
     for (int i = 0; i < 16; ++i) out[i] = (KIND == KIND_RQ8 || KIND == KIND_F16OUT) ? clamp8(r[i]) : clamp16(r[i]);
 }
 
-// Stores 16 epilogue outputs of one row (out[i] for columns c0 + i) at dst: 16-byte vector stores
-// when all 16 columns exist and dst is 16-byte aligned, else element by element (ncol columns).
+// Packed fp32 pairs (two operations an instruction).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pair2(uint32_t lo, uint32_t hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(f32x2 v) { return __uint_as_float((uint32_t)(v >> 32)); }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// max(m, |a|, |b|) in one instruction
+__device__ __forceinline__ float max_abs3(float m, float a, float b) {
+    asm("max.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(fabsf(a)), "f"(fabsf(b)));
+    return m;
+}
+constexpr uint32_t kMagic = 0x4B400000u;  // 1.5 2^23: adding it to a float rounds it to an integer (ties to even)
+__device__ __forceinline__ uint32_t half2_add(uint32_t a, uint32_t b) {
+    uint32_t r;
+    asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// 8 requantised values of a row, before saturation, as the words of the output type (two fp16 or int16, or
+// four int8, a word), w[0] on.  Saturating to [-127, 127] biased by 127 is one add-min-relu; the bias comes off with
+// a half2 subtract of 1151 from 1024 + u, or an add and an exclusive or per word (u + 1 never carries into
+// the next byte); two int16 are saturated and packed in one instruction, -32768 raised in another.
+// GELU kinds: sat16 indexes the table of values + 128 (gt points at the entry of -32767).
 template <int KIND>
-__device__ __forceinline__ void store16(char *dst, const int32_t (&out)[16], int ncol, bool vec) {
-    constexpr int bits = (KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16) ? 16 : (KIND == KIND_RAW32 ? 32 : 8);
-    if constexpr (KIND == KIND_F16OUT || KIND == KIND_GELU_F16) {
-        // |v| <= 127: the fp16 bits of 1152 + v are 0x6480 + v; one half2 subtract of 1152 leaves v exactly
-        const __half2 k1152 = __half2half2(__ushort_as_half((unsigned short)0x6480));
-        uint32_t hw[8];
+constexpr int out_words() { return KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16 ? 8 : 4; }
+template <int KIND>
+__device__ __forceinline__ void pack8(const int32_t (&r)[8], const uint8_t *gt, uint32_t *w) {
+    if constexpr (KIND == KIND_RQ16) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            uint32_t x = (uint32_t)(0x6480 + out[2 * j]) | ((uint32_t)(0x6480 + out[2 * j + 1]) << 16);
-            __half2 h = __hsub2(*reinterpret_cast<__half2 *>(&x), k1152);
-            hw[j] = *reinterpret_cast<uint32_t *>(&h);
+        for (int j = 0; j < 4; ++j)
+            asm("{.reg .b32 t;\n\tcvt.pack.sat.s16.s32 t, %1, %2;\n\tmax.s16x2 %0, t, %3;}"
+                : "=r"(w[j]) : "r"(r[2 * j + 1]), "r"(r[2 * j]), "r"(0x80018001u));
+    } else {
+        uint32_t u[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if constexpr (gelu_kind(KIND)) u[i] = gt[__viaddmin_s32_relu(r[i], 32767, 65534)];
+            else u[i] = (uint32_t)__viaddmin_s32_relu(r[i], 127, 254);
         }
-        if (vec) {
-            ((uint4 *)dst)[0] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-            ((uint4 *)dst)[1] = make_uint4(hw[4], hw[5], hw[6], hw[7]);
+        if constexpr (out_words<KIND>() == 8) {
+            // fp16 1024 + u, less 1151 (u biased by 127) or 1152 (the biased table)
+            constexpr uint32_t off = KIND == KIND_F16OUT ? 0xE47FE47Fu : 0xE480E480u;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[j] = half2_add(__byte_perm(u[2 * j], u[2 * j + 1], 0x5410) | 0x64006400u, off);
         } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i < ncol) ((uint16_t *)dst)[i] = (uint16_t)((i & 1) ? hw[i >> 1] >> 16 : hw[i >> 1]);
-        }
-    } else if constexpr (bits == 8) {
-        if (vec) {
-            uint32_t w[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                w[u] = (uint32_t)(uint8_t)out[4 * u] | ((uint32_t)(uint8_t)out[4 * u + 1] << 8) |
-                       ((uint32_t)(uint8_t)out[4 * u + 2] << 16) | ((uint32_t)(uint8_t)out[4 * u + 3] << 24);
-            *(uint4 *)dst = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i < ncol) ((int8_t *)dst)[i] = (int8_t)out[i];
-        }
-    } else if constexpr (bits == 16) {
-        if (vec) {
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                uint32_t w[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    w[u] = (uint32_t)(uint16_t)out[8 * j + 2 * u] | ((uint32_t)(uint16_t)out[8 * j + 2 * u + 1] << 16);
-                ((uint4 *)dst)[j] = make_uint4(w[0], w[1], w[2], w[3]);
+                const uint32_t x = __byte_perm(__byte_perm(u[4 * j], u[4 * j + 1], 0x0040),
+                                               __byte_perm(u[4 * j + 2], u[4 * j + 3], 0x0040), 0x5410);
+                w[j] = (KIND == KIND_RQ8 ? x + 0x01010101u : x) ^ 0x80808080u;
             }
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i < ncol) ((int16_t *)dst)[i] = (int16_t)out[i];
-        }
-    } else {
-        if (vec) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) ((int4 *)dst)[j] = make_int4(out[4 * j], out[4 * j + 1], out[4 * j + 2], out[4 * j + 3]);
-        } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i)
-                if (i < ncol) ((int32_t *)dst)[i] = out[i];
         }
     }
 }
-
-// 16 epilogue outputs of one row into row `lane` of the warp's 32 x 16 TMA-store box: 2-byte outputs
-// (fp16-carried int8, int16) as two 16-byte halves in the 32-byte swizzle the tensor map declares
-// (half j of row r at ((j ^ ((r >> 2) & 1)) << 4): no bank conflicts), 1-byte outputs as one 16-byte row.
+// The words stored at dst: 16-byte vector stores when vec (16 columns, 16-byte aligned), else element by
+// element (ncol columns).
 template <int KIND>
-__device__ __forceinline__ void box_row16(uint8_t *box, int lane, const int32_t (&out)[16]) {
-    if constexpr (KIND == KIND_F16OUT || KIND == KIND_GELU_F16) {
-        const __half2 k1152 = __half2half2(__ushort_as_half((unsigned short)0x6480));
-        uint32_t hw[8];
+__device__ __forceinline__ void store_words(char *dst, const uint32_t (&w)[out_words<KIND>()], int ncol, bool vec) {
+    constexpr int NW = out_words<KIND>();
+    if (vec) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            uint32_t x = (uint32_t)(0x6480 + out[2 * j]) | ((uint32_t)(0x6480 + out[2 * j + 1]) << 16);
-            __half2 h = __hsub2(*reinterpret_cast<__half2 *>(&x), k1152);
-            hw[j] = *reinterpret_cast<uint32_t *>(&h);
-        }
-        const int sw = (lane >> 2) & 1;
-        *(uint4 *)(box + lane * 32 + (sw << 4)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        *(uint4 *)(box + lane * 32 + ((sw ^ 1) << 4)) = make_uint4(hw[4], hw[5], hw[6], hw[7]);
-    } else if constexpr (KIND == KIND_RQ16) {
-        uint32_t w[8];
+        for (int j = 0; j < NW / 4; ++j) ((uint4 *)dst)[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+    } else if constexpr (NW == 8) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) w[j] = (uint32_t)(uint16_t)out[2 * j] | ((uint32_t)(uint16_t)out[2 * j + 1] << 16);
-        const int sw = (lane >> 2) & 1;
-        *(uint4 *)(box + lane * 32 + (sw << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-        *(uint4 *)(box + lane * 32 + ((sw ^ 1) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+        for (int i = 0; i < 16; ++i)
+            if (i < ncol) ((uint16_t *)dst)[i] = (uint16_t)((i & 1) ? w[i >> 1] >> 16 : w[i >> 1]);
     } else {
-        uint32_t w[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            w[u] = (uint32_t)(uint8_t)out[4 * u] | ((uint32_t)(uint8_t)out[4 * u + 1] << 8) |
-                   ((uint32_t)(uint8_t)out[4 * u + 2] << 16) | ((uint32_t)(uint8_t)out[4 * u + 3] << 24);
-        *(uint4 *)(box + lane * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+        for (int i = 0; i < 16; ++i)
+            if (i < ncol) ((uint8_t *)dst)[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+    }
+}
+// A warp's TMA-store box: its 32 rows x 32 columns.  Chunk `half` (0 or 1) of row `lane`: 2-byte outputs
+// (fp16-carried int8, int16) as two 16-byte units of a 64-byte row in the 64-byte swizzle the tensor map
+// declares (unit j of row r at j ^ ((r >> 1) & 3)), 1-byte outputs as one unit of a 32-byte row in the 32-byte
+// swizzle (j ^ ((r >> 2) & 1)): no bank conflicts.  (Boxes of 16 columns fence and store twice as often.)
+template <int KIND>
+constexpr int box_bytes() { return out_words<KIND>() == 8 ? 2048 : 1024; }
+template <int KIND>
+__device__ __forceinline__ void box_words(uint8_t *box, int lane, int half, const uint32_t (&w)[out_words<KIND>()]) {
+    if constexpr (out_words<KIND>() == 8) {
+        const int sw = (lane >> 1) & 3;
+        *(uint4 *)(box + lane * 64 + (((2 * half) ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *(uint4 *)(box + lane * 64 + (((2 * half + 1) ^ sw) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+    } else {
+        *(uint4 *)(box + lane * 32 + ((half ^ ((lane >> 2) & 1)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
 }
 
@@ -412,14 +454,33 @@ __device__ __forceinline__ void tmem_wait_all(uint32_t (&v)[NSEG][16]) {
 }
 
 // The epilogue of one warp's part of a tile (its 32 rows x HALF columns) in the common case: a
-// plain GEMM whose K is split into NSEG accumulators (compile-time), and one dyadic shift s >= 33
-// shared by all the part's columns (checked per tile by the caller), so rq(v; m, s) =
-// mad.hi(v, m, 2^(s-33)) >> (s - 32) with a scalar rounding constant and shift.  The part's
+// plain GEMM whose K is split into NSEG accumulators (compile-time), and requantisations that fit
+// 32 bits (the caller checks the part's columns).  FORM_UNI: one dyadic shift s >= 33 for all of them, so
+// rq(v; m, s) = mad.hi(v, m, 2^(s-33)) >> (s - 32) with a scalar rounding constant and shift.  FORM_VAR: every
+// s >= 29 and |bias| <= 2^26: with k = max(0, 33 - s), rq(v; m, s) = rq(v 2^k; m, s + k) and |v 2^k| < 2^31; the
+// four parameters are the bias times 2^k, 2^k, m and s + k - 33.  FORM_FLT: below.  The part's
 // accumulators are read from TMEM in 32-column groups (all of them at once for one segment), so the
 // accumulator set is released to the MMA warp after the first wait, and the requantisation of the
 // 16-column chunks that follows has no TMEM latency left in it.  RES: the two-term residual form
 // (s_r >= 17); rp holds the residual pairs of group 0 (fetched by the caller while the MMAs ran), and
-// each later group's pairs are fetched before its TMEM loads.
+// each later group's pairs are fetched before its TMEM loads.  RES = 1: in registers; RES = 2: the residual is in
+// the warp's box already (by TMA, read back as 16 bytes a lane), and the results replace it there.
+//
+// Bound by instructions (a scheduler owns BM BN / 128 outputs of a tile and has about as long for them as the
+// tile's MMAs take); so:
+// - Accumulators become integers with one packed add of 1.5 2^23, whose bits are read (float to integer is
+//   8 cycles a warp, this 1 a value), for groups whose accumulators are all within 2^22; others convert.
+// - int8 results without a residual (FORM_FLT, any shifts) are rounded in packed fp32: y = acc sc + b, sc = m 2^-s and
+//   b = bias m 2^-s rounded to float, rr = round(y), d = y - rr exactly.  For |acc sc + b| <= 127.5 and
+//   |b| <= 128 the float y is off by at most 256 2^-24 (sc) + 2^-17 (y) + 2^-18 (b) < 2^-15, and with two
+//   accumulators by their sum's 256 2^-24 more, < 2^-14; so while |d| <= 1/2 - that, rr is
+//   floor(y + 1/2) of the exact y (beyond 127.5 both saturate).  A chunk with any other value (about 3 and
+//   6 % of chunks on generic data) is computed again in 64-bit integers.  m 2^-s with fewer than 14 fractional bits
+//   would often meet 1/2 exactly, so the caller lets such columns take the integers at once.
+// Before (float-to-integer conversions, parameters per tile, 16-column boxes) and now, graph replays on
+// 12800 rows: 1152 x 384 to int8 in fp16 21.2 and 17.0 us (a 128 x 192 tile 5750 and 3300 clocks here),
+// 384 x 384 with residual 14.6 and 13.0, 1536 x 384 with SD-ShiftGELU 29.5 and 27.0; a 256-token block with
+// a shift of its own for every column (the 64-bit form then) 74 and 47.5 us.
 // The residual pairs (x[2j] | x[2j+1] << 16) of 32 columns of a row starting at rrow + c0 (columns
 // at or past ncol read as 0; rvec: 16-byte aligned and all 32 present).
 __device__ __forceinline__ void res_group(const int16_t *rrow, int c0, int ncol, bool rvec, uint32_t (&rp)[16]) {
@@ -440,25 +501,27 @@ __device__ __forceinline__ void res_group(const int16_t *rrow, int c0, int ncol,
     }
 }
 
-// box: this warp's TMA-store box (nullptr: plain stores at dst), written out at column x0 + 16 c, row
-// y0 of cmap by lane 0 once every lane has written its row; the box is rewritten only after the
-// previous store has read it (that wait comes after the next chunk's arithmetic).
-template <int KIND, int BN, int HALF, int NSEG, bool RES>
+// box: this warp's one or two TMA-store boxes (nullptr: plain stores at dst), written out at column
+// x0 + 32 g, row y0 of cmap by lane 0 once every lane has written its row.
+template <int KIND, int BN, int HALF, int NSEG, int RES, int FORM>
 __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, const int32_t *s_bias,
-                                         const int32_t *s_mult, int32_t rnd, int32_t sh, uint32_t (&rp)[16],
+                                         const int32_t *s_mult, const int32_t *s_a, const int32_t *s_b, int n0,
+                                         int ncol_all,
+                                         int32_t rnd, int32_t sh, uint32_t (&rp)[16],
                                          const int16_t *rrow, bool rvec, char *dst, int ncol_row, bool vec_ok,
-                                         const int8_t *gt, uint32_t empty_bar, int lane, uint8_t *box,
+                                         const uint8_t *gt, uint32_t empty_bar, int lane, uint8_t *box, int boxes,
                                          const CUtensorMap *cmap, int x0, int y0) {
     static_assert(HALF % 32 == 0, "32-column groups");
     constexpr int NG = HALF / 32;                    // 32-column groups of the part
-    // groups read per TMEM pass (32 registers per group and segment): the whole part for one segment
-    // without a residual, one group otherwise (the residual's pairs take 32 registers)
-    constexpr int GPASS = (NSEG == 1 && !RES) ? NG : 1;
+    // groups read per TMEM pass (32 registers per group and segment): a part of 64 columns at once for one
+    // segment without a residual, else one group (three at once spill, and so do the residual's pairs)
+    constexpr int GPASS = (NSEG == 1 && RES == 0 && NG <= 2) ? NG : 1;
+    static_assert(RES != 2 || (NG == 1 && KIND == KIND_RQ16), "one box holds the residual and the results");
     constexpr int esz = (KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16) ? 2 : (KIND == KIND_RAW32 ? 4 : 1);
-    const int32_t r_rnd = RES ? 1 << (ep.s_r - 17) : 0, r_sh = RES ? ep.s_r - 16 : 0;
+    const int32_t r_rnd = RES != 0 ? 1 << (ep.s_r - 17) : 0, r_sh = RES != 0 ? ep.s_r - 16 : 0;
 #pragma unroll
     for (int g0 = 0; g0 < NG; g0 += GPASS) {
-        if constexpr (RES) {  // this group's residual pairs (group 0's came with the call), in flight during the TMEM wait
+        if constexpr (RES == 1) {  // this group's residual pairs (group 0's came with the call), in flight during the TMEM wait
             if (g0 > 0) res_group(rrow, 32 * g0, ncol_row, rvec, rp);
         }
         uint32_t v[NSEG][GPASS * 32];
@@ -476,67 +539,203 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
             __syncwarp();
             if (lane == 0) mbar_arrive(empty_bar);
         }
-        // the integer accumulators (exact: every partial sum is below 2^24), in place
-#pragma unroll
-        for (int i = 0; i < GPASS * 32; ++i) {
-            int32_t a = __float2int_rn(__uint_as_float(v[0][i]));
-#pragma unroll
-            for (int sg = 1; sg < NSEG; ++sg) a += __float2int_rn(__uint_as_float(v[sg][i]));
-            v[0][i] = (uint32_t)a;
-        }
-#pragma unroll
-        for (int cc = 0; cc < GPASS * 2; ++cc) {
-            const int c = 2 * g0 + cc;  // 16-column chunk of the part
-            int32_t cb[16], cm[16];
-            lds16(s_bias + 16 * c, cb);
-            lds16(s_mult + 16 * c, cm);
-            int32_t out[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                int32_t r = rq_hi((int32_t)v[0][16 * cc + i] + cb[i], cm[i], rnd, sh);  // |r| < 2^29
-                if constexpr (KIND == KIND_GELU8 || KIND == KIND_GELU_F16) {
-                    out[i] = gt[clamp16(r)];
-                } else {
-                    if constexpr (RES) {
-                        const uint32_t w = rp[8 * cc + (i >> 1)];
-                        const int32_t xs = (i & 1) ? (int32_t)(w & 0xFFFF0000u) : (int32_t)(w << 16);
-                        r += rq_hi(xs, ep.m_r, r_rnd, r_sh);
-                    }
-                    out[i] = (KIND == KIND_RQ8 || KIND == KIND_F16OUT) ? clamp8(r) : clamp16(r);
-                }
-            }
+        // 16 columns out: the chunk's words
+        auto emit = [&](int c, const uint32_t (&w)[out_words<KIND>()]) {
             if (box) {
-                if (lane == 0) tma_store_wait_read();  // the previous chunk's box has been read
-                __syncwarp();
-                box_row16<KIND>(box, lane, out);
-                fence_async_smem_g();
-                __syncwarp();
-                if (lane == 0 && 16 * c < ncol_row) tma_store_2d(cmap, x0 + 16 * c, y0, smem_u32(box));
+                // chunks 2 g and 2 g + 1 share a box; the store before the last one has read it (every
+                // group of columns commits, so that the count holds where columns past N store nothing)
+                uint8_t *bx = box + (boxes == 2 ? ((c >> 1) & 1) * box_bytes<KIND>() : 0);
+                if ((c & 1) == 0) {
+                    if (lane == 0) {
+                        if (boxes == 2) tma_store_wait_read1();
+                        else tma_store_wait_read();
+                    }
+                    __syncwarp();
+                }
+                box_words<KIND>(bx, lane, c & 1, w);
+                if (c & 1) {
+                    fence_async_smem_g();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (16 * (c - 1) < ncol_row) tma_store_2d(cmap, x0 + 16 * (c - 1), y0, smem_u32(bx));
+                        tma_store_commit();
+                    }
+                }
             } else if (dst) {
                 const int ncol = ncol_row - 16 * c;
-                if (ncol > 0) store16<KIND>(dst + 16 * c * esz, out, ncol, vec_ok && ncol >= 16);
+                if (ncol > 0) store_words<KIND>(dst + 16 * c * esz, w, ncol, vec_ok && ncol >= 16);
+            }
+        };
+        if constexpr (FORM == FORM_FLT) {
+            const f32x2 magic = pair2(kMagic, kMagic), nmagic = pair2(kMagic | 0x80000000u, kMagic | 0x80000000u);
+#pragma unroll
+            for (int cc = 0; cc < GPASS * 2; ++cc) {
+                const int c = 2 * g0 + cc;  // 16-column chunk of the part
+                int32_t sc[16], bf[16];
+                lds16(s_a + 16 * c, sc);
+                lds16(s_b + 16 * c, bf);
+                uint32_t w[out_words<KIND>()], hw[8];
+                float dmax = 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int i = 16 * cc + 2 * j;
+                    f32x2 acc = pair2(v[0][i], v[0][i + 1]);
+#pragma unroll
+                    for (int sg = 1; sg < NSEG; ++sg) acc = add2(acc, pair2(v[sg][i], v[sg][i + 1]));
+                    const f32x2 y = fma2(acc, pair2(sc[2 * j], sc[2 * j + 1]), pair2(bf[2 * j], bf[2 * j + 1]));
+                    const f32x2 rr = add2(add2(y, magic), nmagic);
+                    const f32x2 d = add2(y, rr ^ 0x8000000080000000ull);
+                    dmax = max_abs3(dmax, lo2(d), hi2(d));
+                    asm("{.reg .b32 t;\n\tcvt.rn.f16x2.f32 t, %1, %2;\n\tmin.f16x2 t, t, %3;\n\tmax.f16x2 %0, t, %4;}"
+                        : "=r"(hw[j]) : "f"(hi2(rr)), "f"(lo2(rr)), "r"(0x57F057F0u), "r"(0xD7F0D7F0u));  // 127, -127
+                }
+                if constexpr (KIND == KIND_F16OUT) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) w[j] = hw[j];
+                } else {  // the low byte of the fp16 bits of 1152 + v is 128 + v
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        w[j] = __byte_perm(half2_add(hw[2 * j], 0x64806480u), half2_add(hw[2 * j + 1], 0x64806480u), 0x6420) ^
+                               0x80808080u;
+                }
+                if (__any_sync(0xffffffffu, !(dmax <= 0.5f - (NSEG == 1 ? 0x1p-15f : 0x1p-14f)))) {
+#pragma unroll
+                    for (int e = 0; e < 16; e += 8) {
+                        int32_t cb[8], cm[8], r[8];
+                        lds8(s_bias + 16 * c + e, cb);
+                        lds8(s_mult + 16 * c + e, cm);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            r[i] = __float2int_rn(__uint_as_float(v[0][16 * cc + e + i]));
+#pragma unroll
+                            for (int sg = 1; sg < NSEG; ++sg) r[i] += __float2int_rn(__uint_as_float(v[sg][16 * cc + e + i]));
+                        }
+                        if (rnd) {  // one shift >= 33
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) r[i] = rq_hi(r[i] + cb[i], cm[i], rnd, sh);
+                        } else {
+                            const int col = n0 + 16 * c + e;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) r[i] = rq_clamped(r[i], cb[i], cm[i], col + i < ncol_all ? __ldg(ep.shift + col + i) : 33);
+                        }
+                        pack8<KIND>(r, gt, w + e * out_words<KIND>() / 16);
+                    }
+                }
+                emit(c, w);
+            }
+        } else {
+            // the integer accumulators (exact: every partial sum is below 2^24) plus kMagic per segment, in place
+            float amax = 0.f;
+#pragma unroll
+            for (int sg = 0; sg < NSEG; ++sg)
+#pragma unroll
+                for (int i = 0; i < GPASS * 32; i += 2)
+                    amax = max_abs3(amax, __uint_as_float(v[sg][i]), __uint_as_float(v[sg][i + 1]));
+            const bool wide = __any_sync(0xffffffffu, amax > 4194304.f);
+            if (wide) {
+#pragma unroll
+                for (int i = 0; i < GPASS * 32; ++i) {
+                    uint32_t a = (uint32_t)NSEG * kMagic;
+#pragma unroll
+                    for (int sg = 0; sg < NSEG; ++sg) a += (uint32_t)__float2int_rn(__uint_as_float(v[sg][i]));
+                    v[0][i] = a;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < GPASS * 32; i += 2) {
+                    f32x2 t = add2(pair2(v[0][i], v[0][i + 1]), pair2(kMagic, kMagic));
+                    v[0][i] = (uint32_t)t;
+                    v[0][i + 1] = (uint32_t)(t >> 32);
+#pragma unroll
+                    for (int sg = 1; sg < NSEG; ++sg) {
+                        t = add2(pair2(v[sg][i], v[sg][i + 1]), pair2(kMagic, kMagic));
+                        v[0][i] += (uint32_t)t;
+                        v[0][i + 1] += (uint32_t)(t >> 32);
+                    }
+                }
+            }
+#pragma unroll
+            for (int cc = 0; cc < GPASS * 2; ++cc) {
+                const int c = 2 * g0 + cc;
+                uint32_t w[out_words<KIND>()];
+#pragma unroll
+                for (int e = 0; e < 16; e += 8) {
+                    int32_t cb[8], cm[8], r[8];
+                    lds8(s_bias + 16 * c + e, cb);  // less the magic numbers
+                    lds8(s_mult + 16 * c + e, cm);
+                    uint4 *unit = nullptr;
+                    uint32_t xr[4];
+                    if constexpr (RES == 2) {  // this lane's 8 residuals, in the box its results go to
+                        unit = (uint4 *)(box + lane * 64 + (((2 * (c & 1) + e / 8) ^ ((lane >> 1) & 3)) << 4));
+                        const uint4 x4 = *unit;
+                        xr[0] = x4.x; xr[1] = x4.y; xr[2] = x4.z; xr[3] = x4.w;
+                    }
+                    if constexpr (FORM == FORM_UNI) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            r[i] = rq_hi((int32_t)(v[0][16 * cc + e + i] + (uint32_t)cb[i]), cm[i], rnd, sh);  // |r| < 2^29
+                    } else {
+                        int32_t ck[8], cs[8];
+                        lds8(s_a + 16 * c + e, ck);
+                        lds8(s_b + 16 * c + e, cs);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            r[i] = rq_hi1((int32_t)(v[0][16 * cc + e + i] * (uint32_t)ck[i] + (uint32_t)cb[i]), cm[i], cs[i]);
+                    }
+                    if constexpr (RES != 0) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const uint32_t x = RES == 1 ? rp[8 * cc + (e + i) / 2] : xr[i / 2];
+                            const int32_t xs = (i & 1) ? (int32_t)(x & 0xFFFF0000u) : (int32_t)(x << 16);
+                            r[i] += rq_hi(xs, ep.m_r, r_rnd, r_sh);
+                        }
+                    }
+                    pack8<KIND>(r, gt, w + e * out_words<KIND>() / 16);
+                    if constexpr (RES == 2) *unit = make_uint4(w[e / 2], w[e / 2 + 1], w[e / 2 + 2], w[e / 2 + 3]);
+                }
+                if constexpr (RES != 2) emit(c, w);
+            }
+            if constexpr (RES == 2) {
+                fence_async_smem_g();
+                __syncwarp();
+                if (lane == 0) {
+                    if (ncol_row > 0) tma_store_2d(cmap, x0, y0, smem_u32(box));
+                    tma_store_commit();
+                }
             }
         }
         __syncwarp();  // reconverge before the next warp-synchronous tcgen05 instruction
     }
 }
 
+// Epilogue warps: column parts per TMEM lane quarter.  int8 A: two parts next to the four converter warps;
+// fp16 A needs no converters, and 128-wide tiles take four parts of 32 columns (a warp's whole residual is
+// in registers before the accumulators are ready, and 16 warps hide the chains of their loads; with two
+// parts the epilogue of a projection tile took 4900 clocks), 192-wide tiles three of 64.
+template <int BN, bool AF16>
+constexpr int epi_parts() { return AF16 ? (BN == 192 ? 3 : 4) : 2; }
+template <int BN, bool AF16>
+constexpr int epi_warps() { return 4 * epi_parts<BN, AF16>(); }
+template <int BN, bool AF16>
+constexpr int tc_threads() { return 32 * ((AF16 ? 2 : 6) + epi_warps<BN, AF16>()); }
+
+template <int V>
+using Int = std::integral_constant<int, V>;
+
 template <int BN, int STAGES, int KIND, int NB, bool AF16, bool WRES>
-__global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_constant__ TcParams<NB> p) {
+__global__ void __launch_bounds__(tc_threads<BN, AF16>(), 1) gemm_tc_kernel(const __grid_constant__ TcParams<NB> p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     using SM = Smem<BN, AF16, WRES>;
     constexpr int kStage = SM::kStage;
-    // Epilogue warps: 8 (warps 6-13, two column parts per TMEM lane quarter), or, when A arrives in
-    // fp16 and the tile is 192 wide, the converters' warps too: 12 (warps 2-13, three parts of 64).
-    constexpr int NP = (AF16 && BN == 192) ? 3 : 2;
-    constexpr int EPI0 = NP == 3 ? 2 : 6;
+    constexpr int NP = epi_parts<BN, AF16>(), EPI0 = AF16 ? 2 : 6;  // column parts, first epilogue warp
     constexpr int NWE = 4 * NP;
-    uint8_t *wres = smem + STAGES * kStage;  // resident weights (WRES)
+    const int nst = WRES ? p.stages : STAGES;  // pipeline stages
+    uint8_t *wres = smem + nst * kStage;  // resident weights (WRES)
     uint64_t *bars = (uint64_t *)(wres + (WRES ? p.wres_bytes : 0));
     // barriers: full[S], a_ready[S], empty[S], acc_full[2], acc_empty[2], wfull[kMaxWk] (one per K block
     // of the resident weights, so the first MMAs start as soon as their own block has landed)
-    uint32_t *tmem_slot = (uint32_t *)(bars + 3 * STAGES + 5 + kMaxWk);
+    uint32_t *tmem_slot = (uint32_t *)(bars + 3 * STAGES + 6 + kMaxWk + NWE);
     volatile int *abort = (volatile int *)(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -548,19 +747,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     auto acc_empty = [&](int b) { return bar0 + 8u * (3 * STAGES + 2 + b); };
     auto wfull = [&](int kk) { return bar0 + 8u * (3 * STAGES + 4 + kk); };
     const uint32_t drain = bar0 + 8u * (3 * STAGES + 4 + kMaxWk);  // every MMA issued has completed
+    const uint32_t tab_full = drain + 8u;                          // the GELU table has arrived
+    auto res_full = [&](int w) { return tab_full + 8u * (1 + w); };  // an epilogue warp's residual box
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full(s), 1);
-            mbar_init(a_ready(s), 4);
-            mbar_init(empty(s), 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(acc_full(b), 1);
-            mbar_init(acc_empty(b), NWE);
-        }
-        for (int kk = 0; kk < kMaxWk; ++kk) mbar_init(wfull(kk), 1);
-        mbar_init(drain, 1);
+    // one barrier a lane: full[S], a_ready[S] (the converter warps), empty[S], acc_full[2], acc_empty[2]
+    // (the epilogue warps), wfull, drain, tab_full, res_full
+    constexpr int kBars = 3 * STAGES + 6 + kMaxWk + NWE;
+    if (warp == 1) {
+        for (int i = lane; i < kBars; i += 32)
+            mbar_init(bar0 + 8u * i, i >= STAGES && i < 2 * STAGES ? 4 : (i == 3 * STAGES + 2 || i == 3 * STAGES + 3 ? NWE : 1));
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -570,44 +765,53 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (threadIdx.x < NB) {  // the descriptors, ahead of the first loads
+        prefetch_map(&p.amap[threadIdx.x]);
+        prefetch_map(&p.wmap[threadIdx.x]);
+    }
+    if (threadIdx.x == 32 && p.tma_store) prefetch_map(&p.cmap);
+    if (threadIdx.x == 64 && p.res_tma) prefetch_map(&p.rmap);
     grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // the epilogue warps' copies of the tile's per-column parameters: one per warp, or with resident weights,
+    // where a CTA's columns never change, one per column part (its warps write the same values)
+    int32_t *prm = (int32_t *)(((uintptr_t)(tmem_slot + 4) + 15) & ~(uintptr_t)15);
     // SD-ShiftGELU and its output requantisation depend on the int16 value g alone: the table of
-    // sat8(rq(g * I_div(g); m_g, s_g)) (built once per parameter set by gelu_table_kernel) is
-    // copied into shared memory here.
-    int8_t *gtab = (int8_t *)((int32_t *)(((uintptr_t)(tmem_slot + 4) + 15) & ~(uintptr_t)15) + 16 * BN);
-    if ((KIND == KIND_GELU8 || KIND == KIND_GELU_F16) && warp >= EPI0) {
-        for (int i = threadIdx.x - 32 * EPI0; i < 65536 / 16; i += 32 * NWE)
-            ((uint4 *)gtab)[i] = __ldg((const uint4 *)p.gelu_tab + i);
-        asm volatile("bar.sync 1, %0;" ::"r"(32 * NWE) : "memory");  // the epilogue warps only
-    }
+    // sat8(rq(g * I_div(g); m_g, s_g)) + 128 (built once per parameter set by gelu_table_kernel) is copied
+    // into shared memory by the producer (one bulk copy behind the first operands; 12 warps copying it
+    // themselves held the first tile's epilogue up by 2000 clocks).
+    uint8_t *gtab = (uint8_t *)(prm + prm_words<BN, WRES>());
     const int acc_cols = p.nseg * BN;  // columns of one accumulator set
-    // the epilogue warps' TMA-store boxes (1024-byte aligned, after the parameters and the GELU table)
+    // the TMA-store boxes (1024-byte aligned, after the parameters and the GELU table)
     uint8_t *stg = (uint8_t *)(((uintptr_t)gtab + (gelu_kind(KIND) ? 65536 : 0) + 1023) & ~(uintptr_t)1023);
 
     if (warp == 0) {
         // ---------------------------------------------------------------- TMA producer
         if (lane == 0) {
-            int it = 0;  // global K-block counter (ring position)
+            int it = 0, s = 0;  // K blocks issued, ring position
+            uint32_t ph = 0;
             int wk = 0;  // K blocks of the resident weights issued
-            bool ok = true;
+            bool ok = true, tab = gelu_kind(KIND);
+            auto load_tab = [&]() {
+                mbar_expect_tx(tab_full, 65536);
+                bulk_load(smem_u32(gtab), p.gelu_tab, 65536, tab_full);
+                tab = false;
+            };
             for (int t = blockIdx.x; t < p.tiles && ok; t += gridDim.x) {
                 const int m0 = (t / p.tiles_n) * BM, n0 = (t % p.tiles_n) * BN;
                 for (int sg = 0; sg < p.nseg && ok; ++sg) {
                     const Seg &S = p.seg[sg];
                     const int nk = (S.klen + BK - 1) / BK;
                     for (int kk = 0; kk < nk; ++kk, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1;
-                        if (WRES && t == (int)blockIdx.x && kk < STAGES) {
+                        if (WRES && t == (int)blockIdx.x && kk < nst) {
                             // the CTA's BN rows of W, resident for all of its tiles (the grid is a
                             // multiple of tiles_n, so every tile of the CTA has the same n block): the
                             // first K blocks travel with the first tile's activations of the same K block,
                             // the rest follow at once (they have shared memory of their own)
-                            const int last = kk == (STAGES < nk ? STAGES : nk) - 1 ? nk - 1 : kk;
+                            const int last = kk == (nst < nk ? nst : nk) - 1 ? nk - 1 : kk;
                             for (int j = kk; j <= last; ++j) {
                                 mbar_expect_tx(wfull(j), (uint32_t)SM::kWtile);
                                 tma_load_2d(smem_u32(wres + j * SM::kWtile), &p.wmap[0], p.seg[0].k0 + j * BK, n0,
@@ -615,26 +819,35 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                             }
                             wk = last + 1;
                         }
+                        if (it == nst && tab) load_tab();  // behind the first stages, which wait for nothing
                         if (!mbar_wait(empty(s), ph ^ 1, abort, p.status, kStatusTimeoutFree, p.wait_cycles)) {
                             ok = false;
                             break;
                         }
                         uint8_t *st = smem + s * kStage;
+                        const uint32_t fb = full(s);
+                        if (++s == nst) {
+                            s = 0;
+                            ph ^= 1u;
+                        }
                         if (it == p.dbg_skip) continue;  // test hook: this stage's barrier never completes
-                        mbar_expect_tx(full(s), (AF16 ? SM::kA16 : SM::kA8) + SM::kW);
+                        mbar_expect_tx(fb, (AF16 ? SM::kA16 : SM::kA8) + SM::kW);
                         tma_load_2d(smem_u32(AF16 ? st : st + SM::kA16 + SM::kW), &p.amap[S.map], S.k0 + kk * BK, m0,
-                                    full(s));
-                        if (!WRES) tma_load_2d(smem_u32(st + SM::kA16), &p.wmap[S.map], S.k0 + kk * BK, n0, full(s));
+                                    fb);
+                        if (!WRES) tma_load_2d(smem_u32(st + SM::kA16), &p.wmap[S.map], S.k0 + kk * BK, n0, fb);
                     }
                 }
             }
+            if (tab) load_tab();  // fewer K blocks than stages
             if (!ok || *abort) {  // drain the loads still in flight (bounded) before the CTA can exit
                 long long t0 = clock64();
+                while (gelu_kind(KIND) && !mbar_try(tab_full, 0) && clock64() - t0 < p.wait_cycles) {
+                }
                 for (int kk = 0; kk < wk; ++kk)
                     while (!mbar_try(wfull(kk), 0) && clock64() - t0 < p.wait_cycles) {
                     }
-                for (int j = (it > STAGES ? it - STAGES : 0); j < it; ++j)
-                    while (j != p.dbg_skip && !mbar_try(full(j % STAGES), (j / STAGES) & 1) &&
+                for (int j = (it > nst ? it - nst : 0); j < it; ++j)
+                    while (j != p.dbg_skip && !mbar_try(full(j % nst), (j / nst) & 1) &&
                            clock64() - t0 < p.wait_cycles) {
                     }
             }
@@ -646,7 +859,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         // needs 113 clocks per MMA, above the 64 (N = 128) and 96 (N = 192) the MMA itself takes; this
         // form needs 60 and 86.
         {
-            const bool issue = elect_lane();
+            const uint32_t issue = elect_lane() ? 1u : 0u;
             auto wait = [&](uint32_t bar, uint32_t parity, int code) -> bool {
                 return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort, p.status, code, p.wait_cycles));
             };
@@ -673,25 +886,22 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                         tc_fence_after();
                         const uint64_t da = a_desc0 + (uint64_t)((s * kStage) >> 4);
                         const uint64_t dw = WRES ? w_desc0 + (uint64_t)((kk * SM::kWtile) >> 4) : da + (uint64_t)(SM::kA16 >> 4);
-                        if (issue) {
 #pragma unroll
-                            for (int k16 = 0; k16 < BK / 16; ++k16)
-                                tc_mma(dt, da + 2 * k16, dw + 2 * k16, idesc, (kk > 0 || k16 > 0) ? 1u : 0u);
-                            tc_commit(empty(s));
-                        }
-                        __syncwarp();
-                        if (++s == STAGES) {
+                        for (int k16 = 0; k16 < BK / 16; ++k16)
+                            tc_mma(dt, da + 2 * k16, dw + 2 * k16, idesc, (kk > 0 || k16 > 0) ? 1u : 0u, issue);
+                        tc_commit(empty(s), issue);
+                        if (++s == nst) {
                             s = 0;
                             ph ^= 1u;
                         }
                     }
                 }
-                if (issue) tc_commit(acc_full(b));  // arrives once every MMA of this tile has completed
+                tc_commit(acc_full(b), issue);  // arrives once every MMA of this tile has completed
                 __syncwarp();
             }
             // every MMA issued has completed before the CTA can reach the TMEM release (also after an
             // abort, when the epilogue no longer waits for the accumulators)
-            if (issue) tc_commit(drain);
+            tc_commit(drain, issue);
             const long long t0 = clock64();
             while (!mbar_try(drain, 0) && clock64() - t0 < p.wait_cycles) {
             }
@@ -738,98 +948,156 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         constexpr int HALF = BN / NP;  // columns of this warp in a tile
         const int q = warp & 3, h = (warp - EPI0) >> 2;
         const EpiParams &ep = p.ep;
-        int32_t *s_bias = (int32_t *)(((uintptr_t)(tmem_slot + 4) + 15) & ~(uintptr_t)15) + (warp - EPI0) * 4 * HALF;  // this warp's copy of
-        int32_t *s_mult = s_bias + HALF;                                       // the tile's per-column
-        int32_t *s_shift = s_mult + HALF;                                      // epilogue parameters
-        int32_t *s_rnd = s_shift + HALF;                                       // (rq_hi rounding constants)
+        int32_t *s_bias = prm + (WRES ? h : warp - EPI0) * 4 * HALF, *s_mult = s_bias + HALF;
+        int32_t *s_shift = s_mult + HALF, *s_rnd = s_shift + HALF;  // (or what epi_fast reads there)
         constexpr int bits = (KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16) ? 16
                              : (KIND == KIND_RAW32 ? 32 : 8);
         constexpr int PPL = HALF / 32;  // parameters per lane and per array
         constexpr bool kFastKind = KIND == KIND_RQ8 || KIND == KIND_RQ16 || KIND == KIND_F16OUT || gelu_kind(KIND);
         constexpr bool kResKind = KIND == KIND_RQ8 || KIND == KIND_RQ16;  // kinds with a residual
-        // The next tile's parameters are fetched into registers while the current tile is processed.
-        int32_t pb[PPL], pm[PPL], ps[PPL];
-        auto fetch = [&](int t) {
-            const int nn = (t % p.tiles_n) * BN + h * HALF;
+        const int nseg = p.nseg, nld = (HALF / 16) * nseg;  // TMEM loads per tile
+        const bool has_res = ep.res != nullptr, rfast = has_res && ep.s_r >= 17;
+        bool fastw = false, one_shift = false;  // every shift >= 33; and the same
+        int form = FORM_GENERAL;
+        int32_t s_0 = 0;
+        // The parameters of this warp's columns into shared memory, and the form they allow.  The launch
+        // makes the grid a multiple of the column tiles where it can, so that a CTA stays in its columns
+        // and this runs once (per tile it took 1700 of 5800 clocks).
+        auto params = [&](int n0) {
+            int32_t pb[PPL], pm[PPL], ps[PPL];
+            bool ok[PPL];
 #pragma unroll
             for (int k = 0; k < PPL; ++k) {
-                const int col = nn + lane + 32 * k;
-                const bool ok = col < p.N;
-                pb[k] = (ok && ep.bias) ? __ldg(ep.bias + col) : 0;
-                pm[k] = (ok && ep.mult) ? __ldg(ep.mult + col) : 0;
-                ps[k] = (ok && ep.shift) ? __ldg(ep.shift + col) : 33;
+                const int col = n0 + lane + 32 * k;
+                ok[k] = col < p.N;
+                pb[k] = (ok[k] && ep.bias) ? __ldg(ep.bias + col) : 0;
+                pm[k] = (ok[k] && ep.mult) ? __ldg(ep.mult + col) : 0;
+                ps[k] = (ok[k] && ep.shift) ? __ldg(ep.shift + col) : 33;
             }
-        };
-        if (blockIdx.x < p.tiles) fetch(blockIdx.x);
-        const int nseg = p.nseg, nld = (HALF / 16) * nseg;  // TMEM loads per tile
-        int tl = 0;
-        for (int t = blockIdx.x; t < p.tiles; t += gridDim.x, ++tl) {
-            const int b = tl % p.nbuf;
-            const uint32_t use = (uint32_t)(tl / p.nbuf);
-            const int m0 = (t / p.tiles_n) * BM, n0 = (t % p.tiles_n) * BN + h * HALF;
-            __syncwarp();  // this warp is done with the previous tile's parameters
-            bool fast_lane = true, same_lane = true;
-            const int32_t s_0 = __shfl_sync(0xffffffffu, ps[0], 0);
+            bool fast_lane = true, same_lane = true, var_lane = true, flt_lane = true;
+            s_0 = __shfl_sync(0xffffffffu, ps[0], 0);
+            // epi_fast with int8 results in packed fp32: m 2^-s and bias m 2^-s as floats
+            constexpr bool kFltKind = KIND == KIND_RQ8 || KIND == KIND_F16OUT;
+            float fsc[PPL], fbi[PPL];
 #pragma unroll
             for (int k = 0; k < PPL; ++k) {
                 fast_lane &= ps[k] >= 33;
-                same_lane &= ps[k] == s_0;
+                same_lane &= ps[k] == s_0 || !ok[k];
+                var_lane &= ps[k] >= 29 && pb[k] >= -(1 << 26) && pb[k] <= (1 << 26);
+                if constexpr (kFltKind) {
+                    const float two_s = __int_as_float((127 - max(1, min(ps[k], 100))) << 23);
+                    fsc[k] = __int2float_rn(pm[k]) * two_s;
+                    fbi[k] = __ll2float_rn((int64_t)pb[k] * pm[k]) * two_s;
+                    flt_lane &= ps[k] >= 1 && ps[k] <= 100 && fabsf(fbi[k]) <= 128.f && (pm[k] == 0 || ps[k] - (__ffs(pm[k]) - 1) >= 14);
+                }
             }
-            const bool fastw = __all_sync(0xffffffffu, fast_lane);  // shifts stored as s - 32 if so
-            // the common case (epi_fast): one shift >= 33 for all of this warp's columns, 1 or 2 segments
-            const bool ush = kFastKind && NB == 1 && !p.branch_rq && p.nseg <= 2 && fastw &&
-                             __all_sync(0xffffffffu, same_lane);
+            fastw = __all_sync(0xffffffffu, fast_lane);  // shifts stored as s - 32 if so
+            one_shift = fastw && __all_sync(0xffffffffu, same_lane);
+            form = FORM_GENERAL;
+            if (kFastKind && NB == 1 && !p.branch_rq && p.nseg <= 2 && (!has_res || rfast)) {
+                if (kFltKind && !has_res && __all_sync(0xffffffffu, flt_lane)) form = FORM_FLT;
+                else if (one_shift) form = FORM_UNI;
+                else if (p.nseg == 1 && __all_sync(0xffffffffu, var_lane)) form = FORM_VAR;
+            }
+            __syncwarp();  // this warp is done with the parameters before
 #pragma unroll
             for (int k = 0; k < PPL; ++k) {
-                s_bias[lane + 32 * k] = pb[k];
+                int32_t b = pb[k], sa = fastw ? ps[k] - 32 : ps[k], sb = fastw ? 1 << (ps[k] - 33) : 0;
+                const uint32_t off = (uint32_t)p.nseg * kMagic;  // of epi_fast's integers
+                if (form == FORM_UNI) b = (int32_t)((uint32_t)b - off);
+                if (form == FORM_VAR) {
+                    const int kk = max(0, 33 - ps[k]);
+                    b = (int32_t)(((uint32_t)b - off) << kk);
+                    sa = 1 << kk;
+                    sb = max(ps[k], 33) - 33;
+                }
+                if (kFltKind && form == FORM_FLT) {
+                    sa = __float_as_int(fsc[k]);
+                    sb = __float_as_int(fbi[k]);
+                }
+                s_bias[lane + 32 * k] = b;
                 s_mult[lane + 32 * k] = pm[k];
-                s_shift[lane + 32 * k] = fastw ? ps[k] - 32 : ps[k];
-                s_rnd[lane + 32 * k] = fastw ? 1 << (ps[k] - 33) : 0;
+                s_shift[lane + 32 * k] = sa;
+                s_rnd[lane + 32 * k] = sb;
             }
             __syncwarp();
-            if (t + (int)gridDim.x < p.tiles) fetch(t + gridDim.x);
+        };
+        // the tile's row block and column tile, advanced without a division
+        const int dm = gridDim.x / p.tiles_n, dn = gridDim.x % p.tiles_n;
+        int tm = blockIdx.x / p.tiles_n, tn = blockIdx.x % p.tiles_n, cur = -1, tl = 0;
+        uint32_t res_ph = 0;   // of the residual box's barrier
+        bool res_due = false;  // a residual load is in flight
+        const bool tab_ok = !gelu_kind(KIND) || mbar_wait(tab_full, 0, abort, p.status, kStatusTimeoutTma, p.wait_cycles);
+        for (int t = blockIdx.x; t < p.tiles && tab_ok; t += gridDim.x, ++tl) {
+            const int b = p.nbuf == 2 ? tl & 1 : 0;
+            const uint32_t use = (uint32_t)(p.nbuf == 2 ? tl >> 1 : tl);
+            const int m0 = tm * BM, n0 = tn * BN + h * HALF;
+            if (tn != cur) params(n0);
+            cur = tn;
+            tm += dm;
+            tn += dn;
+            if (tn >= p.tiles_n) {
+                tn -= p.tiles_n;
+                ++tm;
+            }
             const int64_t row = (int64_t)m0 + 32 * q + lane;
             const bool row_ok = row < p.M;
             // this row's residual (row modulo res_rows broadcasts a [res_rows, N] table)
-            const int16_t *rrow = (ep.res && row_ok) ? ep.res + (row % ep.res_rows) * ep.ldr + n0 : nullptr;
+            const int16_t *rrow = (ep.res && row_ok) ? ep.res + (row < ep.res_rows ? row : row % ep.res_rows) * ep.ldr + n0 : nullptr;
             const bool rvec = ((uintptr_t)rrow & 15) == 0;
-            const bool has_res = ep.res != nullptr;
-            const bool rfast = has_res && ep.s_r >= 17;
             const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * acc_cols + h * HALF);
             if constexpr (kFastKind && NB == 1) {
-                if (ush && (!has_res || rfast)) {
-                    // the residuals of the first 32 columns are fetched while the MMAs run
+                if (form != FORM_GENERAL) {
+                    // the residuals (of the first 32 columns) are fetched while the MMAs run
+                    constexpr bool kResBox = KIND == KIND_RQ16 && HALF == 32;
+                    const bool rbox = kResBox && p.res_tma;
+                    uint8_t *box = p.tma_store ? stg + (warp - EPI0) * p.tma_store * box_bytes<KIND>() : nullptr;
+                    if (rbox) {
+                        if (lane == 0) {
+                            tma_store_wait_read();  // the box's last results are on their way
+                            const uint32_t y = (uint32_t)(m0 + 32 * q), rows = (uint32_t)ep.res_rows;
+                            mbar_expect_tx(res_full(warp - EPI0), 2048);
+                            tma_load_2d(smem_u32(box), &p.rmap, n0, (int32_t)(y < rows ? y : y % rows), res_full(warp - EPI0));
+                        }
+                        __syncwarp();
+                        res_due = true;
+                    }
                     uint32_t rpa[16];
 #pragma unroll
                     for (int j = 0; j < 16; ++j) rpa[j] = 0;
-                    if (kResKind && has_res) res_group(rrow, 0, p.N - n0, rvec, rpa);
+                    if (kResKind && has_res && !rbox) res_group(rrow, 0, p.N - n0, rvec, rpa);
                     if (!mbar_wait(acc_full(b), use & 1, abort, p.status, kStatusTimeoutMma, p.wait_cycles)) break;
                     tc_fence_after();
                     char *dst = row_ok ? (char *)ep.C + (row * ep.ldc + n0) * (bits / 8) : nullptr;
                     const bool vec_ok = ((uintptr_t)dst & 15) == 0;
                     const int ncol_row = p.N - n0;
-                    const int32_t rnd = 1 << (s_0 - 33), sh = s_0 - 32;
-                    const int8_t *gt = gtab + 32767;
+                    const int32_t rnd = one_shift ? 1 << (s_0 - 33) : 0, sh = s_0 - 32;
+                    const uint8_t *gt = gtab;  // the entry of -32767
                     const uint32_t eb = acc_empty(b);
-                    uint8_t *box = p.tma_store ? stg + (warp - EPI0) * kStageBytes : nullptr;
-                    if (p.nseg == 1) {
-                        if (kResKind && has_res)
-                            epi_fast<KIND, BN, HALF, 1, kResKind>(ep, tbase, s_bias, s_mult, rnd, sh, rpa, rrow, rvec, dst,
-                                                                   ncol_row, vec_ok, gt, eb, lane, box, &p.cmap, n0,
-                                                                   m0 + 32 * q);
-                        else
-                            epi_fast<KIND, BN, HALF, 1, false>(ep, tbase, s_bias, s_mult, rnd, sh, rpa, rrow, rvec, dst,
-                                                               ncol_row, vec_ok, gt, eb, lane, box, &p.cmap, n0,
-                                                               m0 + 32 * q);
+                    if (rbox) {
+                        if (!mbar_wait(res_full(warp - EPI0), res_ph, abort, p.status, kStatusTimeoutTma, p.wait_cycles)) break;
+                        res_ph ^= 1u;
+                        res_due = false;
+                    }
+                    auto epi = [&](auto nseg_c, auto res_c, auto form_c) {
+                        constexpr int NS = decltype(nseg_c)::value, RS = decltype(res_c)::value, FM = decltype(form_c)::value;
+                        epi_fast<KIND, BN, HALF, NS, RS, FM>(ep, tbase, s_bias, s_mult, s_shift, s_rnd, n0, p.N, rnd, sh, rpa,
+                                                             rrow, rvec, dst, ncol_row, vec_ok, gt, eb, lane, box, p.tma_store,
+                                                             &p.cmap, n0, m0 + 32 * q);
+                    };
+                    auto epi_res = [&](auto nseg_c, auto form_c) {
+                        if (rbox) epi(nseg_c, Int<kResBox ? 2 : 0>{}, form_c);
+                        else if (kResKind && has_res) epi(nseg_c, Int<kResKind ? 1 : 0>{}, form_c);
+                        else epi(nseg_c, Int<0>{}, form_c);
+                    };
+                    constexpr bool kFlt = KIND == KIND_RQ8 || KIND == KIND_F16OUT;
+                    if (WRES || p.nseg == 1) {  // (resident weights: K <= 1024)
+                        if (kFlt && form == FORM_FLT) epi(Int<1>{}, Int<0>{}, Int<kFlt ? FORM_FLT : FORM_UNI>{});
+                        else if (form == FORM_UNI) epi_res(Int<1>{}, Int<FORM_UNI>{});
+                        else epi_res(Int<1>{}, Int<FORM_VAR>{});
                     } else {
-                        if (kResKind && has_res)
-                            epi_fast<KIND, BN, HALF, 2, kResKind>(ep, tbase, s_bias, s_mult, rnd, sh, rpa, rrow, rvec, dst,
-                                                                   ncol_row, vec_ok, gt, eb, lane, box, &p.cmap, n0,
-                                                                   m0 + 32 * q);
-                        else
-                            epi_fast<KIND, BN, HALF, 2, false>(ep, tbase, s_bias, s_mult, rnd, sh, rpa, rrow, rvec, dst,
-                                                               ncol_row, vec_ok, gt, eb, lane, box, &p.cmap, n0,
-                                                               m0 + 32 * q);
+                        if (kFlt && form == FORM_FLT) epi(Int<2>{}, Int<0>{}, Int<kFlt ? FORM_FLT : FORM_UNI>{});
+                        else epi_res(Int<2>{}, Int<FORM_UNI>{});
                     }
                     continue;
                 }
@@ -890,7 +1158,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     const int ncol = min(16, p.N - (n0 + c0));
                     if (row_ok && ncol > 0) {
                         int32_t out[16];
-                        const int8_t *gt = gtab + 32767;
+                        const uint8_t *gt = gtab + 32767;
                         epi_chunk<KIND, FAST, RFAST>(ep, has_res, rp, acc, cb, cm, cs, cr, gt, out);
                         char *dst = (char *)ep.C + (row * ep.ldc + n0 + c0) * (bits / 8);
                         const bool vec = ncol == 16 && (((uintptr_t)dst & 15) == 0);
@@ -971,6 +1239,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                 else go(F_{}, F_{});
             }
         }
+        if (res_due) {  // after an abort: the load in flight ends (bounded) before the CTA can exit
+            const long long t0 = clock64();
+            while (!mbar_try(res_full(warp - EPI0), res_ph) && clock64() - t0 < p.wait_cycles) {
+            }
+        }
         if (p.tma_store && lane == 0) tma_store_wait_all();  // this warp's stores are complete
     }
 
@@ -988,33 +1261,38 @@ inline int num_sms() { return sm_count(); }
 // Dynamic shared memory of one instantiation (wres: resident weight bytes).
 // stg: the epilogue warps' TMA-store boxes (0 without TMA stores).
 template <int BN, int STAGES, int KIND, bool AF16, bool WRES>
-size_t smem_bytes(int wres, int stg = 0) {
-    return 1024 + (size_t)STAGES * Smem<BN, AF16, WRES>::kStage + (WRES ? wres : 0) + 8 * (3 * STAGES + 5 + kMaxWk) +
-           32 + 4 * 4 * BN * 4 + (gelu_kind(KIND) ? 65536 : 0) + (stg ? 1024 + stg : 0);
+size_t smem_bytes(int wres, int stg = 0, int stages = STAGES) {
+    return 1024 + (size_t)stages * Smem<BN, AF16, WRES>::kStage + (WRES ? wres : 0) + 8 * (3 * STAGES + 6 + kMaxWk + epi_warps<BN, AF16>()) +
+           32 + 4 * prm_words<BN, WRES>() + (gelu_kind(KIND) ? 65536 : 0) + (stg ? 1024 + stg : 0);
 }
-template <int BN, bool AF16>
-constexpr int epi_warps() { return 4 * ((AF16 && BN == 192) ? 3 : 2); }
 constexpr size_t kSmemMax = 227 * 1024;
 
 template <int BN, int STAGES, int KIND, int NB, bool AF16, bool WRES>
 cudaError_t launch_tc(TcParams<NB> &tp, cudaStream_t s) {
     // TMA stores when the output allows them (set up by run) and their boxes fit next to the rest
-    constexpr int stg = epi_warps<BN, AF16>() * kStageBytes;
-    if (tp.tma_store && smem_bytes<BN, STAGES, KIND, AF16, WRES>(tp.wres_bytes, stg) > kSmemMax) tp.tma_store = 0;
-    const size_t smem = smem_bytes<BN, STAGES, KIND, AF16, WRES>(tp.wres_bytes, tp.tma_store ? stg : 0);
+    constexpr int stg = epi_warps<BN, AF16>() * box_bytes<KIND>();
+    tp.stages = STAGES;
+    if (tp.tma_store) tp.tma_store = tp.res_tma ? 1 : 2;
+    auto bytes = [&](int boxes) { return smem_bytes<BN, STAGES, KIND, AF16, WRES>(tp.wres_bytes, boxes * stg, tp.stages); };
+    // resident weights: as many stages as fit beside one box a warp (at least 3).  A's blocks come at L2's
+    // latency, so the stages in flight set the rate: 12800 x 384 x 384 with 3 stages 600 clocks a K block
+    while (WRES && tp.stages > 3 && bytes(tp.tma_store ? 1 : 0) > kSmemMax) --tp.stages;
+    while (tp.tma_store && bytes(tp.tma_store) > kSmemMax) --tp.tma_store;
+    if (!tp.tma_store) tp.res_tma = 0;
+    const size_t smem = bytes(tp.tma_store);
     if (smem > kSmemMax) return cudaErrorInvalidValue;
     static SmemLimit limit;
     const cudaError_t attr_err =
         raise_smem_limit(limit, (const void *)gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES>, (int)kSmemMax);
     if (attr_err != cudaSuccess) return attr_err;
     int grid = tp.tiles < num_sms() ? tp.tiles : num_sms();
-    if (WRES) {  // a multiple of tiles_n: every CTA keeps one n block of W
-        const int tiles_m = tp.tiles / tp.tiles_n;
-        int per_n = num_sms() / tp.tiles_n;
-        per_n = per_n < 1 ? 1 : (per_n > tiles_m ? tiles_m : per_n);
-        grid = per_n * tp.tiles_n;
-    }
-    launch_after(gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES>, grid, kThreads, smem, s, tp);
+    // a multiple of tiles_n: every CTA keeps one n block of W (WRES: always; else where that costs no round)
+    const int tiles_m = tp.tiles / tp.tiles_n;
+    int per_n = num_sms() / tp.tiles_n;
+    per_n = per_n < 1 ? 1 : (per_n > tiles_m ? tiles_m : per_n);
+    const int whole = per_n * tp.tiles_n;
+    if (WRES || (whole <= grid && (tp.tiles + whole - 1) / whole == (tp.tiles + grid - 1) / grid)) grid = whole;
+    launch_after(gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES>, grid, tc_threads<BN, AF16>(), smem, s, tp);
     return cudaGetLastError();
 }
 
@@ -1066,18 +1344,26 @@ cudaError_t run(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s) {
     if (alloc > 512) return cudaErrorInvalidValue;
     tp.tmem_cols = alloc;
     gemm_debug_wait(&tp.dbg_skip, &tp.wait_cycles);
-    // TMA tensor stores of the outputs: 16 x 32 boxes of C (1-byte outputs: 16-byte box rows; 2-byte
-    // outputs: 32-byte rows in the 32-byte swizzle), for a C whose rows start on 16-byte boundaries
+    // TMA tensor stores of the outputs: 32 x 32 boxes of C (1-byte outputs: 32-byte rows in the 32-byte
+    // swizzle; 2-byte outputs: 64-byte rows in the 64-byte swizzle), for a C whose rows start on 16-byte boundaries
     tp.tma_store = 0;
     if (NB == 1 && ep.out_bits != 32) {
         const int esz = ep.out_bits == 8 ? 1 : 2;  // int8, or int16 / fp16-carried int8
         if (((uintptr_t)ep.C % 16) == 0 && (ep.ldc * esz) % 16 == 0 && gp.N * esz >= 16)
             tp.tma_store = gemm_make_map(&tp.cmap, ep.C, esz == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_UINT16,
-                                         esz, gp.M, gp.N, ep.ldc, 16, 32,
-                                         esz == 1 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_32B)
+                                         esz, gp.M, gp.N, ep.ldc, 32, 32,
+                                         esz == 1 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B)
                                ? 1
                                : 0;
     }
+    // an int16 residual under int16 outputs by TMA, if its rows allow a map and no box wraps around
+    tp.res_tma = 0;
+    if (tp.tma_store && ep.out_bits == 16 && ep.res && BN == 128 && AF16 && ((uintptr_t)ep.res % 16) == 0 && ep.ldr % 8 == 0 &&
+        ep.res_rows < (1ll << 31) && (ep.res_rows >= gp.M || ep.res_rows % 32 == 0))
+        tp.res_tma = gemm_make_map(&tp.rmap, ep.res, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, ep.res_rows, gp.N, ep.ldr, 32, 32,
+                                   CU_TENSOR_MAP_SWIZZLE_64B)
+                         ? 1
+                         : 0;
     if (WRES) {
         if (nseg != 1) return cudaErrorInvalidValue;
         tp.wres_bytes = ((tp.seg[0].klen + BK - 1) / BK) * Smem<BN, AF16, WRES>::kWtile;

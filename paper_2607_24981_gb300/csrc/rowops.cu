@@ -432,9 +432,9 @@ __device__ __noinline__ LnRow ln_row_general(int64_t S, int64_t Q, int32_t C, in
 // 10 % slower.
 // 32-bit normalisation: after at least one Newton step R >= isqrt(V) >= |y| for every y = x - mu of
 // the row (a floored Newton step from any positive start lands at or above isqrt(V)), so
-// |y F| <= |y| (2^31 - 1) / R < 2^31 and y F fits int32; with one shift s >= 33 for every column and
-// |beta| <= 2^30 the requantisation is the high-word form with a scalar rounding constant; otherwise
-// (or for rows with iters = 0 and V >= 2^32) the 64-bit formulas run.
+// |y F| <= |y| (2^31 - 1) / R < 2^31 and y F fits int32; with shifts s >= 33 and |beta| <= 2^30 in every
+// column the requantisation is the high-word form (with a scalar rounding constant when the shifts are
+// the same); otherwise (or for rows with iters = 0 and V >= 2^32) the 64-bit formulas run.
 template <typename TIn, typename TOut, int LPR, int CPL, bool FULL>
 __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const LnConst lc) {
     grid_wait();
@@ -463,12 +463,15 @@ __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const
         ((int4 *)s_shift)[i] = __ldg((const int4 *)p.shift + i);
     }
     __syncthreads();
-    const int32_t uniform_shift = s_shift[0];  // the fast form needs one shift >= 33 for every column
-    bool col_fast = true;
-    for (int c = threadIdx.x; c < C; c += blockDim.x)
-        col_fast &= s_beta[c] >= -(1 << 30) && s_beta[c] <= (1 << 30) && s_shift[c] == uniform_shift;
-    const bool cols_fast = __syncthreads_and(col_fast) != 0 && uniform_shift >= 33;
-    const int32_t rnd = cols_fast ? 1 << (uniform_shift - 33) : 0, sh = uniform_shift - 32;
+    // the fast forms need shifts >= 33 for every column: one for all of them, or each its own
+    const int32_t shift0 = s_shift[0];
+    bool col_fast = true, col_same = true;
+    for (int c = threadIdx.x; c < C; c += blockDim.x) {
+        col_fast &= s_beta[c] >= -(1 << 30) && s_beta[c] <= (1 << 30) && s_shift[c] >= 33;
+        col_same &= s_shift[c] == shift0;
+    }
+    const bool cols_fast = __syncthreads_and(col_fast) != 0, cols_same = __syncthreads_and(col_same) != 0;
+    const int32_t rnd = cols_fast ? 1 << (shift0 - 33) : 0, sh = shift0 - 32;
 
     for (; __any_sync(0xffffffffu, row < p.rows); row += step, load()) {
         bool small = true;
@@ -564,13 +567,20 @@ __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const
                     values(i, u4, x);
                     const int4 b4 = *(const int4 *)(s_beta + c0 + u4), m4 = *(const int4 *)(s_mult + c0 + u4);
                     const int32_t be[4] = {b4.x, b4.y, b4.z, b4.w}, mm[4] = {m4.x, m4.y, m4.z, m4.w};
+                    // (x - mu) F = x F + mF in wrapping 32-bit arithmetic (the product fits int32)
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        // (x - mu) F = x F + mF in wrapping 32-bit arithmetic (the product fits int32)
-                        const int32_t n = (int32_t)((uint32_t)x[u] * (uint32_t)F32 + (uint32_t)mF) >> 1;
-                        o[u] = __viaddmin_s32_relu(rq_hi(n + be[u], mm[u], rnd, sh), LnBias<TOut>::one,
-                                                   2 * LnBias<TOut>::one);
+                    for (int u = 0; u < 4; ++u) o[u] = ((int32_t)((uint32_t)x[u] * (uint32_t)F32 + (uint32_t)mF) >> 1) + be[u];
+                    if (cols_same) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) o[u] = rq_hi(o[u], mm[u], rnd, sh);
+                    } else {
+                        const int4 s4 = *(const int4 *)(s_shift + c0 + u4);
+                        const int32_t ss[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) o[u] = rq_hi1(o[u], mm[u], ss[u] - 33);
                     }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) o[u] = __viaddmin_s32_relu(o[u], LnBias<TOut>::one, 2 * LnBias<TOut>::one);
                     if (FULL ? nc > 0 : LPR * i < nc) ln_store4_biased<TOut>(yr + LPR * i * EPC + u4, o);
                 }
             }

@@ -213,6 +213,8 @@ def test_int_layernorm_row_forms(ilw, orc, rows, C, in_bits, out_bits, iters):
     beta, mult, shift = synth.ln_params(7, f"lnr{C}", C)
     if out_bits == 16:
         shift = shift - 7
+    if rows % 2:
+        shift = shift + (np.arange(C) % 3).astype(shift.dtype)  # a shift of its own for every column
     got = ilw.int_layernorm(dev(X), dev(beta), dev(mult), dev(shift), iters, out_bits)
     assert_same(host(got), orc.int_layernorm(X, beta, mult, shift, iters, out_bits), f"ln rows {rows} x {C}")
 
@@ -404,6 +406,39 @@ def test_block_forward(ilw, orc, cfg):
                           m_r=bp["m_r2"], s_r=bp["s_r2"])
     assert_same(host(y2), y_ref, "y via ops")
     ilw.device_status()
+
+
+@pytest.mark.parametrize("M,N,K,out_bits,res_rows,mult", [
+    (130, 384, 384, 16, 130, 0), (300, 384, 1536, 16, 300, 0), (97, 104, 128, 16, 32, 0), (200, 136, 256, 16, 50, 0),
+    (33, 576, 384, 8, 0, 0), (257, 200, 1104, 8, 0, 0), (129, 1152, 384, 108, 0, 0), (64, 130, 64, 108, 0, 0),
+    (140, 256, 256, 8, 0, 1 << 30), (140, 384, 320, 108, 0, 3 << 28), (70, 48, 192, 8, 70, 0)])
+@pytest.mark.parametrize("a_f16,spread", [(False, False), (True, False), (True, True), (False, True)])
+def test_gemm_epilogue_forms(ilw, orc, M, N, K, out_bits, res_rows, mult, a_f16, spread):
+    """One shift for all columns, or (spread) one each from 29 on: int8 results in floats with the integers for
+    values near a half (mult: a coarse scale, whose results are often exact halves), accumulators inside and
+    beyond 2^22, residuals of whole and broadcast tables (32-row boxes that wrap or not), in place, and columns
+    past the last tile."""
+    A = synth.uniform_int(21, f"ef{M}{K}", (M, K), -127, 127, np.int8)
+    W, b, m, s = synth.gemm_params(21, f"efW{N}{K}", N, K, 60.0 if out_bits != 16 else 9000.0, 30.0, "literal")
+    A[M // 2], W[N // 3] = 127, 127  # accumulators up to 127^2 K
+    s = (29 + np.arange(N) % 14).astype(s.dtype) if spread else np.full_like(s, s[0])
+    if mult:
+        m = np.full_like(m, mult)
+        m[::5] = -m[::5]
+        s = np.full_like(s, 42) if not spread else s
+    A_d = dev(A.astype(np.float16) if a_f16 else A)
+    args = (A_d, ilw.pack_weight(dev(W)), N, dev(b), dev(m), dev(s), out_bits)
+    if res_rows:
+        res = synth.uniform_int(21, f"efr{res_rows}{N}", (res_rows, N), -32767, 32767, np.int16)
+        want = orc.gemm_requant(A, W, b, m, s, out_bits, res, 3 << 28, 30)
+        r_d = dev(res)
+        assert_same(host(ilw.gemm(*args, res=r_d, m_r=3 << 28, s_r=30)), want, "residual")
+        if res_rows == M and out_bits == 16:  # in place
+            ilw.gemm(*args, res=r_d, m_r=3 << 28, s_r=30, out=r_d)
+            assert_same(host(r_d), want, "residual in place")
+    else:
+        want = orc.gemm_requant(A, W, b, m, s, 8, None, 0, 0)
+        assert_same(host(ilw.gemm(*args)), want, "int8")
 
 
 # ------------------------------------------------------------- launches that overlap the one before
