@@ -126,6 +126,10 @@ int ilwdetr_gemm_gelu(const int8_t *A, int64_t lda, const void *Wp, const int32_
                       const ilw_gelu_t *gelu, int32_t m_g, int32_t s_g, int8_t *H, int64_t ldh,
                       ilw_stream_t stream);
 
+/* ilwdetr_gemm_requant to int8 followed by ReLU: C = max(sat8(rq(A W^T + bias; mult, shift)), 0). */
+int ilwdetr_gemm_relu(const int8_t *A, int64_t lda, const void *Wp, const int32_t *bias, const int32_t *mult,
+                      const int32_t *shift, int32_t M, int32_t N, int32_t K, int8_t *C, int64_t ldc, ilw_stream_t stream);
+
 /* The integer linear layer (Sec. 3.2.1) in its general form: the computation of ilwdetr_gemm_requant
  * (epilogue ILW_EPI_REQUANT) or of ilwdetr_gemm_gelu (ILW_EPI_GELU), with the activation operand
  * A either int8 (a_form 8; lda % 16 == 0) or the same int8 values carried in fp16 (a_form
@@ -423,6 +427,11 @@ int ilwdetr_int_sigmoid(const int32_t *X, int32_t *Y, int64_t n, const ilw_sigmo
 int ilwdetr_ivit_shiftgelu(const int32_t *X, int64_t ldx, int64_t rows, int32_t L, int32_t *Y, int64_t ldy,
                            const ilw_gelu_t *p, ilw_stream_t stream);
 
+/* ilwdetr_requant of int32 X to int16 or int32 Y (out_bits), and sig int32 [rows, ld_sig] = ilwdetr_int_sigmoid of
+ * that result (a box and the reference logits it comes from, in one launch); ld_sig % 4 == 0. */
+int ilwdetr_requant_sigmoid(const int32_t *X, int64_t ldx, int64_t rows, int32_t C, int32_t m1, int32_t s1, const int16_t *Z,
+                            int64_t ldz, int64_t z_rows, int32_t m2, int32_t s2, int32_t out_bits, void *Y, int64_t ldy,
+                            const ilw_sigmoid_t *p, int32_t *sig, int64_t ld_sig, ilw_stream_t stream);
 /* ReLU of int8 values (the hidden layers of the detection head's box branch, Table 5):
  * Y = max(X, 0).  X, Y device [n] (may alias), 4-byte aligned. */
 int ilwdetr_relu_i8(const int8_t *X, int8_t *Y, int64_t n, ilw_stream_t stream);

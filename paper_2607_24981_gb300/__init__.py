@@ -16,7 +16,7 @@ __all__ = [
     "BlockWeights", "block_forward", "block_workspace_bytes", "device_status",
     "patch_embed", "patch_embed_workspace_bytes", "Backbone", "Graphed",
     "requant", "resample_nearest", "DecoderWeights", "decoder_workspace_bytes", "decoder_layer_forward",
-    "Projector", "Detector", "int_sigmoid", "relu_i8", "topk", "gather_rows", "gather_rows_batched", "DetectionHead", "TwoStage",
+    "Projector", "Detector", "int_sigmoid", "requant_sigmoid", "gemm_relu", "relu_i8", "topk", "gather_rows", "gather_rows_batched", "DetectionHead", "TwoStage",
     "QueryPos", "BoxRefine", "ivit_shiftgelu",
 ]
 
@@ -149,6 +149,9 @@ SIGNATURES = {
                          _I64, _VP], C.c_int),
     "ilwdetr_resample_nearest": ([_VP, _I64, _I32, _I32, _I32, _I32, _VP, _I64, _I32, _I32, _VP], C.c_int),
     "ilwdetr_int_sigmoid": ([_VP, _VP, _I64, C.POINTER(SigmoidT), _VP], C.c_int),
+    "ilwdetr_requant_sigmoid": ([_VP, _I64, _I64, _I32, _I32, _I32, _VP, _I64, _I64, _I32, _I32, _I32, _VP, _I64,
+                                 C.POINTER(SigmoidT), _VP, _I64, _VP], C.c_int),
+    "ilwdetr_gemm_relu": ([_VP, _I64, _VP, _VP, _VP, _VP, _I32, _I32, _I32, _VP, _I64, _VP], C.c_int),
     "ilwdetr_relu_i8": ([_VP, _VP, _I64, _VP], C.c_int),
     "ilwdetr_ivit_shiftgelu": ([_VP, _I64, _I64, _I32, _VP, _I64, C.POINTER(GeluT), _VP], C.c_int),
     "ilwdetr_topk": ([_VP, _I64, _I32, _I32, _I32, _VP, _VP, _VP], C.c_int),
@@ -235,6 +238,18 @@ def gemm_requant(A, Wp, N, bias, mult, shift, out_bits=8, res=None, m_r=0, s_r=0
     _check(lib().ilwdetr_gemm_requant(_ptr(A), A.stride(0), _ptr(Wp), _ptr(bias), _ptr(mult),
                                       _ptr(shift), M, N, K, out_bits, _ptr(out), out.stride(0),
                                       None if r is None else C.byref(r), _stream()), "gemm_requant")
+    return out
+
+
+def gemm_relu(A, Wp, N, bias, mult, shift, out=None):
+    """ilwdetr_gemm_relu: A int8 [M, K] x packed W [N, K] -> ReLU of the int8 result [M, N]."""
+    import torch
+
+    M, K = A.shape
+    if out is None:
+        out = torch.empty((M, N), dtype=torch.int8, device=A.device)
+    _check(lib().ilwdetr_gemm_relu(_ptr(A), A.stride(0), _ptr(Wp), _ptr(bias), _ptr(mult), _ptr(shift), M, N, K, _ptr(out),
+                                   out.stride(0), _stream()), "gemm_relu")
     return out
 
 
@@ -720,6 +735,21 @@ def int_sigmoid(X, sig: dict, out=None):
     return out
 
 
+def requant_sigmoid(X, m1, s1, Z, m2, s2, sig: dict, out_bits=16):
+    """ilwdetr_requant_sigmoid: requant of the int32 X [rows, C] with the second term Z -> (that result int16 or
+    int32, its integer sigmoid int32)."""
+    import torch
+
+    rows, Cn = X.shape
+    out = torch.empty((rows, Cn), dtype={16: torch.int16, 32: torch.int32}[out_bits], device=X.device)
+    s = torch.empty((rows, Cn), dtype=torch.int32, device=X.device)
+    zp, ldz, zr = (None, 0, 1) if Z is None else (_ptr(Z), Z.stride(0), Z.shape[0])
+    p = SigmoidT(sig["I0"], sig.get("k_inter", 8), sig.get("k_out", 8))
+    _check(lib().ilwdetr_requant_sigmoid(_ptr(X), X.stride(0), rows, Cn, m1, s1, zp, ldz, zr, m2, s2, out_bits, _ptr(out), Cn,
+                                         C.byref(p), _ptr(s), Cn, _stream()), "requant_sigmoid")
+    return out, s
+
+
 def relu_i8(X, out=None):
     """ilwdetr_relu_i8: max(X, 0) on int8 (in place when out is X)."""
     import torch
@@ -795,13 +825,11 @@ class DetectionHead:
         d = out.shape[1]
         logits = gemm_requant(out, t["w_cls_p"], self.C, t["b_cls"], None, None, 32)
         scores = int_sigmoid(logits, {"I0": hp["cls_I0"], "k_inter": hp["k_inter"], "k_out": hp["cls_k_out"]})
-        h1 = gemm_requant(out, t["w_b1_p"], d, t["b_b1"], t["m_b1"], t["s_b1"], 8)
-        relu_i8(h1, out=h1)
-        h2 = gemm_requant(h1, t["w_b2_p"], d, t["b_b2"], t["m_b2"], t["s_b2"], 8)
-        relu_i8(h2, out=h2)
+        h1 = gemm_relu(out, t["w_b1_p"], d, t["b_b1"], t["m_b1"], t["s_b1"])
+        h2 = gemm_relu(h1, t["w_b2_p"], d, t["b_b2"], t["m_b2"], t["s_b2"])
         dlt = gemm_requant(h2, t["w_b3_p"], 4, t["b_b3"], None, None, 32)
-        z = requant(dlt, hp["m_d"], hp["s_d"], ref16, hp["m_ref"], hp["s_ref"], out_bits=32)
-        boxes = int_sigmoid(z, {"I0": hp["box_I0"], "k_inter": hp["k_inter"], "k_out": 17})
+        z, boxes = requant_sigmoid(dlt, hp["m_d"], hp["s_d"], ref16, hp["m_ref"], hp["s_ref"],
+                                   {"I0": hp["box_I0"], "k_inter": hp["k_inter"], "k_out": 17}, out_bits=32)
         return scores, boxes, z
 
 
@@ -827,15 +855,11 @@ class BoxRefine:
         rp, t = self.rp, self.t
         d = x.shape[1]
         a = requant(x, rp["m_in"], rp["s_in"], out_bits=8)
-        h1 = gemm_requant(a, t["w_b1_p"], d, t["b_b1"], t["m_b1"], t["s_b1"], 8)
-        relu_i8(h1, out=h1)
-        h2 = gemm_requant(h1, t["w_b2_p"], d, t["b_b2"], t["m_b2"], t["s_b2"], 8)
-        relu_i8(h2, out=h2)
+        h1 = gemm_relu(a, t["w_b1_p"], d, t["b_b1"], t["m_b1"], t["s_b1"])
+        h2 = gemm_relu(h1, t["w_b2_p"], d, t["b_b2"], t["m_b2"], t["s_b2"])
         dlt = gemm_requant(h2, t["w_b3_p"], 4, t["b_b3"], None, None, 32)
-        ref = requant(dlt, rp["m_d"], rp["s_d"], ref16, rp["m_ref"], rp["s_ref"], out_bits=16)
-        ref32 = requant(ref, 1 << 30, 30, out_bits=32)
-        boxes = int_sigmoid(ref32, {"I0": rp["box_I0"], "k_inter": rp["k_inter"], "k_out": 17})
-        return ref, boxes
+        return requant_sigmoid(dlt, rp["m_d"], rp["s_d"], ref16, rp["m_ref"], rp["s_ref"],
+                               {"I0": rp["box_I0"], "k_inter": rp["k_inter"], "k_out": 17})
 
 
 class TwoStage:
@@ -866,12 +890,10 @@ class TwoStage:
         # the selected tokens' memory rows (each image its own) and anchors
         sel = gather_rows_batched(memory, idx)
         anc = gather_rows(t["anchor16"], idx.view(-1))
-        h1 = gemm_requant(sel, t["w_p1_p"], d, t["b_p1"], t["m_p1"], t["s_p1"], 8)
-        relu_i8(h1, out=h1)
+        h1 = gemm_relu(sel, t["w_p1_p"], d, t["b_p1"], t["m_p1"], t["s_p1"])
         dlt = gemm_requant(h1, t["w_p2_p"], 4, t["b_p2"], None, None, 32)
-        ref16 = requant(dlt, tp["m_d"], tp["s_d"], anc, tp["m_a"], tp["s_a"], out_bits=16)
-        ref32 = requant(ref16, 1 << 30, 30, out_bits=32)
-        boxes = int_sigmoid(ref32, {"I0": tp["ref_I0"], "k_inter": tp["k_inter"], "k_out": 17})
+        ref16, boxes = requant_sigmoid(dlt, tp["m_d"], tp["s_d"], anc, tp["m_a"], tp["s_a"],
+                                       {"I0": tp["ref_I0"], "k_inter": tp["k_inter"], "k_out": 17})
         return vals, idx, ref16, boxes
 
 
@@ -900,8 +922,7 @@ class QueryPos:
     def forward(self, boxes, out=None):
         pq, t = self.pq, self.t
         requant(boxes, pq["m_box"], pq["s_box"], out_bits=8, out=self.b8[:, :4])
-        h = gemm_requant(self.b8, t["w_q1_p"], self.hidden, t["b_q1"], t["m_q1"], t["s_q1"], 8)
-        relu_i8(h, out=h)
+        h = gemm_relu(self.b8, t["w_q1_p"], self.hidden, t["b_q1"], t["m_q1"], t["s_q1"])
         return gemm_requant(h, t["w_q2_p"], self.d, t["b_q2"], t["m_q2"], t["s_q2"], 16, out=out)
 
 

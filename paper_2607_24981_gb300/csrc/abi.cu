@@ -152,7 +152,7 @@ namespace {
 int gemm_impl(const void *A, int32_t a_form, int64_t lda, const void *Wp, const int32_t *bias, const int32_t *mult,
               const int32_t *shift, int32_t M, int32_t N, int32_t K, int32_t epilogue, int32_t out_bits, void *C,
               int64_t ldc, const ilw_residual_t *res, const ilw_gelu_t *gelu, int32_t m_g, int32_t s_g,
-              ilw_stream_t stream, const char *what) {
+              ilw_stream_t stream, const char *what, bool relu = false) {
     if (a_form != 8 && a_form != ILW_I8_IN_F16)
         return fail(ILW_ERR_INVALID_ARG, "%s: a_form=%d must be 8 or ILW_I8_IN_F16", what, a_form);
     int rc;
@@ -199,6 +199,7 @@ int gemm_impl(const void *A, int32_t a_form, int64_t lda, const void *Wp, const 
     ep.mult = mult;
     ep.shift = shift;
     ep.out_bits = out_bits;
+    ep.relu = relu ? 1 : 0;
     ep.C = C;
     ep.ldc = ldc;
     if (use_res) {
@@ -224,6 +225,12 @@ int ilwdetr_gemm_requant(const int8_t *A, int64_t lda, const void *Wp, const int
                          ilw_stream_t stream) {
     return gemm_impl(A, 8, lda, Wp, bias, mult, shift, M, N, K, ILW_EPI_REQUANT, out_bits, C, ldc, res, nullptr, 0,
                      0, stream, "gemm_requant");
+}
+
+int ilwdetr_gemm_relu(const int8_t *A, int64_t lda, const void *Wp, const int32_t *bias, const int32_t *mult,
+                      const int32_t *shift, int32_t M, int32_t N, int32_t K, int8_t *C, int64_t ldc, ilw_stream_t stream) {
+    return gemm_impl(A, 8, lda, Wp, bias, mult, shift, M, N, K, ILW_EPI_REQUANT, 8, C, ldc, nullptr, nullptr, 0, 0, stream,
+                     "gemm_relu", true);
 }
 
 int ilwdetr_gemm_gelu(const int8_t *A, int64_t lda, const void *Wp, const int32_t *bias,
@@ -364,9 +371,9 @@ int ilwdetr_shiftmax_attn(const void *Q, const void *K, const void *V, int64_t l
     return cuda_status(ilw::launch_attention(ap, (cudaStream_t)stream), "shiftmax_attn");
 }
 
-int ilwdetr_deform_attn(const int8_t *value, const int32_t *level_hw, int32_t L, const int32_t *ref_q16,
+static int deform_params(ilw::DeformParams &dp, const int8_t *value, const int32_t *level_hw, int32_t L, const int32_t *ref_q16,
                         const int32_t *off_q8, const uint8_t *w, int32_t B, int32_t Q, int32_t H, int32_t P,
-                        int32_t dh, int32_t m, int32_t s, int8_t *out, ilw_stream_t stream) {
+                        int32_t dh, int32_t m, int32_t s, int8_t *out) {
     if (L < 1 || L > 8 || !level_hw) return fail(ILW_ERR_INVALID_ARG, "deform: L=%d outside [1, 8]", L);
     if (B < 0 || Q < 0 || H < 1 || P < 1 || dh < 4 || dh % 4) return fail(ILW_ERR_INVALID_ARG, "deform: bad sizes (dh %% 4 == 0)");
     int rc = check_rq_scalar(s, "deform output");
@@ -374,7 +381,7 @@ int ilwdetr_deform_attn(const int8_t *value, const int32_t *level_hw, int32_t L,
     if (B == 0 || Q == 0) return ILW_OK;
     if (!value || !ref_q16 || !off_q8 || !w || !out) return fail(ILW_ERR_INVALID_ARG, "deform: NULL pointer");
     if (!aligned(value, 4) || !aligned(out, 4)) return fail(ILW_ERR_INVALID_ARG, "deform: value/out must be 4-byte aligned");
-    ilw::DeformParams dp{};
+    dp = ilw::DeformParams{};
     dp.value = value;
     dp.L = L;
     int64_t st = 0;
@@ -390,7 +397,14 @@ int ilwdetr_deform_attn(const int8_t *value, const int32_t *level_hw, int32_t L,
     dp.B = B; dp.Q = Q; dp.H = H; dp.P = P; dp.dh = dh;
     dp.m = m; dp.s = s;
     dp.out = out;
-    if (g_check_only) return ILW_OK;
+    return ILW_OK;
+}
+int ilwdetr_deform_attn(const int8_t *value, const int32_t *level_hw, int32_t L, const int32_t *ref_q16,
+                        const int32_t *off_q8, const uint8_t *w, int32_t B, int32_t Q, int32_t H, int32_t P,
+                        int32_t dh, int32_t m, int32_t s, int8_t *out, ilw_stream_t stream) {
+    ilw::DeformParams dp;
+    const int rc = deform_params(dp, value, level_hw, L, ref_q16, off_q8, w, B, Q, H, P, dh, m, s, out);
+    if (rc || B == 0 || Q == 0 || g_check_only) return rc;
     return cuda_status(ilw::launch_deform(dp, (cudaStream_t)stream), "deform_attn");
 }
 
@@ -506,6 +520,24 @@ int ilwdetr_requant(const void *X, int32_t in_bits, int64_t ldx, int64_t rows, i
     return cuda_status(ilw::launch_requant(p, (cudaStream_t)stream), "requant");
 }
 
+int ilwdetr_requant_sigmoid(const int32_t *X, int64_t ldx, int64_t rows, int32_t C, int32_t m1, int32_t s1, const int16_t *Z,
+                            int64_t ldz, int64_t z_rows, int32_t m2, int32_t s2, int32_t out_bits, void *Y, int64_t ldy,
+                            const ilw_sigmoid_t *p, int32_t *sig, int64_t ld_sig, ilw_stream_t stream) {
+    if (out_bits != 16 && out_bits != 32) return fail(ILW_ERR_INVALID_ARG, "requant_sigmoid: out_bits=%d must be 16 or 32", out_bits);
+    {
+        CheckPass pass;  // the two steps' own checks
+        int rc = ilwdetr_requant(X, 32, ldx, rows, C, m1, s1, Z, ldz, z_rows, m2, s2, out_bits, Y, ldy, stream);
+        if (!rc) rc = ilwdetr_int_sigmoid(X, sig, rows < 0 ? 0 : rows * C, p, stream);
+        if (rc) return rc;
+    }
+    if (rows == 0 || C == 0) return ILW_OK;
+    if (ld_sig < C || ld_sig % 4) return fail(ILW_ERR_INVALID_ARG, "requant_sigmoid: ld_sig < C or not a multiple of 4");
+    ilw::RequantParams rp{X, 32, ldx, rows, C, m1, s1, Z, ldz, Z ? z_rows : 1, m2, Z ? s2 : 1, out_bits, Y, ldy};
+    return cuda_status(ilw::launch_requant_sigmoid(rp, sig, ld_sig, ilw::make_shiftexp(p->I0, p->k_inter), p->k_out,
+                                                   (cudaStream_t)stream),
+                       "requant_sigmoid");
+}
+
 int ilwdetr_resample_nearest(const int8_t *X, int64_t x_bstride, int32_t B, int32_t Hi, int32_t Wi,
                              int32_t C, int8_t *Y, int64_t y_bstride, int32_t Ho, int32_t Wo,
                              ilw_stream_t stream) {
@@ -599,16 +631,33 @@ int ilwdetr_decoder_layer_forward(const ilw_decoder_params_t *p, const int16_t *
         int rc;
 #define ILW_TRY(x) \
         if ((rc = (x))) return rc
+        // Launches of a few microseconds are most of a layer, so steps that read the same rows share one; the
+        // checking pass runs the single steps' checks.
+#define ILW_LAUNCH(x, what)                                                         \
+        do {                                                                        \
+            const cudaError_t e = (x);                                              \
+            if (e != cudaSuccess) return cuda_status(e, what);                      \
+        } while (0)
+        const cudaStream_t st = (cudaStream_t)stream;
         // self-attention
-        ILW_TRY(ilwdetr_requant(tgt, 16, d, M, d, p->m_q1, p->s_q1, pos, d, M, p->m_q2, p->s_q2, 8, b.qk_in, d, stream));
-        ILW_TRY(ilwdetr_requant(tgt, 16, d, M, d, p->m_v1, p->s_v1, nullptr, 0, 1, 0, 1, 8, b.v_in, d, stream));
+        if (g_check_only) {
+            ILW_TRY(ilwdetr_requant(tgt, 16, d, M, d, p->m_q1, p->s_q1, pos, d, M, p->m_q2, p->s_q2, 8, b.qk_in, d, stream));
+            ILW_TRY(ilwdetr_requant(tgt, 16, d, M, d, p->m_v1, p->s_v1, nullptr, 0, 1, 0, 1, 8, b.v_in, d, stream));
+        } else {
+            ilw::RequantParams rp{tgt, 16, d, M, d, p->m_q1, p->s_q1, pos, d, M, p->m_q2, p->s_q2, 8, b.qk_in, d,
+                                  b.v_in, d, p->m_v1, p->s_v1};
+            ILW_LAUNCH(ilw::launch_requant(rp, st), "decoder requant");
+        }
         ILW_TRY(ilwdetr_gemm_requant(b.qk_in, d, p->w_qk, p->b_qk, p->m_qk, p->s_qk, M, 2 * d, d, 8, b.qkv, 3 * d, nullptr,
                                      stream));
         ILW_TRY(ilwdetr_gemm_requant(b.v_in, d, p->w_v, p->b_v, p->m_v, p->s_v, M, d, d, 8, b.qkv + 2 * d, 3 * d, nullptr,
                                      stream));
-        if (d / H < 64) {
-            // heads of 32 columns run on the tensor-memory attention of 64-column heads: q|k|v widened with
-            // zero columns (nothing added to q.k, zero outputs), the output narrowed back
+        ilw::AttnParams ap;
+        ILW_TRY(attn_params(ap, b.qkv, b.qkv + d, b.qkv + 2 * d, 3 * d, 8, B, Q, H, d / H, 0, &p->smx, p->m_o, p->s_o, b.o, 8, d));
+        if (d / H < 64 && ilw::launch_attention_res(ap, st, true) == cudaErrorNotSupported) {
+            // heads of 32 columns that the resident attention does not take run on the streaming one of
+            // 64-column heads: q|k|v widened with zero columns (nothing added to q.k, zero outputs), the output
+            // narrowed back
             const int64_t w = (int64_t)H * 64;
             if (!g_check_only) {
                 cudaError_t e = ilw::launch_head_pad64(b.qkv, 3 * d, M, 3 * H, d / H, b.qkv64, (cudaStream_t)stream);
@@ -626,35 +675,61 @@ int ilwdetr_decoder_layer_forward(const ilw_decoder_params_t *p, const int16_t *
         }
         ilw_residual_t r1{tgt, d, M, p->m_r1, p->s_r1};
         ILW_TRY(ilwdetr_gemm_requant(b.o, d, p->w_o, p->b_o, p->m_oc, p->s_oc, M, d, d, 16, b.x1, d, &r1, stream));
-        ILW_TRY(ilwdetr_int_layernorm(b.x1, 16, d, M, d, p->ln1_beta, p->ln1_mult, p->ln1_shift, p->ln_iters, b.t1, 16, d,
-                                      stream));
+        // the LayerNorm and the requantisation of its result
+        if (g_check_only) {
+            ILW_TRY(ilwdetr_int_layernorm(b.x1, 16, d, M, d, p->ln1_beta, p->ln1_mult, p->ln1_shift, p->ln_iters, b.t1, 16, d,
+                                          stream));
+            ILW_TRY(ilwdetr_requant(b.t1, 16, d, M, d, p->m_c1, p->s_c1, pos, d, M, p->m_c2, p->s_c2, 8, b.qc, d, stream));
+        } else {
+            ilw::LnParams lp{b.x1, 16, d, M, d, p->ln1_beta, p->ln1_mult, p->ln1_shift, p->ln_iters, b.t1, 16, d,
+                             b.qc, d, pos, d, p->m_c1, p->s_c1, p->m_c2, p->s_c2};
+            ILW_LAUNCH(ilw::launch_layernorm(lp, st), "decoder layernorm");
+        }
         // deformable cross-attention
-        ILW_TRY(ilwdetr_requant(b.t1, 16, d, M, d, p->m_c1, p->s_c1, pos, d, M, p->m_c2, p->s_c2, 8, b.qc, d, stream));
         ILW_TRY(ilwdetr_gemm_requant(memory, d, p->w_val, p->b_val, p->m_val, p->s_val, (int32_t)MS, d, d, 8, b.value, d,
                                      nullptr, stream));
         ILW_TRY(ilwdetr_gemm_requant(b.qc, d, p->w_off, p->b_off, p->m_off, p->s_off, M, 2 * HLP, d, 16, b.off16, 2 * HLP,
                                      nullptr, stream));
         ILW_TRY(ilwdetr_gemm_requant(b.qc, d, p->w_att, p->b_att, p->m_att, p->s_att, M, HLP, d, 16, b.att16, HLP, nullptr,
                                      stream));
-        // int16 -> int32 containers (rq with m = 2^30, s = 30 is the identity)
-        ILW_TRY(ilwdetr_requant(b.off16, 16, 2 * HLP, M, 2 * HLP, 1 << 30, 30, nullptr, 0, 1, 0, 1, 32, b.off32, 2 * HLP,
-                                stream));
-        ILW_TRY(ilwdetr_requant(b.att16, 16, HLP, M, HLP, 1 << 30, 30, nullptr, 0, 1, 0, 1, 32, b.att32, HLP, stream));
-        ILW_TRY(ilwdetr_shiftmax_rows(b.att32, LP, (int64_t)M * H, LP, &p->smx_w, b.w, LP, stream));
-        ILW_TRY(ilwdetr_deform_attn(b.value, level_hw, L, ref_q16, b.off32, b.w, B, Q, H, P, d / H, p->m_s, p->s_s, b.samp,
+        ilw::DeformParams dp;
+        ILW_TRY(deform_params(dp, b.value, level_hw, L, ref_q16, b.off32, b.w, B, Q, H, P, d / H, p->m_s, p->s_s, b.samp));
+        dp.off16 = b.off16;
+        dp.logits = b.att16;
+        cudaError_t de = cudaErrorNotSupported;
+        if (!g_check_only) {
+            dp.smx = make_smx(p->smx_w);
+            de = ilw::launch_deform_logits(dp, st);
+            if (de != cudaErrorNotSupported) ILW_LAUNCH(de, "decoder deform");
+        }
+        if (de != cudaSuccess) {
+            // (many sample points) int16 -> int32 containers (rq with m = 2^30, s = 30 is the identity)
+            ILW_TRY(ilwdetr_requant(b.off16, 16, 2 * HLP, M, 2 * HLP, 1 << 30, 30, nullptr, 0, 1, 0, 1, 32, b.off32, 2 * HLP,
                                     stream));
+            ILW_TRY(ilwdetr_requant(b.att16, 16, HLP, M, HLP, 1 << 30, 30, nullptr, 0, 1, 0, 1, 32, b.att32, HLP, stream));
+            ILW_TRY(ilwdetr_shiftmax_rows(b.att32, LP, (int64_t)M * H, LP, &p->smx_w, b.w, LP, stream));
+            ILW_TRY(ilwdetr_deform_attn(b.value, level_hw, L, ref_q16, b.off32, b.w, B, Q, H, P, d / H, p->m_s, p->s_s, b.samp,
+                                        stream));
+        }
         ilw_residual_t r2{b.t1, d, M, p->m_r2, p->s_r2};
         ILW_TRY(ilwdetr_gemm_requant(b.samp, d, p->w_o2, p->b_o2, p->m_o2, p->s_o2, M, d, d, 16, b.x2, d, &r2, stream));
-        ILW_TRY(ilwdetr_int_layernorm(b.x2, 16, d, M, d, p->ln2_beta, p->ln2_mult, p->ln2_shift, p->ln_iters, b.t2, 16, d,
-                                      stream));
+        if (g_check_only) {
+            ILW_TRY(ilwdetr_int_layernorm(b.x2, 16, d, M, d, p->ln2_beta, p->ln2_mult, p->ln2_shift, p->ln_iters, b.t2, 16, d,
+                                          stream));
+            ILW_TRY(ilwdetr_requant(b.t2, 16, d, M, d, p->m_f, p->s_f, nullptr, 0, 1, 0, 1, 8, b.fin, d, stream));
+        } else {
+            ilw::LnParams lp{b.x2, 16, d, M, d, p->ln2_beta, p->ln2_mult, p->ln2_shift, p->ln_iters, b.t2, 16, d,
+                             b.fin, d, nullptr, 0, p->m_f, p->s_f, 0, 1};
+            ILW_LAUNCH(ilw::launch_layernorm(lp, st), "decoder layernorm");
+        }
         // FFN
-        ILW_TRY(ilwdetr_requant(b.t2, 16, d, M, d, p->m_f, p->s_f, nullptr, 0, 1, 0, 1, 8, b.fin, d, stream));
         ILW_TRY(ilwdetr_gemm_gelu(b.fin, d, p->w_fc1, p->b_fc1, p->m_fc1, p->s_fc1, M, F, d, &p->gelu, p->m_g, p->s_g, b.h,
                                   F, stream));
         ilw_residual_t r3{b.t2, d, M, p->m_r3, p->s_r3};
         ILW_TRY(ilwdetr_gemm_requant(b.h, F, p->w_fc2, p->b_fc2, p->m_fc2, p->s_fc2, M, d, F, 16, b.x3, d, &r3, stream));
         return ilwdetr_int_layernorm(b.x3, 16, d, M, d, p->ln3_beta, p->ln3_mult, p->ln3_shift, p->ln_iters, out, 16, d,
                                      stream);
+#undef ILW_LAUNCH
 #undef ILW_TRY
     });
 }

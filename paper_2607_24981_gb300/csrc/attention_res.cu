@@ -972,7 +972,7 @@ cudaError_t launch_res(const ResArgs &a, int clusters, cudaStream_t s) {
 // The resident form: per-row s_d, which bounds sum P by 2^k_out and so |O| by 2^15 (with a static s_d
 // neither is bounded), scores of at most 64 columns (|s| <= 2^20) and at most 8 x 448 keys per group;
 // cudaErrorNotSupported otherwise.
-cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s) {
+cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, bool plan_only) {
     const ShiftExpC &se = p.smx.se;
     const bool win = p.nw > 1;
     const int ws = win ? p.grid_side / p.nw : 0, G2 = win ? p.nw * p.nw : 1;
@@ -998,6 +998,7 @@ cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s) {
     // (about 2300 keys, 8 images); it takes fp16-carried q|k|v with 64-column heads only
     const int64_t waves = (jobs + 2 * sm_count() - 1) / (2 * sm_count());
     if (p.qkv_f16 && p.dh == 64 && plan.cost > waves * Tg * 119) return cudaErrorNotSupported;
+    if (plan_only) return cudaSuccess;
     a.kpc = plan.kpc;
     a.rpc = plan.rpc;
     a.ws_rcp = ws > 1 ? (uint32_t)((((uint64_t)1 << 32) + ws - 1) / ws) : 0u;  // ws = 1: a window is one token

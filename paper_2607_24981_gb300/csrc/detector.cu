@@ -51,6 +51,12 @@ __global__ void __launch_bounds__(256) requant_kernel(const RequantParams p) {
                                      (uint32_t)(uint16_t)o[2] | ((uint32_t)(uint16_t)o[3] << 16));
         else
             *(int4 *)y = make_int4((int32_t)o[0], (int32_t)o[1], (int32_t)o[2], (int32_t)o[3]);
+        if (sizeof(TIn) == 2 && sizeof(TOut) == 1 && p.Y2) {
+            uint32_t w = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w |= (uint32_t)(uint8_t)sat8(rq(x[u], p.m3, p.s3)) << (8 * u);
+            *(uint32_t *)(p.Y2 + r * p.ldy2 + c) = w;
+        }
     }
 }
 

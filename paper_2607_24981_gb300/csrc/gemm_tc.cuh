@@ -336,7 +336,7 @@ __device__ __forceinline__ void epi_chunk(const EpiParams &ep, bool has_res, con
         }
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) out[i] = (KIND == KIND_RQ8 || KIND == KIND_F16OUT) ? clamp8(r[i]) : clamp16(r[i]);
+    for (int i = 0; i < 16; ++i) out[i] = (KIND == KIND_RQ8 || KIND == KIND_F16OUT) ? max(clamp8(r[i]), ep.relu ? 0 : -127) : clamp16(r[i]);
 }
 
 // Packed fp32 pairs (two operations an instruction).
@@ -374,11 +374,11 @@ __device__ __forceinline__ uint32_t half2_add(uint32_t a, uint32_t b) {
 // four int8, a word), w[0] on.  Saturating to [-127, 127] biased by 127 is one add-min-relu; the bias comes off with
 // a half2 subtract of 1151 from 1024 + u, or an add and an exclusive or per word (u + 1 never carries into
 // the next byte); two int16 are saturated and packed in one instruction, -32768 raised in another.
-// GELU kinds: sat16 indexes the table of values + 128 (gt points at the entry of -32767).
+// lo: the lowest int8 result, -127 or (ReLU) 0.  GELU kinds: sat16 indexes the table of values + 128 (gt points at the entry of -32767).
 template <int KIND>
 constexpr int out_words() { return KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16 ? 8 : 4; }
 template <int KIND>
-__device__ __forceinline__ void pack8(const int32_t (&r)[8], const uint8_t *gt, uint32_t *w) {
+__device__ __forceinline__ void pack8(const int32_t (&r)[8], const uint8_t *gt, int32_t lo, uint32_t *w) {
     if constexpr (KIND == KIND_RQ16) {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -389,7 +389,7 @@ __device__ __forceinline__ void pack8(const int32_t (&r)[8], const uint8_t *gt, 
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             if constexpr (gelu_kind(KIND)) u[i] = gt[__viaddmin_s32_relu(r[i], 32767, 65534)];
-            else u[i] = (uint32_t)__viaddmin_s32_relu(r[i], 127, 254);
+            else u[i] = (uint32_t)__viaddmin_s32_relu(max(r[i], lo), 127, 254);
         }
         if constexpr (out_words<KIND>() == 8) {
             // fp16 1024 + u, less 1151 (u biased by 127) or 1152 (the biased table)
@@ -518,6 +518,8 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
     constexpr int GPASS = (NSEG == 1 && RES == 0 && NG <= 2) ? NG : 1;
     static_assert(RES != 2 || (NG == 1 && KIND == KIND_RQ16), "one box holds the residual and the results");
     constexpr int esz = (KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16) ? 2 : (KIND == KIND_RAW32 ? 4 : 1);
+    const int32_t lo = ep.relu ? 0 : -127;           // of int8 results
+    const uint32_t lo_h = ep.relu ? 0u : 0xD7F0D7F0u;
     const int32_t r_rnd = RES != 0 ? 1 << (ep.s_r - 17) : 0, r_sh = RES != 0 ? ep.s_r - 16 : 0;
 #pragma unroll
     for (int g0 = 0; g0 < NG; g0 += GPASS) {
@@ -587,7 +589,7 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
                     const f32x2 d = add2(y, rr ^ 0x8000000080000000ull);
                     dmax = max_abs3(dmax, lo2(d), hi2(d));
                     asm("{.reg .b32 t;\n\tcvt.rn.f16x2.f32 t, %1, %2;\n\tmin.f16x2 t, t, %3;\n\tmax.f16x2 %0, t, %4;}"
-                        : "=r"(hw[j]) : "f"(hi2(rr)), "f"(lo2(rr)), "r"(0x57F057F0u), "r"(0xD7F0D7F0u));  // 127, -127
+                        : "=r"(hw[j]) : "f"(hi2(rr)), "f"(lo2(rr)), "r"(0x57F057F0u), "r"(lo_h));  // 127 and lo
                 }
                 if constexpr (KIND == KIND_F16OUT) {
 #pragma unroll
@@ -618,7 +620,7 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
 #pragma unroll
                             for (int i = 0; i < 8; ++i) r[i] = rq_clamped(r[i], cb[i], cm[i], col + i < ncol_all ? __ldg(ep.shift + col + i) : 33);
                         }
-                        pack8<KIND>(r, gt, w + e * out_words<KIND>() / 16);
+                        pack8<KIND>(r, gt, lo, w + e * out_words<KIND>() / 16);
                     }
                 }
                 emit(c, w);
@@ -690,7 +692,7 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
                             r[i] += rq_hi(xs, ep.m_r, r_rnd, r_sh);
                         }
                     }
-                    pack8<KIND>(r, gt, w + e * out_words<KIND>() / 16);
+                    pack8<KIND>(r, gt, lo, w + e * out_words<KIND>() / 16);
                     if constexpr (RES == 2) *unit = make_uint4(w[e / 2], w[e / 2 + 1], w[e / 2 + 2], w[e / 2 + 3]);
                 }
                 if constexpr (RES != 2) emit(c, w);

@@ -35,6 +35,38 @@ __global__ void __launch_bounds__(256) int_sigmoid_kernel(const int32_t *__restr
         Y[i] = int_sigmoid1(X[i], se, out_sh);
 }
 
+// requant_kernel's formula with the sigmoid of its result, 4 elements a thread: reference logits and boxes
+// (4 columns) in one launch instead of two or three.
+template <typename TOut>
+__global__ void __launch_bounds__(256) requant_sigmoid_kernel(const RequantParams p, int32_t *sig, int64_t ld_sig, ShiftExpC se,
+                                                              int32_t out_sh) {
+    grid_wait();
+    const int32_t cq = p.C >> 2;
+    const int64_t total = p.rows * cq;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = i / cq;
+        const int32_t c = (int32_t)(i - r * cq) * 4;
+        const int4 x4 = *(const int4 *)((const int32_t *)p.X + r * p.ldx + c);
+        const int32_t x[4] = {x4.x, x4.y, x4.z, x4.w};
+        const int16_t *z = p.Z ? p.Z + (r % p.z_rows) * p.ldz + c : nullptr;
+        int32_t o[4], g[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            int64_t v = rq(x[u], p.m1, p.s1);
+            if (z) v += rq(z[u], p.m2, p.s2);
+            o[u] = sizeof(TOut) == 2 ? sat16(v) : (int32_t)v;
+            g[u] = int_sigmoid1(o[u], se, out_sh);
+        }
+        TOut *y = (TOut *)p.Y + r * p.ldy + c;
+        if constexpr (sizeof(TOut) == 2)
+            *(uint2 *)y = make_uint2((uint32_t)(uint16_t)o[0] | ((uint32_t)(uint16_t)o[1] << 16),
+                                     (uint32_t)(uint16_t)o[2] | ((uint32_t)(uint16_t)o[3] << 16));
+        else
+            *(int4 *)y = make_int4(o[0], o[1], o[2], o[3]);
+        *(int4 *)(sig + r * ld_sig + c) = make_int4(g[0], g[1], g[2], g[3]);
+    }
+}
+
 // ReLU of int8 values, four per thread step (n4 words), then the tail
 __global__ void __launch_bounds__(256) relu_i8_kernel(const int8_t *__restrict__ X, int8_t *__restrict__ Y, int64_t n) {
     grid_wait();
@@ -277,6 +309,15 @@ cudaError_t launch_ivit_shiftgelu(const int32_t *X, int64_t ldx, int64_t rows, i
                                   const GeluC &c, cudaStream_t s) {
     if (rows == 0) return cudaSuccess;
     launch_after(ivit_shiftgelu_kernel, grid_for((rows + 7) / 8, 1), 256, 0, s, X, ldx, rows, L, Y, ldy, c.se, c.out_sh);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_requant_sigmoid(const RequantParams &p, int32_t *sig, int64_t ld_sig, const ShiftExpC &se, int32_t k_out,
+                                   cudaStream_t s) {
+    if (p.rows == 0 || p.C == 0) return cudaSuccess;
+    const unsigned g = grid_for(p.rows * (p.C / 4), 256);
+    if (p.out_bits == 16) launch_after(requant_sigmoid_kernel<int16_t>, g, 256, 0, s, p, sig, ld_sig, se, 32 - k_out);
+    else launch_after(requant_sigmoid_kernel<int32_t>, g, 256, 0, s, p, sig, ld_sig, se, 32 - k_out);
     return cudaGetLastError();
 }
 

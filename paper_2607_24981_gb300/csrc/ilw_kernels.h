@@ -99,6 +99,8 @@ struct EpiParams {
     // GELU (EPI_GELU): int8 output in C
     GeluC gelu;
     int32_t m_g, s_g;
+    // EPI_REQUANT with int8 outputs (also carried in fp16): max(., 0) of the result
+    int32_t relu;
 };
 
 // Packed weight layout: the same integers as fp16 [N, K] (row-major), the tensor-core operand.
@@ -130,6 +132,13 @@ struct LnParams {
     void *Y;
     int32_t out_bits;
     int64_t ldy;
+    // int16 in and out only: a second result Y2 = sat8(rq(y; m1, s1) + rq(Z; m2, s2)) of the normalised y
+    // (Z optional, [rows, ldz])
+    int8_t *Y2;
+    int64_t ldy2;
+    const int16_t *Z;
+    int64_t ldz;
+    int32_t m1, s1, m2, s2;
 };
 cudaError_t launch_layernorm(const LnParams &p, cudaStream_t s);
 
@@ -154,7 +163,8 @@ cudaError_t launch_attention(const AttnParams &p, cudaStream_t s);
 cudaError_t launch_attention_tc(const AttnParams &p, cudaStream_t s);
 // The form whose scores stay in tensor memory (groups of at most 2048 keys, per-row s_d; any q|k|v
 // carrier, dh 32 or 64); cudaErrorNotSupported when the problem is outside that.
-cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s);
+// plan_only: whether it would run (its sizes and parameters; no pointer is looked at)
+cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, bool plan_only = false);
 
 // ---------------------------------------------------------------- deformable sampling
 struct DeformParams {
@@ -168,7 +178,11 @@ struct DeformParams {
     int32_t B, Q, H, P, dh;
     int32_t m, s;
     int8_t *out;
+    // launch_deform_logits: the offsets as int16 and, instead of w, the int16 logits of its Shiftmax
+    const int16_t *off16, *logits;
+    ShiftmaxC smx;
 };
+cudaError_t launch_deform_logits(const DeformParams &p, cudaStream_t s);
 cudaError_t launch_deform(const DeformParams &p, cudaStream_t s);
 
 // ---------------------------------------------------------------- patch embedding
@@ -201,8 +215,14 @@ struct RequantParams {
     int32_t out_bits;    // 8, 16 (saturating) or 32
     void *Y;
     int64_t ldy;
+    int8_t *Y2;          // int16 in, int8 out only, optional: sat8(rq(X; m3, s3)), rows of ldy2
+    int64_t ldy2;
+    int32_t m3, s3;
 };
 cudaError_t launch_requant(const RequantParams &p, cudaStream_t s);
+// Y = the requantisation of p (int32 in, int16 or int32 out) and sig [rows, ld_sig] = its integer sigmoid
+cudaError_t launch_requant_sigmoid(const RequantParams &p, int32_t *sig, int64_t ld_sig, const ShiftExpC &se, int32_t k_out,
+                                   cudaStream_t s);
 cudaError_t launch_resample(const int8_t *X, int64_t x_bstride, int32_t B, int32_t Hi, int32_t Wi, int32_t C,
                             int8_t *Y, int64_t y_bstride, int32_t Ho, int32_t Wo, cudaStream_t s);
 // Attention heads of dh < 64 widened to 64 columns for the tensor-memory attention (zero columns

@@ -344,6 +344,22 @@ __device__ __forceinline__ void ln_store4_biased(TOut *y, const int32_t (&u)[4])
     }
 }
 
+// The second result of 4 normalised values y of a row.
+__device__ __forceinline__ void ln_second4(const LnParams &p, int64_t row, int c, const int32_t (&y)[4]) {
+    int64_t z[4] = {0, 0, 0, 0};
+    if (p.Z) {
+        const uint2 w = *(const uint2 *)(p.Z + row * p.ldz + c);
+        z[0] = rq((int16_t)(w.x & 0xFFFFu), p.m2, p.s2);
+        z[1] = rq((int16_t)(w.x >> 16), p.m2, p.s2);
+        z[2] = rq((int16_t)(w.y & 0xFFFFu), p.m2, p.s2);
+        z[3] = rq((int16_t)(w.y >> 16), p.m2, p.s2);
+    }
+    uint32_t w = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w |= (uint32_t)(uint8_t)sat8(rq(y[u], p.m1, p.s1) + z[u]) << (8 * u);
+    *(uint32_t *)(p.Y2 + row * p.ldy2 + c) = w;
+}
+
 // acc += a * b with a 64-bit accumulator in one wide multiply-add
 __device__ __forceinline__ void madw(int64_t &acc, int32_t a, int32_t b) {
     asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(a), "r"(b));
@@ -435,7 +451,8 @@ __device__ __noinline__ LnRow ln_row_general(int64_t S, int64_t Q, int32_t C, in
 // |y F| <= |y| (2^31 - 1) / R < 2^31 and y F fits int32; with shifts s >= 33 and |beta| <= 2^30 in every
 // column the requantisation is the high-word form (with a scalar rounding constant when the shifts are
 // the same); otherwise (or for rows with iters = 0 and V >= 2^32) the 64-bit formulas run.
-template <typename TIn, typename TOut, int LPR, int CPL, bool FULL>
+// SECOND: the second result of LnParams.
+template <typename TIn, typename TOut, int LPR, int CPL, bool FULL, bool SECOND = false>
 __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const LnConst lc) {
     grid_wait();
     extern __shared__ __align__(16) int32_t ln_par[];  // beta, mult, shift of CP columns
@@ -581,7 +598,14 @@ __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) o[u] = __viaddmin_s32_relu(o[u], LnBias<TOut>::one, 2 * LnBias<TOut>::one);
-                    if (FULL ? nc > 0 : LPR * i < nc) ln_store4_biased<TOut>(yr + LPR * i * EPC + u4, o);
+                    if (FULL ? nc > 0 : LPR * i < nc) {
+                        ln_store4_biased<TOut>(yr + LPR * i * EPC + u4, o);
+                        if constexpr (SECOND) {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) o[u] -= LnBias<TOut>::one;
+                            ln_second4(p, row, c0 + u4, o);
+                        }
+                    }
                 }
             }
         } else {
@@ -601,6 +625,7 @@ __global__ void __launch_bounds__(256, 3) layernorm_rows(const LnParams p, const
                     }
                     ln_norm4_exact(x, mu, F, be, mm, ss, LnOut<TOut>::bits, o);
                     ln_store4<TOut>(yr + LPR * i * EPC + u4, o);
+                    if constexpr (SECOND) ln_second4(p, row, c0 + u4, o);
                 }
             }
         }
@@ -684,7 +709,7 @@ LnConst ln_const(int iters, int C) {
 }
 
 template <typename TIn, typename TOut>
-cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
+cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s, bool &second) {
     const int eb = sizeof(TIn), ob = sizeof(TOut);
     const bool tiled = p.C % 4 == 0 && (p.C * eb) % 16 == 0 && (p.ldx * eb) % 16 == 0 && p.ldy % 4 == 0 &&
                        ((uintptr_t)p.X % 16) == 0 && ((uintptr_t)p.Y % (4 * ob)) == 0 &&
@@ -709,6 +734,13 @@ cudaError_t ln_dispatch(const LnParams &p, cudaStream_t s) {
         // chunks per lane: 6 for int16 rows (8 values each), 12 for int32 rows (4 values each), so a
         // lane holds at most 48 values; lanes per row from the row's chunk count
         constexpr int CPL = sizeof(TIn) == 2 ? 6 : 12;
+        if constexpr (sizeof(TIn) == 2 && sizeof(TOut) == 2 && LnOut<TOut>::bits == 16) {
+            if (p.Y2 && p.ldy2 % 4 == 0 && ((uintptr_t)p.Y2 % 4) == 0 && p.ldz % 4 == 0 && ((uintptr_t)p.Z % 8) == 0 && nch <= 16 * CPL) {
+                second = true;
+                if (nch <= 8 * CPL) return go(layernorm_rows<TIn, TOut, 8, CPL, false, true>, 8, CPL);
+                return go(layernorm_rows<TIn, TOut, 16, CPL, false, true>, 16, CPL);
+            }
+        }
         // (rows of 192 and 384 fill their lanes and need no test of a chunk against the row's end)
         if (nch == 4 * CPL) return go(layernorm_rows<TIn, TOut, 4, CPL, true>, 4, CPL);
         if (nch == 8 * CPL) return go(layernorm_rows<TIn, TOut, 8, CPL, true>, 8, CPL);
@@ -787,12 +819,16 @@ cudaError_t launch_sdshiftgelu(const int32_t *X, int32_t *Y, int64_t n, const Ge
 
 cudaError_t launch_layernorm(const LnParams &p, cudaStream_t s) {
     if (p.rows == 0) return cudaSuccess;
+    bool second = false;  // the launch wrote the second result
     if (p.out_bits == kOutI8InF16)
-        return p.in_bits == 16 ? ln_dispatch<int16_t, __half>(p, s) : ln_dispatch<int32_t, __half>(p, s);
-    if (p.in_bits == 16 && p.out_bits == 8) return ln_dispatch<int16_t, int8_t>(p, s);
-    if (p.in_bits == 16 && p.out_bits == 16) return ln_dispatch<int16_t, int16_t>(p, s);
-    if (p.in_bits == 32 && p.out_bits == 8) return ln_dispatch<int32_t, int8_t>(p, s);
-    return ln_dispatch<int32_t, int16_t>(p, s);
+        return p.in_bits == 16 ? ln_dispatch<int16_t, __half>(p, s, second) : ln_dispatch<int32_t, __half>(p, s, second);
+    if (p.in_bits == 16 && p.out_bits == 8) return ln_dispatch<int16_t, int8_t>(p, s, second);
+    if (p.in_bits == 32 && p.out_bits == 8) return ln_dispatch<int32_t, int8_t>(p, s, second);
+    if (p.in_bits == 32) return ln_dispatch<int32_t, int16_t>(p, s, second);
+    const cudaError_t e = ln_dispatch<int16_t, int16_t>(p, s, second);
+    if (e != cudaSuccess || !p.Y2 || second) return e;
+    RequantParams q{p.Y, 16, p.ldy, p.rows, p.C, p.m1, p.s1, p.Z, p.ldz, p.rows, p.m2, p.s2, 8, p.Y2, p.ldy2};
+    return launch_requant(q, s);
 }
 
 }  // namespace ilw

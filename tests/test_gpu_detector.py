@@ -72,6 +72,22 @@ def test_projector(ilw, orc):
     same(got, want, "projector memory")
 
 
+@pytest.mark.parametrize("d,H,levels,P,Q", [
+    (256, 4, [(9, 7)], 1, 50), (128, 4, [(12, 10), (6, 5)], 3, 33), (64, 2, [(8, 8)] * 8, 40, 17), (1024, 16, [(10, 8)], 4, 20)])
+def test_decoder_layer_shapes(ilw, orc, d, H, levels, P, Q):
+    """Heads of 32 and 64 columns, one sample point and more than the fused sampling takes, widths whose
+    I-LayerNorm does and does not write the next step's int8 rows itself."""
+    B, L, S = 2, len(levels), sum(h * w for h, w in levels)
+    dp = synth.decoder_params(3, 0, d=d, H=H, F=2 * d, L=L, P=P)
+    inp = synth.decoder_inputs(3, B, Q, d=d)
+    mem = synth.laplace_int(3, f"dec.mem{d}", (B * S, d), 20.0, 127, np.int8)
+    ws = torch.empty(ilw.decoder_workspace_bytes(B, Q, S, d, dp["F"], H, L, P), dtype=torch.uint8, device="cuda")
+    got = ilw.decoder_layer_forward(ilw.DecoderWeights(dp), dev(inp["tgt"]), dev(inp["pos"]), dev(mem), levels,
+                                    dev(inp["refs"]), B, Q, ws)
+    same(host(got), orc.decoder_layer(dp, inp["tgt"], inp["pos"], mem, levels, inp["refs"], B, Q), f"decoder d={d} H={H}")
+    ilw.device_status()
+
+
 @pytest.mark.parametrize("B,Q", [(2, 300), (1, 37)])
 def test_decoder_layer(ilw, orc, B, Q):
     cfg = synth.CONFIGS["medium_detector_b16"]

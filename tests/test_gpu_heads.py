@@ -83,6 +83,29 @@ def test_topk_selection(ilw, orc, rows, N, K, lo, hi):
     same(host(v), wv, f"topk values {rows}x{N} K={K}")
 
 
+@pytest.mark.parametrize("M,N,K,spread", [(300, 256, 256, 0), (33, 130, 64, 14), (130, 200, 1104, 0)])
+def test_gemm_relu(ilw, M, N, K, spread):
+    """The ReLU in the GEMM's epilogue against the two steps (float, per-column-shift and two-part forms)."""
+    A = dev(synth.uniform_int(5, f"gr{M}", (M, K), -127, 127, np.int8))
+    W, b, m, s = synth.gemm_params(5, f"gr{N}", N, K, 73.0, 40.0, "literal" if spread else "calibrated")
+    if spread:
+        s = (29 + np.arange(N) % spread).astype(s.dtype)
+    args = (A, ilw.pack_weight(dev(W)), N, dev(b), dev(m), dev(s))
+    want = ilw.relu_i8(ilw.gemm_requant(*args, 8))
+    assert torch.equal(ilw.gemm_relu(*args), want) and int(want.max()) > 0
+
+
+@pytest.mark.parametrize("rows,C,z_rows,out_bits", [(1, 4, 1, 16), (1000, 4, 1000, 32), (77, 12, 7, 16)])
+def test_requant_sigmoid(ilw, rows, C, z_rows, out_bits):
+    """One launch against the requantisation and the sigmoid of its result."""
+    X = dev(synth.uniform_int(5, f"rsx{rows}", (rows, C), -(1 << 24), 1 << 24, np.int32))
+    Z = dev(synth.uniform_int(5, f"rsz{rows}", (z_rows, C), -32767, 32767, np.int16))
+    sig = {"I0": 700, "k_inter": 8, "k_out": 17}
+    y = ilw.requant(X, 3 << 28, 36, Z, 3 << 28, 30, out_bits=out_bits)
+    got, box = ilw.requant_sigmoid(X, 3 << 28, 36, Z, 3 << 28, 30, sig, out_bits=out_bits)
+    assert torch.equal(got, y) and torch.equal(box, ilw.int_sigmoid(y.to(torch.int32), sig))
+
+
 def test_gather_rows_batched(ilw, orc):
     X = synth.uniform_int(77, "gatherb", (3 * 50, 8), -128, 127, np.int8)
     idx = synth.uniform_int(78, "gatherb.i", (3, 21), 0, 49)
