@@ -50,6 +50,9 @@ const uint8_t *gemm_gelu_table(const GeluC &c, int32_t m_g, int32_t s_g, cudaStr
 void gemm_debug_wait(int32_t *skip, long long *cycles);
 struct GemmProblem;
 struct EpiParams;
+// The 64-wide launch shapes (gemm_tc_n64.cu).
+template <bool AF16, bool GELU>
+cudaError_t run_n64(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s);
 // The int8-A launch shapes (gemm_tc_i8.cu): run<BN, STAGES, NB, false, false, GELU>.
 template <int BN, int STAGES, int NB, bool GELU>
 cudaError_t run_i8(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s);
@@ -715,7 +718,7 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
 // in registers before the accumulators are ready, and 16 warps hide the chains of their loads; with two
 // parts the epilogue of a projection tile took 4900 clocks), 192-wide tiles three of 64.
 template <int BN, bool AF16>
-constexpr int epi_parts() { return AF16 ? (BN == 192 ? 3 : 4) : 2; }
+constexpr int epi_parts() { return AF16 ? (BN == 192 ? 3 : BN / 32) : 2; }
 template <int BN, bool AF16>
 constexpr int epi_warps() { return 4 * epi_parts<BN, AF16>(); }
 template <int BN, bool AF16>
@@ -1360,7 +1363,7 @@ cudaError_t run(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s) {
     }
     // an int16 residual under int16 outputs by TMA, if its rows allow a map and no box wraps around
     tp.res_tma = 0;
-    if (tp.tma_store && ep.out_bits == 16 && ep.res && BN == 128 && AF16 && ((uintptr_t)ep.res % 16) == 0 && ep.ldr % 8 == 0 &&
+    if (tp.tma_store && ep.out_bits == 16 && ep.res && BN == 32 * epi_parts<BN, AF16>() && ((uintptr_t)ep.res % 16) == 0 && ep.ldr % 8 == 0 &&
         ep.res_rows < (1ll << 31) && (ep.res_rows >= gp.M || ep.res_rows % 32 == 0))
         tp.res_tma = gemm_make_map(&tp.rmap, ep.res, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, ep.res_rows, gp.N, ep.ldr, 32, 32,
                                    CU_TENSOR_MAP_SWIZZLE_64B)

@@ -411,6 +411,7 @@ def test_block_forward(ilw, orc, cfg):
 @pytest.mark.parametrize("M,N,K,out_bits,res_rows,mult", [
     (130, 384, 384, 16, 130, 0), (300, 384, 1536, 16, 300, 0), (97, 104, 128, 16, 32, 0), (200, 136, 256, 16, 50, 0),
     (33, 576, 384, 8, 0, 0), (257, 200, 1104, 8, 0, 0), (129, 1152, 384, 108, 0, 0), (64, 130, 64, 108, 0, 0),
+    (2500, 576, 384, 108, 0, 0), (2500, 584, 320, 8, 0, 0), (3300, 384, 1536, 16, 3300, 0),
     (140, 256, 256, 8, 0, 1 << 30), (140, 384, 320, 108, 0, 3 << 28), (70, 48, 192, 8, 70, 0)])
 @pytest.mark.parametrize("a_f16,spread", [(False, False), (True, False), (True, True), (False, True)])
 def test_gemm_epilogue_forms(ilw, orc, M, N, K, out_bits, res_rows, mult, a_f16, spread):
@@ -439,6 +440,21 @@ def test_gemm_epilogue_forms(ilw, orc, M, N, K, out_bits, res_rows, mult, a_f16,
     else:
         want = orc.gemm_requant(A, W, b, m, s, 8, None, 0, 0)
         assert_same(host(ilw.gemm(*args)), want, "int8")
+
+
+@pytest.mark.parametrize("M,N,K", [(2500, 576, 384), (2500, 1024, 256), (700, 1024, 256), (129, 200, 64)])
+@pytest.mark.parametrize("a_f16,out_bits", [(True, 108), (True, 8), (False, 8)])
+def test_gemm_gelu_widths(ilw, orc, M, N, K, a_f16, out_bits):
+    """SD-ShiftGELU through tiles of 192, 128 and 64 columns."""
+    A = synth.uniform_int(22, f"gw{M}{K}", (M, K), -127, 127, np.int8)
+    W, b, m, s = synth.gemm_params(22, f"gwW{N}{K}", N, K, 60.0, 900.0, "calibrated")
+    gelu = {"I0": 500, "k_inter": 16, "k_out": 8}
+    got = ilw.gemm(dev(A.astype(np.float16) if a_f16 else A), ilw.pack_weight(dev(W)), N, dev(b), dev(m), dev(s), out_bits,
+                   gelu=gelu, m_g=5 << 28, s_g=41)
+    h = orc.sdshiftgelu(orc.gemm_requant(A, W, b, m, s, 16), gelu["I0"]).astype(np.int64)
+    want = np.clip((h * (5 << 28) + (1 << 40)) >> 41, -127, 127)
+    assert_same(host(got), want, "gelu")
+    assert len(np.unique(want)) > 20
 
 
 # ------------------------------------------------------------- launches that overlap the one before
