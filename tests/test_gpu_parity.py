@@ -197,7 +197,7 @@ def test_int_layernorm(ilw, orc, C, in_bits, out_bits, iters):
 
 
 @pytest.mark.parametrize("rows,C,in_bits,out_bits,iters", [
-    (1, 192, 16, 8, 10), (33, 384, 32, 8, 10), (1030, 256, 32, 16, 4), (70, 384, 16, 16, 3), (65, 768, 16, 8, 16),
+    (1, 192, 16, 8, 10), (33, 384, 32, 8, 10), (1030, 256, 32, 16, 4), (70, 384, 16, 16, 3), (65, 768, 16, 8, 16), (91, 256, 16, 16, 10),
     (130, 512, 32, 8, 12)])
 def test_int_layernorm_row_forms(ilw, orc, rows, C, in_bits, out_bits, iters):
     """Neighbouring rows inside and outside the range of V whose root needs no Newton steps, rows with
