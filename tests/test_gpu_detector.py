@@ -53,6 +53,20 @@ def test_requant(ilw, orc, in_bits, out_bits, with_z):
     same(host(got), want, f"requant {in_bits}->{out_bits}")
 
 
+@pytest.mark.parametrize("rows,C,z_rows,s1,s2,out_bits", [
+    (5, 8, 5, 17, 17, 32), (77, 24, 7, 46, 17, 16), (1, 392, 1, 33, 46, 8), (301, 16, 0, 17, 1, 32), (301, 16, 0, 16, 1, 32),
+    (9, 12, 9, 30, 30, 8)])
+def test_requant_int16_forms(ilw, orc, rows, C, z_rows, s1, s2, out_bits):
+    """The ends of the 32-bit form's shifts, the row's ends of the int16 range, a shift below it and a width
+    that is no multiple of 8 (the general form)."""
+    X = synth.uniform_int(62, f"rf.x{rows}", (rows, C), -32768, 32767, np.int16)
+    X[0, :4] = [-32768, 32767, 0, -1]
+    Z = synth.uniform_int(62, f"rf.z{rows}", (z_rows, C), -32768, 32767, np.int16) if z_rows else None
+    for m in (2147483647, -2147483648, -1987654321):
+        got = ilw.requant(dev(X), m, s1, None if Z is None else dev(Z), 2147483647, s2, out_bits)
+        same(host(got), orc.requant(X, m, s1, Z, 2147483647, s2, out_bits), f"requant m={m} s={s1}")
+
+
 def test_resample_nearest(ilw, orc):
     B, g, C = 3, 40, 256
     X = synth.uniform_int(62, "rs.x", (B * g * g, C), -127, 127, np.int8)
