@@ -13,7 +13,7 @@
 // Split-convolution branches are segments too, each rescaled by its own dyadic (m_b, s_b)
 // before the integer sum.
 //
-// Persistent kernel, one CTA per SM, 128 x BN output tiles, 14 warps:
+// Persistent kernel, one CTA per SM, 128 x BN output tiles, 10 to 18 warps:
 //   warp 0      TMA producer: per K stage the activation tile (int8 128 x 64 bytes, or, when A is
 //               carried in fp16, the fp16 128 x 64 tile in the MMA's 128-byte swizzled layout) and
 //               the fp16 weight tile (BN x 64, 128-byte swizzle); with resident weights the CTA's
@@ -21,12 +21,13 @@
 //   warp 1      MMA issuer: 4 x (128 x BN x 16) MMAs per 64-wide K stage
 //   warps 2-5   operand converters (int8 A only): int8 activation rows (smem) -> fp16 rows in the
 //               same 128-byte swizzled K-major layout TMA produces for the weights
-//   warps 6-13  epilogue: TMEM -> registers -> integer epilogue -> HBM, one row per thread and
-//               half of the tile's columns per warp (fp16 A with 192-wide tiles: warps 2-13, a
-//               third of the columns each, since there is nothing to convert)
+//   the rest    epilogue (from warp 6, or with fp16 A from warp 2): TMEM -> registers -> integer or
+//               packed fp32 epilogue -> HBM, one row per thread and a part of the tile's columns per
+//               warp (epi_parts)
 // Two TMEM accumulator sets (when they fit) let the epilogue of tile i overlap the MMAs of tile
-// i+1.  With resident weights the grid is a multiple of the number of column blocks, so every
-// tile of a CTA uses the same BN rows of W and L2 serves only the activations.
+// i+1.  The grid is a multiple of the number of column blocks (with resident weights always, else where
+// that costs no round), so every tile of a CTA has the same columns: their parameters are prepared
+// once, and resident rows of W leave L2 only the activations to serve.
 // Every mbarrier wait is bounded (about one second); on expiry the kernel latches the device
 // status word, stops issuing work, drains the loads it issued and frees its TMEM.
 #include <cuda.h>
