@@ -54,6 +54,7 @@ struct EpiParams;
 // The 64-wide launch shapes (gemm_tc_n64.cu).
 template <bool AF16, bool GELU>
 cudaError_t run_n64(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s);
+cudaError_t run_n64_split(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s);
 // The int8-A launch shapes (gemm_tc_i8.cu): run<BN, STAGES, NB, false, false, GELU>.
 template <int BN, int STAGES, int NB, bool GELU>
 cudaError_t run_i8(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s);

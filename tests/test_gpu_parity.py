@@ -357,6 +357,21 @@ def test_split_conv(ilw, orc):
     assert_same(host(got), want, "split conv")
 
 
+@pytest.mark.parametrize("M,N,Ks,s_b", [(100, 64, (64,), [27]), (130, 200, (384, 80, 1024), [26, 33, 45]),
+                                        (9900, 136, (64, 128), [30, 28])])
+def test_split_conv_forms(ilw, orc, M, N, Ks, s_b):
+    """Tiles of 64 and 128 columns, ragged sizes, branch shifts from 26 on."""
+    Xs = [synth.uniform_int(19, f"sx{i}{M}", (M, k), -127, 127, np.int8) for i, k in enumerate(Ks)]
+    Ws = [synth.uniform_int(19, f"sw{i}{N}", (N, k), -127, 127, np.int8) for i, k in enumerate(Ks)]
+    Xs[0][0], Ws[0][0], Ws[0][1] = 127, 127, -127  # the largest accumulators
+    bias = synth.uniform_int(19, f"sb{N}", (N,), -(1 << 15), 1 << 15)
+    mult = synth.uniform_int(19, f"sm{N}", (N,), 1 << 30, (1 << 31) - 1)
+    shift = np.full(N, 45, np.int32)
+    m_b = [(1 << 24) + 12345 * i if s < 29 else 3 << 28 for i, s in enumerate(s_b)]
+    got = ilw.split_conv([dev(x) for x in Xs], [ilw.pack_weight(dev(w)) for w in Ws], N, m_b, s_b, dev(bias), dev(mult), dev(shift))
+    assert_same(host(got), orc.split_conv(Xs, Ws, m_b, s_b, bias, mult, shift), "split conv")
+
+
 # ------------------------------------------------------------------------------ deformable sampling
 def test_deform_attn(ilw, orc):
     B, Q, H, L, P, dh = 2, 300, 8, 3, 4, 32
