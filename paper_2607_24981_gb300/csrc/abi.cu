@@ -30,8 +30,9 @@ int fail(int code, const char *fmt, ...) {
 // ilwdetr_validate_only sets it for the calling thread until it is cleared again.
 thread_local bool g_check_only = false;
 struct CheckPass {
+    const bool before = g_check_only;
     CheckPass() { g_check_only = true; }
-    ~CheckPass() { g_check_only = false; }
+    ~CheckPass() { g_check_only = before; }
 };
 template <typename Body> int checked_then_run(Body body) {
     if (g_check_only) return body();  // inside another composite's checking pass
@@ -532,6 +533,7 @@ int ilwdetr_requant_sigmoid(const int32_t *X, int64_t ldx, int64_t rows, int32_t
     }
     if (rows == 0 || C == 0) return ILW_OK;
     if (ld_sig < C || ld_sig % 4) return fail(ILW_ERR_INVALID_ARG, "requant_sigmoid: ld_sig < C or not a multiple of 4");
+    if (g_check_only) return ILW_OK;
     ilw::RequantParams rp{X, 32, ldx, rows, C, m1, s1, Z, ldz, Z ? z_rows : 1, m2, Z ? s2 : 1, out_bits, Y, ldy};
     return cuda_status(ilw::launch_requant_sigmoid(rp, sig, ld_sig, ilw::make_shiftexp(p->I0, p->k_inter), p->k_out,
                                                    (cudaStream_t)stream),

@@ -192,7 +192,7 @@ cudaError_t launch_gemm(const GemmProblem &gp, const EpiParams &ep, cudaStream_t
     // 64-wide tiles where the chip holds all of them at once: such a call is one tile's chain of latencies
     // and its operands at 64 bytes a clock and SM, both shorter for half the columns, and twice the SMs work
     // on it (12 layers of 1600 x 192: 331 us with 128 and 192 wide tiles, 294 with these where they fit; a decoder
-    // layer of 1200 rows 112 and 102 us; the detector's split convolutions at 1 image 10 us less of 1131). 
+    // layer of 1200 rows 112 and 102 us; the detector's split convolutions at 1 image 10 us less of 1131).
     const int64_t tiles64 = (int64_t)((gp.M + BM - 1) / BM) * ((gp.N + 63) / 64);
     if (gp.nb > 1)
         return tiles64 <= num_sms() ? run_n64_split(gp, ep, s) : run_i8<128, 5, kMaxBranches, false>(gp, ep, s);

@@ -346,6 +346,21 @@ def test_oracle_sources_never_reach_the_product():
             assert needle not in text, (path, needle)
 
 
+def test_fused_entry_points_validate_only(validate_only):
+    """The fused steps check and launch nothing in validate-only mode, and leave the mode on."""
+    L = validate_only
+    import paper_2607_24981_gb300 as ilw
+
+    v, w = ctypes.c_void_p(0x100000), ctypes.c_void_p(0x200000)
+    sg = ctypes.byref(ilw.SigmoidT(1024, 8, 17))
+    for _ in range(2):  # the second call meets the mode the first one left
+        assert L.ilwdetr_requant_sigmoid(v, 4, 10, 4, 1 << 30, 30, None, 0, 1, 0, 1, 16, w, 4, sg, w, 4, None) == 0
+        assert L.ilwdetr_gemm_relu(v, 64, w, v, v, v, 100, 64, 64, v, 64, None) == 0
+        assert L.ilwdetr_gather_rows_batched(v, 64, 10, v, 3, 2, 64, w, 64, None) == 0
+    assert L.ilwdetr_requant_sigmoid(v, 4, 10, 4, 1 << 30, 30, None, 0, 1, 0, 1, 8, w, 4, sg, w, 4, None) != 0
+    assert L.ilwdetr_requant_sigmoid(v, 4, 10, 4, 1 << 30, 30, None, 0, 1, 0, 1, 16, w, 4, sg, w, 3, None) != 0
+
+
 def test_validate_only_mode_checks_without_launching(built_lib):
     """In validate-only mode every launching entry point runs its usual checks and returns ILW_OK
     (or the error found) without launching: valid calls on fake, aligned addresses succeed and bad
