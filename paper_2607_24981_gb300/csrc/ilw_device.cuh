@@ -16,8 +16,8 @@ constexpr uint32_t kInt31Max = 0x7fffffffu;
 // Every kernel is launched by launch_after, which lets it start as soon as the last CTA of the kernel
 // before it on the stream has ended, and calls grid_wait() before it touches global memory: that waits
 // until the earlier kernel's writes are visible.  So a launch, its barrier set-up and its tensor-memory
-// allocation overlap the end of the kernel before it (9 launches of a 256-token block: 88 us without,
-// 72 us with; a decoder layer of 26 launches 179 and 128 us).  No kernel lets its follower start before
+// allocation overlap the end of the kernel before it (7 launches of a 256-token block: 88 us without,
+// 72 us with; a decoder layer of 23 launches 179 and 128 us).  No kernel lets its follower start before
 // its own CTAs end (griddepcontrol.launch_dependents): that was slower, 79 and 130 us, and a follower on
 // the same SM could then find lines in L1 that were read before they were written.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
