@@ -549,12 +549,14 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
         // 16 columns out: the chunk's words
         auto emit = [&](int c, const uint32_t (&w)[out_words<KIND>()]) {
             if (box) {
-                // chunks 2 g and 2 g + 1 share a box; the store before the last one has read it (every
-                // group of columns commits, so that the count holds where columns past N store nothing)
+                // chunks 2 g and 2 g + 1 share a box, which an earlier store must have read: with two boxes the
+                // store before the last one, but where a part has an odd number of groups, the last one itself
+                // used the box of a tile's first group.  (Every group of columns commits, so that the count
+                // holds where columns past N store nothing.)
                 uint8_t *bx = box + (boxes == 2 ? ((c >> 1) & 1) * box_bytes<KIND>() : 0);
                 if ((c & 1) == 0) {
                     if (lane == 0) {
-                        if (boxes == 2) tma_store_wait_read1();
+                        if (boxes == 2 && !(NG % 2 != 0 && c == 0)) tma_store_wait_read1();
                         else tma_store_wait_read();
                     }
                     __syncwarp();
@@ -1279,7 +1281,8 @@ cudaError_t launch_tc(TcParams<NB> &tp, cudaStream_t s) {
     // TMA stores when the output allows them (set up by run) and their boxes fit next to the rest
     constexpr int stg = epi_warps<BN, AF16>() * box_bytes<KIND>();
     tp.stages = STAGES;
-    if (tp.tma_store) tp.tma_store = tp.res_tma ? 1 : 2;
+    // (a part of one group of columns stores once a tile, long after the last tile's store: one box)
+    if (tp.tma_store) tp.tma_store = tp.res_tma || BN == 32 * epi_parts<BN, AF16>() ? 1 : 2;
     auto bytes = [&](int boxes) { return smem_bytes<BN, STAGES, KIND, AF16, WRES>(tp.wres_bytes, boxes * stg, tp.stages); };
     // resident weights: as many stages as fit beside one box a warp (at least 3).  A's blocks come at L2's
     // latency, so the stages in flight set the rate: 12800 x 384 x 384 with 3 stages 600 clocks a K block

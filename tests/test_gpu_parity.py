@@ -457,6 +457,27 @@ def test_gemm_epilogue_forms(ilw, orc, M, N, K, out_bits, res_rows, mult, a_f16,
         assert_same(host(ilw.gemm(*args)), want, "int8")
 
 
+@pytest.mark.parametrize("M,N,K,a_f16,out_bits", [
+    (30000, 1152, 64, False, 8), (30000, 1536, 192, False, 8),  # three groups of 32 columns a warp
+    (14400, 576, 192, True, 108), (40000, 640, 192, True, 108), (40000, 640, 320, True, 8),  # one, resident weights
+    (40000, 256, 1104, True, 8)])                               # one, streamed weights
+def test_gemm_store_boxes_over_tiles(ilw, orc, M, N, K, a_f16, out_bits):
+    """Results stored through shared memory, an odd number of column groups in a warp's part of a tile and four or
+    more tiles a CTA, so that a store box is filled again while earlier stores may be under way: every element of
+    repeated calls (1000 distinct rows, repeated)."""
+    n = 1000
+    A = synth.uniform_int(23, f"sb{K}", (n, K), -127, 127, np.int8)
+    W, b, m, s = synth.gemm_params(23, f"sbW{N}{K}", N, K, 60.0, 30.0, "literal")
+    want = dev(orc.gemm_requant(A, W, b, m, s, 8, None, 0, 0).astype(np.float16 if out_bits == 108 else np.int8))
+    A_d = dev(A.astype(np.float16) if a_f16 else A).repeat(M // n + 1, 1)[:M].contiguous()
+    Wp, b, m, s = ilw.pack_weight(dev(W)), dev(b), dev(m), dev(s)
+    for _ in range(5):
+        got = ilw.gemm(A_d, Wp, N, b, m, s, out_bits)
+        for r in range(0, M, n):
+            assert torch.equal(got[r:r + n], want[:min(n, M - r)]), r
+    ilw.device_status()
+
+
 @pytest.mark.parametrize("M,N,K", [(2500, 576, 384), (2500, 1024, 256), (700, 1024, 256), (129, 200, 64)])
 @pytest.mark.parametrize("a_f16,out_bits", [(True, 108), (True, 8), (False, 8)])
 def test_gemm_gelu_widths(ilw, orc, M, N, K, a_f16, out_bits):

@@ -595,6 +595,28 @@ def test_gemm_resident_weight_grid(tiles_m, tiles_n, sms=152):
     assert (seen == 1).all()
 
 
+@pytest.mark.parametrize("boxes", [1, 2])
+@pytest.mark.parametrize("groups", [1, 2, 3])
+def test_gemm_store_box_never_still_being_read(groups, boxes, tiles=5):
+    """The GEMM epilogue's store boxes: a warp stores `groups` boxes a tile, group g from box g % boxes.  Before
+    it fills a box it waits until all of its stores, or all but the last (two boxes), have read theirs; that
+    one may still be reading the box of a tile's first group if the number of groups is odd, so there it
+    waits for all of them."""
+
+    def fills_unread(first_waits_for_all):
+        stores = []  # the boxes of the stores so far
+        for _ in range(tiles):
+            for g in range(groups):
+                left_out = 1 if boxes == 2 and not (first_waits_for_all and groups % 2 and g == 0) else 0
+                if g % boxes in stores[len(stores) - left_out:]:
+                    return True
+                stores.append(g % boxes)
+        return False
+
+    assert not fills_unread(True)
+    assert fills_unread(False) == (boxes == 2 and groups % 2 == 1)
+
+
 def test_layernorm_fast_normalisation_fits_int32():
     """I-LayerNorm's 32-bit normalisation: after at least one Newton step from 2^16 the iterate R is
     at least isqrt(V) >= |y| for every y = x - mu of the row, so F = floor((2^31 - 1) / R) gives
