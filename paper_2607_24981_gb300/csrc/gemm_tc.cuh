@@ -302,7 +302,8 @@ __device__ __forceinline__ int32_t rq_clamped(int32_t acc, int32_t bias, int32_t
 // The fused epilogue of 16 consecutive columns of one row, computed stage by stage so that the
 // 16 independent elements overlap.  FAST (uniform across the warp, decided per tile) says every
 // shift of the warp's columns is >= 33; ss then holds s - 32 and sr 2^(s-33) (rq_hi), else ss
-// holds s.  RFAST: the residual's shift s_r is >= 17.  gtab points at entry 0 of the SD-ShiftGELU output table (index -32767 .. 32767).
+// holds s.  RFAST: the residual's shift s_r is in [17, 46] (2^(s_r - 17) and |x m_r| 2^-16 add up within 32
+// bits).  gtab points at entry 0 of the SD-ShiftGELU output table (index -32767 .. 32767).
 template <int KIND, bool FAST, bool RFAST>
 __device__ __forceinline__ void epi_chunk(const EpiParams &ep, bool has_res, const uint32_t (&rp)[8],
                                           const int32_t (&acc)[16], const int32_t (&sb)[16],
@@ -333,11 +334,18 @@ __device__ __forceinline__ void epi_chunk(const EpiParams &ep, bool has_res, con
     }
     if (has_res) {
         // rp holds the 16 int16 residuals in pairs; x * 2^16 is the pair word masked or shifted
-        // (RFAST: rq(x; m_r, s_r) = rq(x * 2^16; m_r, s_r + 16) with s_r + 16 >= 33)
+        // (RFAST: rq(x; m_r, s_r) = rq(x * 2^16; m_r, s_r + 16) with s_r + 16 >= 33; both terms are then below
+        // 2^30 or saturate.  Else the sum is formed in 64 bits)
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int32_t xs = (i & 1) ? (int32_t)(rp[i >> 1] & 0xFFFF0000u) : (int32_t)(rp[i >> 1] << 16);
-            r[i] += RFAST ? rq_hi(xs, ep.m_r, 1 << (ep.s_r - 17), ep.s_r - 16) : (int32_t)rq((int64_t)(xs >> 16), ep.m_r, ep.s_r);
+            if (RFAST) {
+                r[i] += rq_hi(xs, ep.m_r, 1 << (ep.s_r - 17), ep.s_r - 16);
+            } else {
+                const int64_t t = (FAST ? (int64_t)r[i] : rq((int64_t)acc[i] + sb[i], sm[i], ss[i])) +
+                                  rq((int64_t)(xs >> 16), ep.m_r, ep.s_r);
+                r[i] = sat16(t);  // (int8 results saturate further below)
+            }
         }
     }
 #pragma unroll
@@ -467,7 +475,7 @@ __device__ __forceinline__ void tmem_wait_all(uint32_t (&v)[NSEG][16]) {
 // accumulators are read from TMEM in 32-column groups (all of them at once for one segment), so the
 // accumulator set is released to the MMA warp after the first wait, and the requantisation of the
 // 16-column chunks that follows has no TMEM latency left in it.  RES: the two-term residual form
-// (s_r >= 17); rp holds the residual pairs of group 0 (fetched by the caller while the MMAs ran), and
+// (17 <= s_r <= 46); rp holds the residual pairs of group 0 (fetched by the caller while the MMAs ran), and
 // each later group's pairs are fetched before its TMEM loads.  RES = 1: in registers; RES = 2: the residual is in
 // the warp's box already (by TMA, read back as 16 bytes a lane), and the results replace it there.
 //
@@ -965,7 +973,7 @@ __global__ void __launch_bounds__(tc_threads<BN, AF16>(), 1) gemm_tc_kernel(cons
         constexpr bool kFastKind = KIND == KIND_RQ8 || KIND == KIND_RQ16 || KIND == KIND_F16OUT || gelu_kind(KIND);
         constexpr bool kResKind = KIND == KIND_RQ8 || KIND == KIND_RQ16;  // kinds with a residual
         const int nseg = p.nseg, nld = (HALF / 16) * nseg;  // TMEM loads per tile
-        const bool has_res = ep.res != nullptr, rfast = has_res && ep.s_r >= 17;
+        const bool has_res = ep.res != nullptr, rfast = has_res && ep.s_r >= 17 && ep.s_r <= 46;
         bool fastw = false, one_shift = false;  // every shift >= 33; and the same
         int form = FORM_GENERAL;
         int32_t s_0 = 0;

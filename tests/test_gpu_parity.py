@@ -478,6 +478,23 @@ def test_gemm_store_boxes_over_tiles(ilw, orc, M, N, K, a_f16, out_bits):
     ilw.device_status()
 
 
+@pytest.mark.parametrize("s_r", [1, 16, 17, 46, 47, 48, 62])
+@pytest.mark.parametrize("M,N,a_f16", [(70, 200, False), (4000, 384, True)])  # 64-wide tiles, resident weights
+def test_gemm_residual_shifts(ilw, orc, M, N, a_f16, s_r):
+    """The residual's shift on both sides of the 32-bit form's range and at its ends, with the largest residuals and
+    multipliers of either sign; accumulators whose own term nears 2^31 where the shifts are small."""
+    A = synth.uniform_int(24, f"rs{M}", (M, 64), -127, 127, np.int8)
+    W, b, m, s = synth.gemm_params(24, f"rsW{N}", N, 64, 60.0, 9000.0, "literal")
+    res = synth.uniform_int(24, f"rsr{M}{N}", (M, N), -32768, 32767, np.int16)
+    res[:, :3] = [-32768, 32767, -1]
+    A_d, Wp, r_d = dev(A.astype(np.float16) if a_f16 else A), ilw.pack_weight(dev(W)), dev(res)
+    for out_bits in (8, 16):
+        for m_r, shift in ((1 << 30, s), (-(1 << 31), s), ((1 << 31) - 1, np.where(np.arange(N) % 2, 18, s).astype(s.dtype))):
+            want = orc.gemm_requant(A, W, b, m, shift, out_bits, res, m_r, s_r)
+            got = ilw.gemm(A_d, Wp, N, dev(b), dev(m), dev(shift), out_bits, res=r_d, m_r=m_r, s_r=s_r)
+            assert_same(host(got), want, f"out {out_bits} m_r={m_r} s_r={s_r}")
+
+
 @pytest.mark.parametrize("M,N,K", [(2500, 576, 384), (2500, 1024, 256), (700, 1024, 256), (129, 200, 64)])
 @pytest.mark.parametrize("a_f16,out_bits", [(True, 108), (True, 8), (False, 8)])
 def test_gemm_gelu_widths(ilw, orc, M, N, K, a_f16, out_bits):
