@@ -792,10 +792,12 @@ def gather_rows_batched(X, idx, out=None):
     import torch
 
     B, n = idx.shape
+    if B and X.shape[0] % B:
+        raise ValueError(f"gather_rows_batched: {X.shape[0]} rows are not {B} sources of equal size")
     rb = X.shape[1] * X.element_size()
     if out is None:
         out = torch.empty((B * n, X.shape[1]), dtype=X.dtype, device=X.device)
-    _check(lib().ilwdetr_gather_rows_batched(_ptr(X), X.stride(0) * X.element_size(), X.shape[0] // B, _ptr(idx), n, B, rb,
+    _check(lib().ilwdetr_gather_rows_batched(_ptr(X), X.stride(0) * X.element_size(), X.shape[0] // max(B, 1), _ptr(idx), n, B, rb,
                                              _ptr(out), out.stride(0) * out.element_size(), _stream()),
            "gather_rows_batched")
     return out

@@ -162,6 +162,20 @@ def test_two_stage(ilw, orc):
     same(host(boxes), wb, "reference boxes")
 
 
+def test_two_stage_without_images(ilw):
+    """An empty batch gives empty results, as an empty extent of any call does."""
+    levels = ((8, 8), (4, 4))
+    ts = ilw.TwoStage(synth.two_stage_params(9, d=64, C=16, levels=levels))
+    vals, idx, ref16, boxes = ts.forward(torch.empty((0, 64), dtype=torch.int8, device="cuda"), 0, 80, 10)
+    assert vals.shape == idx.shape == (0, 10) and ref16.shape == boxes.shape == (0, 4)
+
+
+def test_gather_rows_batched_refuses_unequal_sources(ilw):
+    X, idx = torch.zeros((101, 8), dtype=torch.int8, device="cuda"), torch.zeros((2, 3), dtype=torch.int32, device="cuda")
+    with pytest.raises(ValueError, match="equal size"):
+        ilw.gather_rows_batched(X, idx)
+
+
 @pytest.mark.parametrize("rows,L,I0,k_inter", [(300, 1536, 600, 16), (7, 1000, 1000, 8), (1, 5, 3, 16),
                                                (64, 64, 20000, 0)])
 def test_ivit_shiftgelu(ilw, orc, rows, L, I0, k_inter):
