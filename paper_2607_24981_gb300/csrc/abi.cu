@@ -656,10 +656,16 @@ int ilwdetr_decoder_layer_forward(const ilw_decoder_params_t *p, const int16_t *
                                      stream));
         ilw::AttnParams ap;
         ILW_TRY(attn_params(ap, b.qkv, b.qkv + d, b.qkv + 2 * d, 3 * d, 8, B, Q, H, d / H, 0, &p->smx, p->m_o, p->s_o, b.o, 8, d));
-        if (d / H < 64 && ilw::launch_attention_res(ap, st, true) == cudaErrorNotSupported) {
-            // heads of 32 columns that the resident attention does not take run on the streaming one of
-            // 64-column heads: q|k|v widened with zero columns (nothing added to q.k, zero outputs), the output
-            // narrowed back
+        // heads of 32 columns that the resident attention does not take run on the streaming one of
+        // 64-column heads: q|k|v widened with zero columns (nothing added to q.k, zero outputs), the output
+        // narrowed back.  The choice asks the device, so the checking pass checks both
+        bool widened = false;
+        if (d / H < 64 && !g_check_only) {
+            const cudaError_t e = ilw::launch_attention_res(ap, st, true);
+            if (e != cudaSuccess && e != cudaErrorNotSupported) return cuda_status(e, "decoder attention");
+            widened = e == cudaErrorNotSupported;
+        }
+        if (widened || (d / H < 64 && g_check_only)) {
             const int64_t w = (int64_t)H * 64;
             if (!g_check_only) {
                 cudaError_t e = ilw::launch_head_pad64(b.qkv, 3 * d, M, 3 * H, d / H, b.qkv64, (cudaStream_t)stream);
@@ -671,7 +677,8 @@ int ilwdetr_decoder_layer_forward(const ilw_decoder_params_t *p, const int16_t *
                 cudaError_t e = ilw::launch_head_compact(b.o64, w, M, H, d / H, b.o, d, (cudaStream_t)stream);
                 if (e != cudaSuccess) return cuda_status(e, "decoder head compact");
             }
-        } else {
+        }
+        if (!widened) {
             ILW_TRY(ilwdetr_shiftmax_attn(b.qkv, b.qkv + d, b.qkv + 2 * d, 3 * d, 8, B, Q, H, d / H, 0, &p->smx, p->m_o,
                                           p->s_o, b.o, 8, d, stream));
         }

@@ -4,6 +4,8 @@ are exercised up to the first CUDA call, which fails on a machine without a devi
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -243,6 +245,21 @@ def _composite_checks(ilw, L):
     assert patch() == 0
     assert patch(Wp=0x200010) == -1 and b"256-byte" in L.ilwdetr_last_error()  # the GEMM's check, before the gather
     assert patch(s_pos=63) == -1 and b"residual" in L.ilwdetr_last_error()
+
+
+@pytest.mark.skipif(not sys.platform.startswith("linux"), reason="reads the dynamic linker's log")
+def test_validation_never_asks_for_a_device(built_lib, tmp_path):
+    """Validating the composite calls (a decoder with heads of 32 among them) makes no CUDA call: the runtime never
+    loads the driver, which its first call that needs a device does, as the linker's log shows."""
+    code = ("import ctypes, sys; sys.path[:0] = %r\n"
+            "import paper_2607_24981_gb300 as ilw, test_abi_exports as t\n"
+            "L = ilw.lib(); L.ilwdetr_validate_only(1); t._composite_checks(ilw, L)\n"
+            % [ROOT, os.path.join(ROOT, "tests")])
+    env = dict(os.environ, LD_DEBUG="libs", LD_DEBUG_OUTPUT=str(tmp_path / "ld"))
+    r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stderr[-2000:]
+    log = "".join(open(p).read() for p in tmp_path.iterdir())
+    assert "libilwdetr.so" in log and "libcuda.so" not in log
 
 
 def test_int8_tcgen05_mma_is_not_available_on_sm103a(tmp_path):
