@@ -1,6 +1,8 @@
 """Bit-exact parity of every CUDA entry point with the CPU oracle, element by element, on seeded
 inputs that span several tiles plus ragged tails, and on the edge cases of each operator.
 The whole path is integer, so the tolerance is zero everywhere."""
+import time
+
 import numpy as np
 import pytest
 
@@ -301,6 +303,27 @@ def test_attention_extreme_scores(ilw, orc):
     smx = {"I0": 1 << 14, "k_inter": 16, "k_out": 8, "s_d": -1, "m_p": 4, "M_hw": 31}
     got = ilw.shiftmax_attn(dev(qkv), B, T, H, dh, 0, smx, 1 << 30, 33)
     assert_same(host(got), orc.attention(qkv, B, T, H, dh, 0, smx, 1 << 30, 33), "attn extreme")
+
+
+def test_int_layernorm_host_time_does_not_depend_on_steps(ilw):
+    """The search for the roots that need no Newton steps (long at 10 steps, short at 20) is not part of a call: 200
+    calls of a short kernel take the host as long at either count (the best of 10; 14.5 and 10.2 us a call with
+    the search in each)."""
+    x = torch.zeros((16, 192), dtype=torch.int16, device="cuda")
+    out = torch.empty((16, 192), dtype=torch.int8, device="cuda")
+    ln = [dev(a) for a in synth.ln_params(7, "lnhost", 192)]
+
+    def best(iters):
+        t = []
+        for _ in range(11):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            for _ in range(200):
+                ilw.int_layernorm(x, *ln, iters, 8, out=out)
+            t.append(time.perf_counter() - t0)
+        return min(t[1:])
+
+    assert best(10) < 1.2 * best(20)
 
 
 @pytest.mark.parametrize("B,T,H,dh,win,form", [
