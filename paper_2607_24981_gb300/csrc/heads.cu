@@ -1,6 +1,7 @@
 // heads.cu -- the detection head's elementwise and selection kernels: integer sigmoid (the head's
 // exponential by ShiftExp, Table 5, in SD-ShiftGELU's sign-dependent sigmoid form, Sec. 3.3.1 and
 // Algorithm 1), ReLU on int8, per-row integer top-K (two-stage query selection) and row gather.
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 
@@ -81,40 +82,89 @@ __global__ void __launch_bounds__(256) relu_i8_kernel(const int8_t *__restrict__
         Y[i] = X[i] < 0 ? (int8_t)0 : X[i];
 }
 
-// Per-row top-K, one CTA per row, ties to the lower index.  Bound by latency (a row's 33 KB at 8400
-// values are nothing): sorting the whole padded row took 105 steps over 16384 keys, 211 us; selecting
-// first leaves K keys to order.  Thread t holds values t VPT .. (VPT of them) in registers.
+// Per-row top-K, ties to the lower index: T threads (a multiple of 32) work on a row.  Bound by latency (a
+// row's 33 KB at 8400 values are nothing) and, for many short rows, by the threads a row holds.  Sorting the
+// whole padded row takes 105 steps over 16384 keys, 207 us for 8 rows of 8400; selecting first leaves K keys to
+// order, 15 us.  Thread t of a row holds values t VPT .. (VPT of them) in registers.
 //   1. the K-th largest value, found bit by bit below the row's maximum: every step counts the values at
-//      or above a candidate over the CTA;
+//      or above a candidate over the row;
 //   2. a scan over the threads gives every value above it its place among the selected, and the values
 //      equal to it, in index order, the places left;
-//   3. the selected keys (value, lower index first) are ordered by counting the larger ones for
-//      K <= kRankMax, else by a bitonic sort of the K keys.
+//   3. the selected keys (value, lower index first) are ordered by counting the larger ones where that is
+//      little work a thread (K <= kRankMax for a whole CTA, else K^2 <= kRankWork T), else by a bitonic sort of the K keys.
+// Where K pads to the same power of two as the row does there is nothing to select: topk_sort_kernel.
+// A row takes the whole CTA, or a CTA of up to 256 threads takes 256 / T rows.
 // Keys: (value biased to unsigned) << 32 | (2^32 - 1 - index), so one descending order puts larger
 // values first and, for equal values, smaller indices first.  Padding keys are 0, below every real key.
 constexpr int kTopkThreads = 1024;
 constexpr int kRankMax = 512;
-template <int VPT>
-__global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t N,
-                                                            int32_t kpad, int32_t K, int32_t *__restrict__ vals,
+constexpr int kRankWork = 512;  // (4000 rows: 300 of 2000, T 256, 145 us against 185; 2000 rows: 500 of 2500, T 288, 146 against 107)
+enum { kCta = 0, kWarp = 1, kWarps = 2 };  // a row's threads: the whole CTA, a warp, some warps of the CTA
+// The T threads of a row meet (kWarps: each of the CTA's rows has a barrier of its own).
+template <int ROW>
+__device__ __forceinline__ void row_sync(int slot, int T) {
+    if (ROW == kCta) __syncthreads();
+    else if (ROW == kWarp) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "r"(T) : "memory");
+}
+__device__ __forceinline__ unsigned long long topk_key(uint32_t biased, int i) {
+    return ((unsigned long long)biased << 32) | (0xFFFFFFFFu - (uint32_t)i);
+}
+// Result `at` of a row from its key
+struct TopkOut {
+    int32_t *vals, *idx;  // of the row
+    __device__ __forceinline__ void put(int at, unsigned long long key) const {
+        vals[at] = (int32_t)((uint32_t)(key >> 32) ^ 0x80000000u);
+        idx[at] = (int32_t)(0xFFFFFFFFu - (uint32_t)key);
+    }
+};
+// Orders kpad keys by T threads, largest first, and writes the first K
+template <int ROW>
+__device__ __forceinline__ void topk_sort(unsigned long long *keys, int kpad, int K, int tid, int T, int slot, const TopkOut &out) {
+    for (int k = 2; k <= kpad; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int i = tid; i < kpad; i += T) {
+                const int ixj = i ^ j;
+                if (ixj > i) {
+                    const unsigned long long a = keys[i], b = keys[ixj];
+                    if (((i & k) == 0) ? (a < b) : (a > b)) {
+                        keys[i] = b;
+                        keys[ixj] = a;
+                    }
+                }
+            }
+            row_sync<ROW>(slot, T);
+        }
+    for (int i = tid; i < K; i += T) out.put(i, keys[i]);
+}
+
+template <int VPT, int ROW>
+__global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t rows, int32_t N,
+                                                            int32_t threads, int32_t kpad, int32_t K, int32_t *__restrict__ vals,
                                                             int32_t *__restrict__ idx) {
     grid_wait();
-    extern __shared__ unsigned long long keys[];  // kpad
-    __shared__ uint32_t part[2][32];
-    const int32_t *s = S + (int64_t)blockIdx.x * lds;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, i0 = tid * VPT;
+    extern __shared__ unsigned long long topk_keys[];  // kpad a row
+    __shared__ uint32_t parts[2][32];                  // a value per warp
+    const int T = ROW == kCta ? kTopkThreads : (ROW == kWarp ? 32 : threads), slot = ROW == kCta ? 0 : threadIdx.x / T, tid = threadIdx.x - slot * T, W = T >> 5;
+    const int64_t row = ROW == kCta ? blockIdx.x : (int64_t)blockIdx.x * (blockDim.x / T) + slot;
+    if (row >= rows) return;  // (all of the row's threads)
+    const int32_t *s = S + row * lds;
+    unsigned long long *keys = topk_keys + slot * kpad;
+    uint32_t *part0 = parts[0] + slot * W, *part1 = parts[1] + slot * W;
+    const int warp = tid >> 5, lane = tid & 31, i0 = tid * VPT;
     // biased values; past the row 0, which step 2 never selects (it is told apart by its index)
     uint32_t v[VPT];
 #pragma unroll
     for (int j = 0; j < VPT; ++j) v[j] = i0 + j < N ? (uint32_t)s[i0 + j] ^ 0x80000000u : 0u;
-    // the CTA's sum of one value per thread (alternating buffers: one barrier per call)
+    // the row's sum of one value per thread (alternating buffers: one barrier per call)
     int buf = 0;
-    auto cta_sum = [&](uint32_t x) -> uint32_t {
+    auto row_sum = [&](uint32_t x) -> uint32_t {
         x = __reduce_add_sync(0xffffffffu, x);
-        if (lane == 0) part[buf][warp] = x;
-        __syncthreads();
-        x = __reduce_add_sync(0xffffffffu, part[buf][lane]);
-        buf ^= 1;
+        if (W == 1) return x;
+        if (lane == 0) part0[buf + warp] = x;
+        row_sync<ROW>(slot, T);
+        x = __reduce_add_sync(0xffffffffu, lane < W ? part0[buf + lane] : 0u);
+        buf ^= 32;
         return x;
     };
     // bits above the highest in which the row's values differ are the maximum's
@@ -127,14 +177,16 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__res
         }
     hi = __reduce_max_sync(0xffffffffu, hi);
     lo = __reduce_min_sync(0xffffffffu, lo);
-    if (lane == 0) {
-        part[0][warp] = hi;
-        part[1][warp] = lo;
+    if (W > 1) {
+        if (lane == 0) {
+            part0[warp] = hi;
+            part1[warp] = lo;
+        }
+        row_sync<ROW>(slot, T);
+        hi = __reduce_max_sync(0xffffffffu, lane < W ? part0[lane] : 0u);
+        lo = __reduce_min_sync(0xffffffffu, lane < W ? part1[lane] : 0xffffffffu);
+        row_sync<ROW>(slot, T);
     }
-    __syncthreads();
-    hi = __reduce_max_sync(0xffffffffu, part[0][lane]);
-    lo = __reduce_min_sync(0xffffffffu, part[1][lane]);
-    __syncthreads();
     // thr: the largest value with at least K values at or above it (that many are at or above `lo`)
     const int top = 32 - __clz(hi ^ lo);
     uint32_t thr = top == 32 ? 0u : hi >> top << top;
@@ -143,7 +195,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__res
         uint32_t c = 0;
 #pragma unroll
         for (int j = 0; j < VPT; ++j) c += (i0 + j < N && v[j] >= cand) ? 1u : 0u;
-        if (cta_sum(c) >= (uint32_t)K) thr = cand;
+        if (row_sum(c) >= (uint32_t)K) thr = cand;
     }
     // places: (values above thr) << 16 | (values equal to it), summed over the threads before this one
     uint32_t c = 0;
@@ -156,11 +208,11 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__res
         const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
-    __syncthreads();
-    if (lane == 31) part[0][warp] = incl;
-    for (int i = K + tid; i < kpad; i += kTopkThreads) keys[i] = 0ull;
-    __syncthreads();
-    const uint32_t w = part[0][lane];
+    row_sync<ROW>(slot, T);
+    if (lane == 31) part0[warp] = incl;
+    for (int i = K + tid; i < kpad; i += T) keys[i] = 0ull;
+    row_sync<ROW>(slot, T);
+    const uint32_t w = lane < W ? part0[lane] : 0u;
     const uint32_t total = __reduce_add_sync(0xffffffffu, w);
     uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? w : 0u) + incl - c;
     const uint32_t above = total >> 16;
@@ -169,42 +221,42 @@ __global__ void __launch_bounds__(kTopkThreads) topk_kernel(const int32_t *__res
     for (int j = 0; j < VPT; ++j) {
         if (i0 + j >= N || v[j] < thr) continue;
         const uint32_t pos = v[j] > thr ? pg++ : pe++;
-        if (pos < (uint32_t)K) keys[pos] = ((unsigned long long)v[j] << 32) | (0xFFFFFFFFu - (uint32_t)(i0 + j));
+        if (pos < (uint32_t)K) keys[pos] = topk_key(v[j], i0 + j);
     }
-    __syncthreads();
-    auto put = [&](int at, unsigned long long key) {
-        vals[(int64_t)blockIdx.x * K + at] = (int32_t)((uint32_t)(key >> 32) ^ 0x80000000u);
-        idx[(int64_t)blockIdx.x * K + at] = (int32_t)(0xFFFFFFFFu - (uint32_t)key);
-    };
-    if (K <= kRankMax) {
-        // 2 threads (adjacent lanes) per key, each over half of the keys: its place is the number of larger ones
-        const int e = tid >> 1, h = tid & 1;
-        if (e - (lane >> 1) < K) {  // the warp has a key
-            const unsigned long long key = e < K ? keys[e] : ~0ull;
-            const int half = (K + 1) >> 1, b = h * half, n = h ? K - half : half;
-            int rank = 0;
-#pragma unroll 8
-            for (int i = 0; i < n; ++i) rank += keys[b + i] > key ? 1 : 0;
-            rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-            if (e < K && h == 0) put(rank, key);
-        }
+    row_sync<ROW>(slot, T);
+    const TopkOut out{vals + row * K, idx + row * K};
+    if (ROW == kCta ? K > kRankMax : K * K > kRankWork * T) {
+        topk_sort<ROW>(keys, kpad, K, tid, T, slot, out);
         return;
     }
-    for (int k = 2; k <= kpad; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = tid; i < kpad; i += kTopkThreads) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const unsigned long long a = keys[i], b = keys[ixj];
-                    if (((i & k) == 0) ? (a < b) : (a > b)) {
-                        keys[i] = b;
-                        keys[ixj] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
-    for (int i = tid; i < K; i += kTopkThreads) put(i, keys[i]);
+    // 2 threads (adjacent lanes) per key, each over half of the keys: its place is the number of larger ones
+    for (int e2 = tid; (e2 - lane) >> 1 < K; e2 += T) {  // while the warp has a key
+        const int e = e2 >> 1, h = e2 & 1;
+        const unsigned long long key = e < K ? keys[e] : ~0ull;
+        const int half = (K + 1) >> 1, b = h * half, n = h ? K - half : half;
+        int rank = 0;
+#pragma unroll 8
+        for (int i = 0; i < n; ++i) rank += keys[b + i] > key ? 1 : 0;
+        rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+        if (e < K && h == 0) out.put(rank, key);
+    }
+}
+
+// The same where every value of the (padded) row is ordered.
+template <int ROW>
+__global__ void __launch_bounds__(kTopkThreads) topk_sort_kernel(const int32_t *__restrict__ S, int64_t lds, int32_t rows, int32_t N,
+                                                                 int32_t threads, int32_t kpad, int32_t K, int32_t *__restrict__ vals,
+                                                                 int32_t *__restrict__ idx) {
+    grid_wait();
+    extern __shared__ unsigned long long topk_keys[];
+    const int T = ROW == kCta ? blockDim.x : (ROW == kWarp ? 32 : threads), slot = ROW == kCta ? 0 : threadIdx.x / T, tid = threadIdx.x - slot * T;
+    const int64_t row = ROW == kCta ? blockIdx.x : (int64_t)blockIdx.x * (blockDim.x / T) + slot;
+    if (row >= rows) return;
+    const int32_t *s = S + row * lds;
+    unsigned long long *keys = topk_keys + slot * kpad;
+    for (int i = tid; i < kpad; i += T) keys[i] = i < N ? topk_key((uint32_t)s[i] ^ 0x80000000u, i) : 0ull;
+    row_sync<ROW>(slot, T);
+    topk_sort<ROW>(keys, kpad, K, tid, T, slot, TopkOut{vals + row * K, idx + row * K});
 }
 
 // K = 1: one warp per row keeps the largest value with the smallest index among its columns, and
@@ -336,17 +388,32 @@ cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, 
     }
     int kpad = 2;
     while (kpad < K) kpad <<= 1;
-    const size_t smem = (size_t)kpad * 8;
-    auto go = [&](auto kern, SmemLimit &limit) -> cudaError_t {
+    if (N <= 32)  // too little to select from: 134400 rows, 4 of 16, 65 us, 113 with the selection
+        while (kpad < N) kpad <<= 1;
+    auto go = [&](auto kern, SmemLimit &limit, int threads, int per) -> cudaError_t {  // per: rows of a CTA
         const cudaError_t e = raise_smem_limit(limit, (const void *)kern, 16384 * 8);
         if (e != cudaSuccess) return e;
-        launch_after(kern, (unsigned)rows, kTopkThreads, smem, s, S, lds, N, kpad, K, vals, idx);
+        launch_after(kern, (unsigned)(((int64_t)rows + per - 1) / per), per * threads, (size_t)per * kpad * 8, s, S, lds, rows, N,
+                     threads, kpad, K, vals, idx);
         return cudaGetLastError();
     };
-    static SmemLimit l2, l9, l16;
-    if (N <= 2 * kTopkThreads) return go(topk_kernel<2>, l2);
-    if (N <= 9 * kTopkThreads) return go(topk_kernel<9>, l9);  // the detector's 8400 memory tokens
-    return go(topk_kernel<16>, l16);
+    static SmemLimit sw, s1, s8, w2, w9, w16, n2, n4, n8;
+    if (kpad >= N) {
+        const int threads = std::min(std::max(kpad / 2, 32), kTopkThreads);
+        if (threads == 32) return go(topk_sort_kernel<kWarp>, sw, 32, 8);
+        return threads < 256 ? go(topk_sort_kernel<kWarps>, s8, threads, 256 / threads) : go(topk_sort_kernel<kCta>, s1, threads, 1);
+    }
+    // A whole CTA per row for long rows (the detector's 8400 memory tokens), and for shorter ones while the chip
+    // holds all of them at once; where it does not, and for the shortest always, as few threads as hold the
+    // row.  (A CTA per row and this: 134400 rows, 5 of 80, 3926 us and 113; 20000, 100 of 512, 633 and 135; one row of 80
+    // 7.4 and 3.5; 8 rows, 100 of 300, 7.9 and 10.4, and 1000 rows, 300 of 8400, 103 and 117, which stay.)
+    auto threads = [&](int vpt) { return (N + 32 * vpt - 1) / (32 * vpt) * 32; };
+    if (N <= 64) return go(topk_kernel<2, kWarp>, n2, 32, 8);
+    if (N <= 128) return go(topk_kernel<4, kWarp>, n4, 32, 8);
+    if (N <= 2048 && rows > 2 * sm_count()) return go(topk_kernel<8, kWarps>, n8, threads(8), std::max(256 / threads(8), 1));
+    if (N <= 2 * kTopkThreads) return go(topk_kernel<2, kCta>, w2, kTopkThreads, 1);
+    if (N <= 9 * kTopkThreads) return go(topk_kernel<9, kCta>, w9, kTopkThreads, 1);
+    return go(topk_kernel<16, kCta>, w16, kTopkThreads, 1);
 }
 
 cudaError_t launch_gather_rows(const void *src, int64_t src_ld_bytes, int64_t src_rows, const int32_t *idx, int64_t n,

@@ -83,6 +83,42 @@ def test_topk_selection(ilw, orc, rows, N, K, lo, hi):
     same(host(v), wv, f"topk values {rows}x{N} K={K}")
 
 
+@pytest.mark.parametrize("rows,N,K", [
+    (1, 2, 2), (9, 31, 3), (1000, 32, 5), (17, 33, 2), (1003, 64, 32), (1001, 65, 32), (3, 80, 5), (2049, 128, 64), (1000, 128, 65),
+    (305, 129, 64), (610, 256, 100), (611, 257, 128), (400, 1000, 181), (400, 1000, 182), (310, 2048, 362), (310, 2048, 363),
+    (310, 2048, 1024), (310, 2047, 1025), (304, 2048, 500), (12, 512, 512), (5, 5000, 4097)])
+def test_topk_rows_of_a_cta(ilw, orc, rows, N, K):
+    """Rows of one and of several warps, several of them a CTA (the last CTA part empty), K on both sides of where
+    counting, sorting the selected and sorting the row meet; every third row has few values."""
+    S = synth.uniform_int(79, f"topkr{rows}.{N}", (rows, N), -(1 << 31), (1 << 31) - 1)
+    S[::3] %= 3
+    v, i = ilw.topk(dev(S), K)
+    wv, wi = orc.topk(S, K)
+    same(host(i), wi, f"topk idx {rows}x{N} K={K}")
+    same(host(v), wv, f"topk values {rows}x{N} K={K}")
+
+
+def test_topk_short_rows_take_no_longer_than_long_ones(ilw):
+    """The same number of values in rows of 80 and of 8400 (113 and 106 us measured): short rows do not hold a whole
+    CTA each, which took 30 times as long."""
+
+    def us(rows, N):
+        S = torch.randint(-(1 << 20), 1 << 20, (rows, N), dtype=torch.int32, device="cuda")
+        v, i = ilw.topk(S, 5)
+        t = []
+        for _ in range(5):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            for _ in range(5):
+                ilw.topk(S, 5, v, i)
+            b.record()
+            torch.cuda.synchronize()
+            t.append(a.elapsed_time(b) * 200)
+        return min(t)
+
+    assert us(105 * 1280, 80) < 4 * us(1280, 8400)
+
+
 @pytest.mark.parametrize("M,N,K,spread", [(300, 256, 256, 0), (33, 130, 64, 14), (130, 200, 1104, 0)])
 def test_gemm_relu(ilw, M, N, K, spread):
     """The ReLU in the GEMM's epilogue against the two steps (float, per-column-shift and two-part forms)."""
