@@ -194,11 +194,17 @@ __device__ __forceinline__ void tst8(uint32_t taddr, const uint32_t (&v)[8]) {
                  : "memory");
 }
 __device__ __forceinline__ void twait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// D += A B with A in TMEM (fp16 pairs: column c holds K elements 2c and 2c + 1 of the lane's row)
-__device__ __forceinline__ void mma_ts(uint32_t dt, uint32_t at, uint64_t b, uint32_t idesc, uint32_t acc) {
+// D += A B with A in TMEM (fp16 pairs: column c holds K elements 2c and 2c + 1 of the lane's row), if `on`: a
+// predicate on the instruction, so that every MMA of the issuer stands in the one flat branch of the elected lane.
+// A branch of its own around an MMA inside that one (an earlier form of the loop) issued some MMAs with the operands
+// of another step.  Why has not been shown; the operands of an MMA are read from uniform registers, which a
+// branch within a one-lane branch has to fill again.  (A predicate in place of the elected lane's branch as
+// well, as in the GEMM: 8 images of the Medium encoder 1958 us against 1914.)
+__device__ __forceinline__ void mma_ts(uint32_t dt, uint32_t at, uint64_t b, uint32_t idesc, uint32_t acc, uint32_t on) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dt),
-        "r"(at), "l"(b), "r"(idesc), "r"(acc)
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(dt),
+        "r"(at), "l"(b), "r"(idesc), "r"(acc), "r"(on)
         : "memory");
 }
 
@@ -431,9 +437,9 @@ __global__ void __launch_bounds__(kResThreads, 1) attn_res_kernel(const __grid_c
                     const int ub = ubeg(c), u = ub + 2 * st, n = ubeg(c + 1) - u;  // this warp's units left: two of them now
                     const uint32_t pc = tmem + (uint32_t)(8 * (u + ub));
                     const uint64_t vd = dv + (uint64_t)(128 * u);
-                    if (issue && n > 0) {
-                        mma_ts(tmem + kOCol, pc, vd, id_o, (st | c) ? 1u : 0u);
-                        if (n > 1) mma_ts(tmem + kOCol, pc + 8u, vd + 128u, id_o, 1u);
+                    if (issue) {
+                        mma_ts(tmem + kOCol, pc, vd, id_o, (st | c) ? 1u : 0u, n > 0 ? 1u : 0u);
+                        mma_ts(tmem + kOCol, pc + 8u, vd + 128u, id_o, 1u, n > 1 ? 1u : 0u);
                     }
                     __syncwarp();
                 }
