@@ -286,6 +286,12 @@ int ilwdetr_validate_only(int32_t on);
  * while other threads launch GEMMs.  Call ilwdetr_debug_gemm_wait(-1, 0) to restore. */
 int ilwdetr_debug_gemm_wait(int32_t skip_load, int64_t wait_cycles);
 
+/* Test hook: which attention kernel ilwdetr_shiftmax_attn takes for these sizes (arguments as there).  *ctas is the
+ * number of CTAs that share a group's keys where it is the kernel whose scores stay in tensor memory, and 0 where it is
+ * another.  Asks the current device; launches nothing. */
+int ilwdetr_debug_attention_ctas(int32_t B, int32_t T, int32_t H, int32_t dh, int32_t win_side, int32_t qkv_form,
+                                 const ilw_shiftmax_t *p, int32_t *ctas);
+
 /* ------------------------------------------------------------------ encoder block */
 
 /* Integer parameters of one encoder block (all pointers are device pointers; weights packed

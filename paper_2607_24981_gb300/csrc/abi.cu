@@ -372,6 +372,17 @@ int ilwdetr_shiftmax_attn(const void *Q, const void *K, const void *V, int64_t l
     return cuda_status(ilw::launch_attention(ap, (cudaStream_t)stream), "shiftmax_attn");
 }
 
+int ilwdetr_debug_attention_ctas(int32_t B, int32_t T, int32_t H, int32_t dh, int32_t win_side, int32_t qkv_form,
+                                 const ilw_shiftmax_t *p, int32_t *ctas) {
+    if (!ctas || B < 1 || T < 1) return fail(ILW_ERR_INVALID_ARG, "debug_attention_ctas: NULL result or empty problem");
+    ilw::AttnParams ap;
+    const void *any = (const void *)256;  // (no pointer is looked at)
+    const int rc = attn_params(ap, any, any, any, (int64_t)H * dh, qkv_form, B, T, H, dh, win_side, p, 1, 1, (void *)any, 8,
+                               (int64_t)H * dh);
+    if (rc) return rc;
+    return cuda_status(ilw::attention_resident_ctas(ap, ctas), "debug_attention_ctas");
+}
+
 static int deform_params(ilw::DeformParams &dp, const int8_t *value, const int32_t *level_hw, int32_t L, const int32_t *ref_q16,
                         const int32_t *off_q8, const uint8_t *w, int32_t B, int32_t Q, int32_t H, int32_t P,
                         int32_t dh, int32_t m, int32_t s, int8_t *out) {
@@ -656,12 +667,13 @@ int ilwdetr_decoder_layer_forward(const ilw_decoder_params_t *p, const int16_t *
                                      stream));
         ilw::AttnParams ap;
         ILW_TRY(attn_params(ap, b.qkv, b.qkv + d, b.qkv + 2 * d, 3 * d, 8, B, Q, H, d / H, 0, &p->smx, p->m_o, p->s_o, b.o, 8, d));
-        // heads of 32 columns that the resident attention does not take run on the streaming one of
+        // heads of 32 columns that the resident attention cannot take run on the streaming one of
         // 64-column heads: q|k|v widened with zero columns (nothing added to q.k, zero outputs), the output
         // narrowed back.  The choice asks the device, so the checking pass checks both
         bool widened = false;
         if (d / H < 64 && !g_check_only) {
-            const cudaError_t e = ilw::launch_attention_res(ap, st, true);
+            int ctas;
+            const cudaError_t e = ilw::launch_attention_res(ap, st, INT64_MAX, &ctas);
             if (e != cudaSuccess && e != cudaErrorNotSupported) return cuda_status(e, "decoder attention");
             widened = e == cudaErrorNotSupported;
         }

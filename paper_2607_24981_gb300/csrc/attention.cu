@@ -12,6 +12,7 @@
 // fp32 accumulation is exact.  (On this GPU the fp16 warp MMA is about 3.8x faster than the int8
 // one.)  Q, K, V are read from HBM as int8 and converted while staged into shared memory; the
 // score fragments of pass 3 are already laid out as the A operand of P V.
+#include <algorithm>
 #include <climits>
 #include <cstdint>
 #include <cstdlib>
@@ -474,6 +475,44 @@ static bool attention_tc_enabled() {
     return on;
 }
 
+// The clocks of the other kernels, for the choice of the resident one.  All three were timed by graph replays on
+// 1 to 2400 (image, head) units of 1 to 3584 keys, 544 points; with these figures 16 of them take a kernel more than
+// 1.5 % slower than the fastest, 7 % at most.  (Before, groups of one key tile went to the resident kernel: 2400 units of
+// 64 keys, int8, 64 columns, 79 us against 45, 32 columns 76 against 29; and fp16 with 64 columns to the streaming one:
+// 77 us against 42, and 200 keys 336 against 175.)
+// Warp-MMA kernel, up to 256 keys: its key tiles of 64 in a CTA alone, or the CTAs of an SM one after another, of which
+// the first four overlap.  A last tile that is not whole costs extra.  (In us, int8: a CTA alone 3.5, 6.4 and 9.1 with 1,
+// 2 and 3 tiles of 64 columns, 2.1, 4.0 and 5.8 of 32; one of many 2.6, 4.2, 6.4 and 1.7, 3.1, 4.2.)
+static int64_t mma_clocks(const AttnParams &p, int Tg, int64_t units) {
+    if (Tg > 256) return INT64_MAX;
+    const int64_t kt = (Tg + 63) / 64, n = (units * kt + sm_count() - 1) / sm_count();
+    const bool ragged = Tg % 64 != 0;
+    const int64_t alone = (p.dh == 32 ? 600 + 3700 * kt : 1500 + 5700 * kt) + (ragged ? 3000 : 0);
+    const int64_t many = n * ((p.dh == 32 ? 800 + 2600 * kt : 1700 + 3600 * kt) + (ragged ? 600 : 0));
+    return std::max(alone, n > 2 && n <= 4 ? many * 7 / 8 : many);
+}
+// Streaming kernel: waves of two CTAs of 128 queries per SM; a last wave of one per SM takes 3 / 5 of a whole one.  (1600
+// keys 99 us a wave, 2300 119 to 122, 3584 165, 400 29.)
+static int64_t tc_clocks(const AttnParams &p, int Tg, int64_t units) {
+    if (!p.qkv_f16 || p.dh != 64) return INT64_MAX;
+    const int64_t sms = sm_count(), jobs = units * ((Tg + 127) / 128), wave = 15000 + 100 * (int64_t)Tg;
+    const int64_t last = jobs % (2 * sms);
+    return jobs / (2 * sms) * wave + (last == 0 ? 0 : (last <= sms ? wave * 3 / 5 : wave));
+}
+static int64_t other_clocks(const AttnParams &p) {
+    const int G2 = p.nw > 1 ? p.nw * p.nw : 1;
+    const int Tg = p.nw > 1 ? (p.grid_side / p.nw) * (p.grid_side / p.nw) : p.T;
+    const int64_t units = (int64_t)p.B * p.H * G2;
+    return std::min(mma_clocks(p, Tg, units), tc_clocks(p, Tg, units));
+}
+
+cudaError_t attention_resident_ctas(const AttnParams &p, int *ctas) {
+    *ctas = 0;
+    if (!attention_tc_enabled()) return cudaSuccess;
+    const cudaError_t e = launch_attention_res(p, nullptr, other_clocks(p), ctas);
+    return e == cudaErrorNotSupported ? cudaSuccess : e;
+}
+
 cudaError_t launch_attention(const AttnParams &p0, cudaStream_t s) {
     AttnParams p = p0;
     p.status = status_word_ptr();
@@ -481,8 +520,9 @@ cudaError_t launch_attention(const AttnParams &p0, cudaStream_t s) {
     const int Tg = p.nw > 1 ? (p.grid_side / p.nw) * (p.grid_side / p.nw) : p.T;
     if (p.B == 0 || Tg == 0) return cudaSuccess;
     if (attention_tc_enabled()) {
-        cudaError_t e = launch_attention_res(p, s);
-        if (e == cudaErrorNotSupported) e = launch_attention_tc(p, s);
+        cudaError_t e = launch_attention_res(p, s, other_clocks(p));
+        // (of one key tile the warp-MMA kernel is the faster)
+        if (e == cudaErrorNotSupported && (Tg > 64 || p.smx.s_d >= 0)) e = launch_attention_tc(p, s);
         if (e != cudaErrorNotSupported) return e;
     }
     dim3 grid((Tg + QT - 1) / QT, p.H, p.B * G2);

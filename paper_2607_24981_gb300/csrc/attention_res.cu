@@ -937,7 +937,7 @@ struct ResPlan {
     int64_t cost = 0;
 };
 template <int CS>
-cudaError_t plan_one(int Tg, int ws, int64_t jobs, ResPlan *best) {
+cudaError_t plan_one(int Tg, int ws, int64_t jobs, int job_cost, int key_cost, ResPlan *best) {
     int kpc, rpc;
     if (!res_split(Tg, ws, CS, &kpc, &rpc)) return cudaSuccess;
     const int nkp = (kpc + 15) / 16 * 16;
@@ -947,11 +947,14 @@ cudaError_t plan_one(int Tg, int ws, int64_t jobs, ResPlan *best) {
     const int nc = active_clusters<CS>(&e);
     if (e != cudaSuccess) return e;
     if (nc < 1) return cudaSuccess;
-    // rounds of jobs x the clocks of one: a part for the exchanges and one that grows with the CTA's keys
-    // (8 images x 6 heads: 155 us for 1600 keys over 4 CTAs, 266 over 8; 51 us for windows of 400 in one
-    // CTA, 78 over 2)
+    // clocks: rounds of jobs x those of one, a part for the exchanges and one that grows with the CTA's keys (more of
+    // both where the softmax warps load the rows themselves), and a cluster's launch.  Rounds measured, in us: fp16
+    // and 64 columns, one CTA, 64 keys 4.1, 192 5.3, 448 8.7; int8 5.0, 7.5, 10.3 (32 columns 4.8, 6.3); fp16 and 32
+    // columns 4.8, 7.6, 10.2; fp16, 64 columns, clusters of 4 with 400 keys a CTA 8.4, of 8 with 448 9.0.  A single
+    // job of 64 keys split over 4 CTAs takes 1.2 us longer than one of 48 in one CTA
     const int64_t rounds = (jobs + nc - 1) / nc;
-    const int64_t cost = rounds * ((CS > 1 ? 8500 : 8000) + 24 * (int64_t)nkp);
+    const int64_t one = job_cost + (CS > 1 ? 300 : 0) + key_cost * (int64_t)nkp;
+    const int64_t cost = rounds * one + (CS > 1 ? 2000 : 0);
     if (!best->cs || cost < best->cost) *best = {CS, kpc, rpc, (int)std::min<int64_t>(nc, jobs), cost};
     return cudaSuccess;
 }
@@ -978,7 +981,7 @@ cudaError_t launch_res(const ResArgs &a, int clusters, cudaStream_t s) {
 // The resident form: per-row s_d, which bounds sum P by 2^k_out and so |O| by 2^15 (with a static s_d
 // neither is bounded), scores of at most 64 columns (|s| <= 2^20) and at most 8 x 448 keys per group;
 // cudaErrorNotSupported otherwise.
-cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, bool plan_only) {
+cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, int64_t below, int *plan_ctas) {
     const ShiftExpC &se = p.smx.se;
     const bool win = p.nw > 1;
     const int ws = win ? p.grid_side / p.nw : 0, G2 = win ? p.nw * p.nw : 1;
@@ -995,16 +998,16 @@ cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, bool plan_
     a.jobs = (int32_t)jobs;
     ResPlan plan;
     cudaError_t e;
-    if ((e = plan_one<1>(Tg, ws, jobs, &plan)) != cudaSuccess || (e = plan_one<2>(Tg, ws, jobs, &plan)) != cudaSuccess ||
-        (e = plan_one<4>(Tg, ws, jobs, &plan)) != cudaSuccess || (e = plan_one<8>(Tg, ws, jobs, &plan)) != cudaSuccess)
+    a.tma = p.qkv_f16 && p.dh == 64;
+    const int jc = a.tma ? 6500 : (p.qkv_f16 ? 8200 : 7800), kc = a.tma ? 24 : (p.qkv_f16 ? 34 : 27);
+    if ((e = plan_one<1>(Tg, ws, jobs, jc, kc, &plan)) != cudaSuccess || (e = plan_one<2>(Tg, ws, jobs, jc, kc, &plan)) != cudaSuccess ||
+        (e = plan_one<4>(Tg, ws, jobs, jc, kc, &plan)) != cudaSuccess || (e = plan_one<8>(Tg, ws, jobs, jc, kc, &plan)) != cudaSuccess)
         return e;
-    if (!plan.cs) return cudaErrorNotSupported;
-    // the streaming kernel's clocks: waves of two CTAs per SM, 119 clocks per key (201 us for 8 x 6 units of
-    // 1600 keys).  It is ahead where a cluster of 8, which leaves a fifth of the SMs empty, meets many jobs
-    // (about 2300 keys, 8 images); it takes fp16-carried q|k|v with 64-column heads only
-    const int64_t waves = (jobs + 2 * sm_count() - 1) / (2 * sm_count());
-    if (p.qkv_f16 && p.dh == 64 && plan.cost > waves * Tg * 119) return cudaErrorNotSupported;
-    if (plan_only) return cudaSuccess;
+    if (!plan.cs || plan.cost > below) return cudaErrorNotSupported;
+    if (plan_ctas) {
+        *plan_ctas = plan.cs;
+        return cudaSuccess;
+    }
     a.kpc = plan.kpc;
     a.rpc = plan.rpc;
     a.ws_rcp = ws > 1 ? (uint32_t)((((uint64_t)1 << 32) + ws - 1) / ws) : 0u;  // ws = 1: a window is one token
@@ -1014,7 +1017,6 @@ cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, bool plan_
     if ((double)a.rcp * se.I0 < 1.0) a.rcp = std::nextafter(a.rcp, 2.0f);
     const int esz_o = p.o_f16 ? 2 : 1;
     a.ovec = (p.ld_o * esz_o) % 16 == 0 && ((uintptr_t)p.O % 16) == 0;
-    a.tma = p.qkv_f16 && p.dh == 64;
     if (a.tma && !(res_map(&a.qmap, p.Q, p, ws, win ? a.rqw : RQ) && res_map(&a.kmap, p.K, p, ws, win ? a.rpc : a.kbox) &&
                    res_map(&a.vmap, p.V, p, ws, win ? a.rpc : a.kbox)))
         return cudaErrorNotSupported;

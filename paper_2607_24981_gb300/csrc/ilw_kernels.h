@@ -161,10 +161,13 @@ cudaError_t launch_attention(const AttnParams &p, cudaStream_t s);
 // The tensor-memory (tcgen05) form for dh = 64 with fp16-carried q|k|v, 16-byte aligned rows and
 // windows of side <= 128; cudaErrorNotSupported when the problem is outside that.
 cudaError_t launch_attention_tc(const AttnParams &p, cudaStream_t s);
-// The form whose scores stay in tensor memory (groups of at most 2048 keys, per-row s_d; any q|k|v
-// carrier, dh 32 or 64); cudaErrorNotSupported when the problem is outside that.
-// plan_only: whether it would run (its sizes and parameters; no pointer is looked at)
-cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, bool plan_only = false);
+// The form whose scores stay in tensor memory (groups of at most 448 keys a CTA and 8 CTAs, for windows whole
+// window rows a CTA; per-row s_d; any q|k|v carrier, dh 32 or 64); cudaErrorNotSupported when the problem is
+// outside that or takes it more than `below` clocks by its own estimate.
+// plan_ctas: only whether it would run, and the CTAs that share a group (no pointer is looked at)
+cudaError_t launch_attention_res(const AttnParams &p, cudaStream_t s, int64_t below, int *plan_ctas = nullptr);
+// The CTAs that share a group where launch_attention takes the resident form, else 0
+cudaError_t attention_resident_ctas(const AttnParams &p, int *ctas);
 
 // ---------------------------------------------------------------- deformable sampling
 struct DeformParams {

@@ -1,6 +1,8 @@
 """Bit-exact parity of every CUDA entry point with the CPU oracle, element by element, on seeded
 inputs that span several tiles plus ragged tails, and on the edge cases of each operator.
 The whole path is integer, so the tolerance is zero everywhere."""
+import ctypes
+import os
 import time
 
 import numpy as np
@@ -11,6 +13,8 @@ from paper_2607_24981_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
+
+TENSOR_MEMORY = not os.environ.get("ILWDETR_ATTENTION_TC", "").startswith("0")
 
 
 @pytest.fixture(scope="module")
@@ -326,25 +330,57 @@ def test_int_layernorm_host_time_does_not_depend_on_steps(ilw):
     assert best(10) < 1.2 * best(20)
 
 
-@pytest.mark.parametrize("B,T,H,dh,win,form", [
-    (1, 1, 1, 64, 0, "f16"), (1, 16, 1, 64, 0, "f16"), (1, 33, 2, 32, 0, "f16"),  # one unit of 16 keys, a partial one
-    (2, 257, 1, 64, 0, "f16"), (1, 448, 1, 64, 0, "f16"),  # past one MMA's 256 keys, a CTA's 448
-    (1, 449, 1, 64, 0, "i8"), (1, 897, 1, 64, 0, "f16"), (1, 1793, 1, 64, 0, "f16"),  # clusters of 2, 4 and 8 CTAs
-    (1, 3585, 1, 64, 0, "f16"),                            # past a cluster of 8: the streaming kernel
-    (90, 40, 2, 32, 0, "i8"), (41, 130, 2, 64, 0, "f16"),  # several jobs per CTA, units changing
-    (12, 600, 2, 64, 0, "f16"), (5, 900, 3, 32, 0, "i8"),  # the same in clusters
-    (2, 900, 2, 64, 2, "i8"), (1, 5329, 1, 64, 1, "f16"), (1, 441, 2, 64, 21, "f16"), (2, 1764, 1, 32, 2, "f16")])
-def test_attention_resident_shapes(ilw, orc, B, T, H, dh, win, form):
-    """The kernel whose scores stay in tensor memory, at the edges of its tiles and of its split over
-    a cluster; images beyond the first few repeat them, and every repeat is compared."""
+def attention_ctas(ilw, B, T, H, dh, win, form, smx):
+    """The CTAs that share a group in the resident kernel; 0: another kernel takes the problem (every problem's is the
+    warp-MMA kernel under ILWDETR_ATTENTION_TC=0)."""
+    ctas = ctypes.c_int32(-1)
+    p = ilw.ShiftmaxT(*(smx[k] for k in ("I0", "k_inter", "k_out", "s_d", "m_p", "M_hw")))
+    assert ilw.lib().ilwdetr_debug_attention_ctas(B, T, H, dh, win, 8 if form == "i8" else ilw.I8_IN_F16, ctypes.byref(p),
+                                                  ctypes.byref(ctas)) == 0
+    return ctas.value
+
+
+def check_attention_images(ilw, orc, B, T, H, dh, win, form, smx):
+    """Every image against the oracle; images beyond the first few repeat them."""
     d, n = H * dh, min(B, 3)
     qkv = synth.uniform_int(16, f"qkvr{T}{H}{dh}", (n * T, 3 * d), -90, 90, np.int8)
     full = np.concatenate([qkv.reshape(n, -1)] * (B // n + 1))[:B].reshape(B * T, 3 * d)
-    smx = {"I0": 4000, "k_inter": 16, "k_out": 8, "s_d": -1, "m_p": 4, "M_hw": 31}
     got = host(ilw.shiftmax_attn(dev(full if form == "i8" else full.astype(np.float16)), B, T, H, dh, win, smx, 3 << 29, 36))
     want = orc.attention(qkv, n, T, H, dh, win, smx, 3 << 29, 36).reshape(n, -1)
     for b in range(B):
-        assert_same(got.reshape(B, -1)[b], want[b % n], f"resident T={T} win={win} image {b}")
+        assert_same(got.reshape(B, -1)[b], want[b % n], f"attention T={T} win={win} image {b}")
+
+
+@pytest.mark.parametrize("B,T,H,dh,win,form,ctas", [
+    (1, 1, 1, 64, 0, "f16", 1), (1, 16, 1, 64, 0, "f16", 1), (1, 33, 2, 64, 0, "f16", 1),  # one unit of 16 keys, a partial one
+    (2, 257, 1, 64, 0, "f16", 4), (40, 260, 2, 32, 0, "f16", 1),  # past one MMA's 256 keys
+    (30, 448, 2, 64, 0, "f16", 1), (1, 449, 1, 64, 0, "i8", 8),    # a CTA's 448 and past them
+    (8, 897, 2, 64, 0, "f16", 4), (1, 1793, 1, 64, 0, "f16", 8),   # clusters of 4 and 8 CTAs
+    (20, 890, 1, 64, 0, "f16", 2),                                 # of 2
+    (1, 3584, 1, 64, 0, "f16", 8), (1, 3585, 1, 64, 0, "f16", 0),  # the last of a cluster of 8, and past it
+    (90, 200, 2, 32, 0, "i8", 1), (82, 130, 2, 64, 0, "f16", 1),   # several jobs per CTA, units changing
+    (12, 600, 2, 64, 0, "f16", 2), (5, 900, 3, 32, 0, "i8", 4),    # the same in clusters
+    (2, 900, 2, 64, 2, "i8", 4), (1, 49, 2, 64, 7, "f16", 1), (2, 1764, 1, 32, 2, "f16", 4)])
+def test_attention_resident_shapes(ilw, orc, B, T, H, dh, win, form, ctas):
+    """The kernel whose scores stay in tensor memory, at the edges of its tiles and of its split over a cluster."""
+    smx = {"I0": 4000, "k_inter": 16, "k_out": 8, "s_d": -1, "m_p": 4, "M_hw": 31}
+    assert attention_ctas(ilw, B, T, H, dh, win, form, smx) == (ctas if TENSOR_MEMORY else 0)
+    check_attention_images(ilw, orc, B, T, H, dh, win, form, smx)
+
+
+@pytest.mark.parametrize("B,T,H,dh,win,form,resident", [
+    (600, 64, 2, 64, 0, "f16", False), (600, 64, 2, 64, 0, "i8", False), (200, 16, 2, 32, 0, "f16", False),
+    (100, 63, 2, 64, 0, "f16", False), (200, 1, 2, 64, 0, "i8", False), (4, 1600, 3, 64, 10, "f16", False),  # one key tile
+    (1, 64, 3, 32, 0, "i8", False), (1, 128, 3, 32, 0, "i8", False), (300, 65, 2, 64, 0, "f16", True),
+    (100, 100, 6, 64, 0, "f16", True), (100, 192, 6, 32, 0, "f16", False), (8, 300, 8, 32, 0, "i8", True),
+    (16, 2300, 6, 64, 0, "f16", False), (16, 1600, 6, 64, 0, "f16", True)])
+def test_attention_choice(ilw, orc, B, T, H, dh, win, form, resident):
+    """The kernel that was faster where all were timed, and the result of the short groups, whose kernel depends on the number
+    of groups and on the form of q|k|v."""
+    smx = {"I0": 4000, "k_inter": 16, "k_out": 8, "s_d": -1, "m_p": 4, "M_hw": 31}
+    assert (attention_ctas(ilw, B, T, H, dh, win, form, smx) > 0) == (resident and TENSOR_MEMORY)
+    if T <= 300 or win:
+        check_attention_images(ilw, orc, B, T, H, dh, win, form, smx)
 
 
 @pytest.mark.parametrize("I0,k_inter,k_out,m_p", [(1, 16, 8, 4), (3, 10, 4, 0), (700, 0, 8, 4), (16384, 16, 8, 4),
