@@ -291,23 +291,31 @@ __global__ void __launch_bounds__(256) top1_kernel(const int32_t *__restrict__ S
     }
 }
 
-// Row gather in 4-byte words: dst row i = row idx[i] of source i / n (src_rows rows each).  An index
+// Row gather in 4-byte words: dst row b n + i = row idx[b n + i] of source b (src_rows rows each); the blocks' y is
+// the source.  Bound by the division that finds a word's row (I: 32-bit where the words of a source's rows
+// allow it; 134400 rows of 256 bytes 17.9 us, 26.0 with 64 bits, 31.5 with a second one for the source).  An index
 // outside [0, src_rows) gives a zero row and latches kStatusBadIndex in the device status word.
+template <typename I>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint32_t *__restrict__ src, int64_t src_ldw,
                                                           int64_t src_rows, const int32_t *__restrict__ idx, int64_t n,
-                                                          int64_t batches, int64_t roww, uint32_t *__restrict__ dst,
+                                                          int64_t batches, I roww, uint32_t *__restrict__ dst,
                                                           int64_t dst_ldw, int *status) {
     grid_wait();
-    const int64_t total = n * batches * roww;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = t / roww, w = t - i * roww;
-        const int64_t r = idx[i];
-        if (r < 0 || r >= src_rows) {
-            dst[i * dst_ldw + w] = 0u;
-            if (w == 0 && status) atomicExch(status, kStatusBadIndex);
-            continue;
+    const I total = (I)n * roww;
+    for (int64_t b = blockIdx.y; b < batches; b += gridDim.y) {
+        const uint32_t *s = src + b * src_rows * src_ldw;
+        const int32_t *ix = idx + b * n;
+        uint32_t *d = dst + b * n * dst_ldw;
+        for (I t = blockIdx.x * (I)blockDim.x + threadIdx.x; t < total; t += (I)gridDim.x * blockDim.x) {
+            const I i = t / roww, w = t - i * roww;
+            const int64_t r = ix[i];
+            if (r < 0 || r >= src_rows) {
+                d[i * dst_ldw + w] = 0u;
+                if (w == 0 && status) atomicExch(status, kStatusBadIndex);
+                continue;
+            }
+            d[i * dst_ldw + w] = s[r * src_ldw + w];
         }
-        dst[i * dst_ldw + w] = src[((i / n) * src_rows + r) * src_ldw + w];
     }
 }
 
@@ -419,8 +427,13 @@ cudaError_t launch_topk(const int32_t *S, int64_t lds, int32_t rows, int32_t N, 
 cudaError_t launch_gather_rows(const void *src, int64_t src_ld_bytes, int64_t src_rows, const int32_t *idx, int64_t n,
                                int64_t batches, int64_t row_bytes, void *dst, int64_t dst_ld_bytes, cudaStream_t s) {
     if (n == 0 || batches == 0 || row_bytes == 0) return cudaSuccess;
-    launch_after(gather_rows_kernel, grid_for(n * batches * (row_bytes / 4), 256), 256, 0, s, (const uint32_t *)src, src_ld_bytes / 4, src_rows, idx, n, batches, row_bytes / 4, (uint32_t *)dst,
-        dst_ld_bytes / 4, status_word_ptr());
+    const dim3 grid(grid_for(n * (row_bytes / 4), 256), (unsigned)std::min<int64_t>(batches, 65535));
+    auto go = [&](auto kern, auto roww) {
+        launch_after(kern, grid, 256, 0, s, (const uint32_t *)src, src_ld_bytes / 4, src_rows, idx, n, batches, roww,
+                     (uint32_t *)dst, dst_ld_bytes / 4, status_word_ptr());
+    };
+    if (n * (row_bytes / 4) < (1ll << 31)) go(gather_rows_kernel<uint32_t>, (uint32_t)(row_bytes / 4));
+    else go(gather_rows_kernel<int64_t>, row_bytes / 4);
     return cudaGetLastError();
 }
 

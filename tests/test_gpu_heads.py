@@ -149,6 +149,15 @@ def test_gather_rows_batched(ilw, orc):
     same(host(ilw.gather_rows_batched(dev(X), dev(idx))), want, "batched gather")
 
 
+def test_gather_rows_batched_many_sources(ilw):
+    """More sources than a grid has blocks in y."""
+    B = 65535 + 4000
+    X = synth.uniform_int(77, "gatherm", (B * 3, 4), -128, 127, np.int8)
+    idx = synth.uniform_int(78, "gatherm.i", (B, 2), 0, 2)
+    want = X.reshape(B, 3, 4)[np.arange(B)[:, None], idx].reshape(2 * B, 4)
+    same(host(ilw.gather_rows_batched(dev(X), dev(idx))), want, "batched gather, many sources")
+
+
 def test_gather_rows(ilw, orc):
     X = synth.uniform_int(74, "gather", (1000, 6), -(1 << 30), 1 << 30)
     idx = synth.uniform_int(75, "gather.i", (777,), 0, 999)
