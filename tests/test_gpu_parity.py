@@ -351,6 +351,20 @@ def check_attention_images(ilw, orc, B, T, H, dh, win, form, smx):
         assert_same(got.reshape(B, -1)[b], want[b % n], f"attention T={T} win={win} image {b}")
 
 
+@pytest.mark.parametrize("C,lim", [(192, 1 << 20), (384, (1 << 24) - 1), (256, 1 << 23), (100, 1 << 16)])
+def test_int_layernorm_wide_values(ilw, orc, C, lim):
+    """int32 rows past 16 bits (up to the 2^24 that the operator takes): sums that fit 32 bits and sums that do not, of either sign, with the variance inside and
+    beyond the range whose root needs no steps, and V = s^2 + 2 s."""
+    rng = np.random.default_rng(C)
+    X = np.concatenate([rng.integers(-lim, lim, (20, C)), lim - rng.integers(0, 3, (20, C)), rng.integers(0, 3, (20, C)) - lim,
+                        np.full((20, C), -lim // 2) + rng.integers(-500, 500, (20, C))]).astype(np.int32)
+    X[-1], X[-1, :3] = lim // 2, [lim // 2 + 1, lim // 2 - 1, lim // 2 + 1]  # V = 3
+    beta, mult, shift = synth.ln_params(7, f"lnw{C}", C)
+    for iters in (10, 20):
+        got = ilw.int_layernorm(dev(X), dev(beta), dev(mult), dev(shift), iters, 8)
+        assert_same(host(got), orc.int_layernorm(X, beta, mult, shift, iters, 8), f"ln wide {C} {lim} {iters}")
+
+
 @pytest.mark.parametrize("B,T,H,dh,win,form,ctas", [
     (1, 1, 1, 64, 0, "f16", 1), (1, 16, 1, 64, 0, "f16", 1), (1, 33, 2, 64, 0, "f16", 1),  # one unit of 16 keys, a partial one
     (2, 257, 1, 64, 0, "f16", 4), (40, 260, 2, 32, 0, "f16", 1),  # past one MMA's 256 keys
