@@ -616,11 +616,10 @@ def roofline_entry(name, k, work, peaks, clocks, sms):
         a = w / avg_s / 1e12
         return {"kernel": name, "bound": "tensor", "achieved": a, "peak": peak, "unit": "TFLOP/s",
                 "frac": a / peak, "traffic": NCU_TRAFFIC.get(name), "peak_source": src}
-    # ALU: integer operations per score of the exact three-pass method (row maximum; ShiftExp and the
-    # int64 sum; ShiftExp again, the normalising multiply and shift, the fp16 P), the midpoint of the
-    # 30-40 that the method needs, against SMs x 128 lanes x the median SM clock; the figure at 16
-    # operations (ShiftExp counted once per score) is reported beside it
-    ops_per_score = 35.0
+    # ALU: integer operations per score with the scores kept (row maximum 1, ShiftExp 12, the sum 1, the output 2), as
+    # the kernel these launches run does it, against SMs x 128 lanes x the median SM clock.  (A kernel that streams the
+    # keys computes scores and ShiftExp again in every pass and needs 30-40.)
+    ops_per_score = 16.0
     mhz = clocks.get("sm_mhz") or 1500.0
     peak = sms * 128 * mhz * 1e6 / 1e12
     a = w * ops_per_score / avg_s / 1e12
