@@ -188,7 +188,6 @@ cudaError_t launch_pack_weight(const int8_t *W, int32_t N, int32_t K, void *pack
 cudaError_t launch_gemm(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s) {
     if (gp.M == 0 || gp.N == 0) return cudaSuccess;
     const bool gelu = ep.kind == EPI_GELU;
-    // 192-wide tiles when N splits evenly into them (fewer re-reads of A per flop), else 128
     // 64-wide tiles where the chip holds all of them at once: such a call is one tile's chain of latencies
     // and its operands at 64 bytes a clock and SM, both shorter for half the columns, and twice the SMs work
     // on it (12 layers of 1600 x 192: 331 us with 128 and 192 wide tiles, 294 with these where they fit; a decoder
@@ -200,6 +199,7 @@ cudaError_t launch_gemm(const GemmProblem &gp, const EpiParams &ep, cudaStream_t
         if (gp.a_f16) return gelu ? run_n64<true, true>(gp, ep, s) : run_n64<true, false>(gp, ep, s);
         return gelu ? run_n64<false, true>(gp, ep, s) : run_n64<false, false>(gp, ep, s);
     }
+    // else 192-wide tiles when N splits evenly into them (fewer re-reads of A per flop), else 128
     if (gp.a_f16) {
         // fp16 A: no conversion stage, so 192-wide tiles get 12 epilogue warps.  Weights resident
         // in shared memory when the CTA's BN rows of W fit next to the A stages (K <= 1024).

@@ -87,7 +87,7 @@ struct TcParams {  // CUtensorMap members keep the 64-byte alignment TMA needs
     int32_t tma_store;  // boxes per epilogue warp (2 or 1) of the outputs' TMA stores through shared memory; 0: plain stores
     int32_t dbg_skip;   // test hook: the producer issues no load for this K-block counter value (-1: none)
     long long wait_cycles;  // the bound of every wait (about one second, shorter for the test hook)
-    CUtensorMap cmap;   // C [M, N] with 16 x 32 boxes (2-byte outputs: 32-byte swizzle)
+    CUtensorMap cmap;   // C [M, N] with 32 x 32 boxes (2-byte outputs: 64-byte swizzle, 1-byte: 32-byte)
     CUtensorMap rmap;   // the int16 residual in 32 x 32 boxes (res_tma)
     int32_t res_tma;    // 1: each epilogue warp loads its residual box by TMA and writes its results over it
     int32_t stages;     // pipeline stages in use (STAGES at most)
@@ -454,16 +454,24 @@ __device__ __forceinline__ void box_words(uint8_t *box, int lane, int half, cons
     }
 }
 
-// Waits for this thread's TMEM loads; every register of v is marked as written by the wait.
-template <int NSEG>
-__device__ __forceinline__ void tmem_wait_all(uint32_t (&v)[NSEG][16]) {
-    tmem_wait_ld16(v[0]);
+// The residual pairs (x[2j] | x[2j+1] << 16) of 32 columns of a row starting at rrow + c0 (columns
+// at or past ncol read as 0; rvec: 16-byte aligned and all 32 present).
+__device__ __forceinline__ void res_group(const int16_t *rrow, int c0, int ncol, bool rvec, uint32_t (&rp)[16]) {
+    if (rrow && rvec && c0 + 32 <= ncol) {
 #pragma unroll
-    for (int sg = 1; sg < NSEG; ++sg)
-        asm volatile(""
-                     : "+r"(v[sg][0]), "+r"(v[sg][1]), "+r"(v[sg][2]), "+r"(v[sg][3]), "+r"(v[sg][4]), "+r"(v[sg][5]),
-                       "+r"(v[sg][6]), "+r"(v[sg][7]), "+r"(v[sg][8]), "+r"(v[sg][9]), "+r"(v[sg][10]), "+r"(v[sg][11]),
-                       "+r"(v[sg][12]), "+r"(v[sg][13]), "+r"(v[sg][14]), "+r"(v[sg][15])::"memory");
+        for (int j = 0; j < 4; ++j) {
+            const uint4 a = __ldg((const uint4 *)(rrow + c0) + j);
+            rp[4 * j] = a.x; rp[4 * j + 1] = a.y; rp[4 * j + 2] = a.z; rp[4 * j + 3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const int cl = c0 + 2 * j;
+            const uint32_t lo = (rrow && cl < ncol) ? (uint16_t)rrow[cl] : 0u;
+            const uint32_t hi = (rrow && cl + 1 < ncol) ? (uint16_t)rrow[cl + 1] : 0u;
+            rp[j] = lo | (hi << 16);
+        }
+    }
 }
 
 // The epilogue of one warp's part of a tile (its 32 rows x HALF columns) in the common case: a
@@ -494,26 +502,7 @@ __device__ __forceinline__ void tmem_wait_all(uint32_t (&v)[NSEG][16]) {
 // 12800 rows: 1152 x 384 to int8 in fp16 21.2 and 17.0 us (a 128 x 192 tile 5750 and 3300 clocks here),
 // 384 x 384 with residual 14.6 and 13.0, 1536 x 384 with SD-ShiftGELU 29.5 and 27.0; a 256-token block with
 // a shift of its own for every column (the 64-bit form then) 74 and 47.5 us.
-// The residual pairs (x[2j] | x[2j+1] << 16) of 32 columns of a row starting at rrow + c0 (columns
-// at or past ncol read as 0; rvec: 16-byte aligned and all 32 present).
-__device__ __forceinline__ void res_group(const int16_t *rrow, int c0, int ncol, bool rvec, uint32_t (&rp)[16]) {
-    if (rrow && rvec && c0 + 32 <= ncol) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint4 a = __ldg((const uint4 *)(rrow + c0) + j);
-            rp[4 * j] = a.x; rp[4 * j + 1] = a.y; rp[4 * j + 2] = a.z; rp[4 * j + 3] = a.w;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int cl = c0 + 2 * j;
-            const uint32_t lo = (rrow && cl < ncol) ? (uint16_t)rrow[cl] : 0u;
-            const uint32_t hi = (rrow && cl + 1 < ncol) ? (uint16_t)rrow[cl + 1] : 0u;
-            rp[j] = lo | (hi << 16);
-        }
-    }
-}
-
+//
 // box: this warp's one or two TMA-store boxes (nullptr: plain stores at dst), written out at column
 // x0 + 32 g, row y0 of cmap by lane 0 once every lane has written its row.
 template <int KIND, int BN, int HALF, int NSEG, int RES, int FORM>
