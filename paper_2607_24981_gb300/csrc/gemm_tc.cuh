@@ -520,7 +520,7 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
     constexpr int GPASS = (NSEG == 1 && RES == 0 && NG <= 2) ? NG : 1;
     static_assert(RES != 2 || (NG == 1 && KIND == KIND_RQ16), "one box holds the residual and the results");
     constexpr int esz = (KIND == KIND_RQ16 || KIND == KIND_F16OUT || KIND == KIND_GELU_F16) ? 2 : (KIND == KIND_RAW32 ? 4 : 1);
-    const int32_t lo = ep.relu ? 0 : -127;           // of int8 results
+    const int32_t lo = RES != 0 ? INT32_MIN : (ep.relu ? 0 : -127);  // of int8 results (a ReLU comes without a residual)
     const uint32_t lo_h = ep.relu ? 0u : 0xD7F0D7F0u;
     const int32_t r_rnd = RES != 0 ? 1 << (ep.s_r - 17) : 0, r_sh = RES != 0 ? ep.s_r - 16 : 0;
 #pragma unroll
@@ -718,23 +718,28 @@ __device__ __forceinline__ void epi_fast(const EpiParams &ep, uint32_t tbase, co
 // fp16 A needs no converters, and 128-wide tiles take four parts of 32 columns (a warp's whole residual is
 // in registers before the accumulators are ready, and 16 warps hide the chains of their loads; with two
 // parts the epilogue of a projection tile took 4900 clocks), 192-wide tiles three of 64.
-template <int BN, bool AF16>
-constexpr int epi_parts() { return AF16 ? (BN == 192 ? 3 : BN / 32) : 2; }
-template <int BN, bool AF16>
-constexpr int epi_warps() { return 4 * epi_parts<BN, AF16>(); }
-template <int BN, bool AF16>
-constexpr int tc_threads() { return 32 * ((AF16 ? 2 : 6) + epi_warps<BN, AF16>()); }
+// EP: that many parts instead (0: these).  128-wide tiles of fp16 A take two where 18 warps have no such loads to hide
+// and their 96 registers spill: raw accumulators, and of streamed weights int16 results without a residual box, int8
+// results with a residual and more than two accumulators.  (With four parts and with two: 12800 x 1536 x 384 to int16 27.3
+// and 21.6 us, 12800 x 2048 x 512 to int8 with a residual 48.8 and 44.6, 12800 x 128 x 4096 to int16 31.8 and 29.1, 51200 x 1100 x
+// 256 raw 123.7 and 104.9.)
+template <int BN, bool AF16, int EP>
+constexpr int epi_parts() { return EP ? EP : (AF16 ? (BN == 192 ? 3 : BN / 32) : 2); }
+template <int BN, bool AF16, int EP>
+constexpr int epi_warps() { return 4 * epi_parts<BN, AF16, EP>(); }
+template <int BN, bool AF16, int EP>
+constexpr int tc_threads() { return 32 * ((AF16 ? 2 : 6) + epi_warps<BN, AF16, EP>()); }
 
 template <int V>
 using Int = std::integral_constant<int, V>;
 
-template <int BN, int STAGES, int KIND, int NB, bool AF16, bool WRES>
-__global__ void __launch_bounds__(tc_threads<BN, AF16>(), 1) gemm_tc_kernel(const __grid_constant__ TcParams<NB> p) {
+template <int BN, int STAGES, int KIND, int NB, bool AF16, bool WRES, int EP>
+__global__ void __launch_bounds__(tc_threads<BN, AF16, EP>(), 1) gemm_tc_kernel(const __grid_constant__ TcParams<NB> p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     using SM = Smem<BN, AF16, WRES>;
     constexpr int kStage = SM::kStage;
-    constexpr int NP = epi_parts<BN, AF16>(), EPI0 = AF16 ? 2 : 6;  // column parts, first epilogue warp
+    constexpr int NP = epi_parts<BN, AF16, EP>(), EPI0 = AF16 ? 2 : 6;  // column parts, first epilogue warp
     constexpr int NWE = 4 * NP;
     const int nst = WRES ? p.stages : STAGES;  // pipeline stages
     uint8_t *wres = smem + nst * kStage;  // resident weights (WRES)
@@ -1266,21 +1271,21 @@ inline int num_sms() { return sm_count(); }
 
 // Dynamic shared memory of one instantiation (wres: resident weight bytes).
 // stg: the epilogue warps' TMA-store boxes (0 without TMA stores).
-template <int BN, int STAGES, int KIND, bool AF16, bool WRES>
+template <int BN, int STAGES, int KIND, bool AF16, bool WRES, int EP = 0>
 size_t smem_bytes(int wres, int stg = 0, int stages = STAGES) {
-    return 1024 + (size_t)stages * Smem<BN, AF16, WRES>::kStage + (WRES ? wres : 0) + 8 * (3 * STAGES + 6 + kMaxWk + epi_warps<BN, AF16>()) +
+    return 1024 + (size_t)stages * Smem<BN, AF16, WRES>::kStage + (WRES ? wres : 0) + 8 * (3 * STAGES + 6 + kMaxWk + epi_warps<BN, AF16, EP>()) +
            32 + 4 * prm_words<BN, WRES>() + (gelu_kind(KIND) ? 65536 : 0) + (stg ? 1024 + stg : 0);
 }
 constexpr size_t kSmemMax = 227 * 1024;
 
-template <int BN, int STAGES, int KIND, int NB, bool AF16, bool WRES>
+template <int BN, int STAGES, int KIND, int NB, bool AF16, bool WRES, int EP = 0>
 cudaError_t launch_tc(TcParams<NB> &tp, cudaStream_t s) {
     // TMA stores when the output allows them (set up by run) and their boxes fit next to the rest
-    constexpr int stg = epi_warps<BN, AF16>() * box_bytes<KIND>();
+    constexpr int stg = epi_warps<BN, AF16, EP>() * box_bytes<KIND>();
     tp.stages = STAGES;
     // (a part of one group of columns stores once a tile, long after the last tile's store: one box)
-    if (tp.tma_store) tp.tma_store = tp.res_tma || BN == 32 * epi_parts<BN, AF16>() ? 1 : 2;
-    auto bytes = [&](int boxes) { return smem_bytes<BN, STAGES, KIND, AF16, WRES>(tp.wres_bytes, boxes * stg, tp.stages); };
+    if (tp.tma_store) tp.tma_store = tp.res_tma || BN == 32 * epi_parts<BN, AF16, EP>() ? 1 : 2;
+    auto bytes = [&](int boxes) { return smem_bytes<BN, STAGES, KIND, AF16, WRES, EP>(tp.wres_bytes, boxes * stg, tp.stages); };
     // resident weights: as many stages as fit beside one box a warp (at least 3).  A's blocks come at L2's
     // latency, so the stages in flight set the rate: 12800 x 384 x 384 with 3 stages 600 clocks a K block
     while (WRES && tp.stages > 3 && bytes(tp.tma_store ? 1 : 0) > kSmemMax) --tp.stages;
@@ -1290,16 +1295,18 @@ cudaError_t launch_tc(TcParams<NB> &tp, cudaStream_t s) {
     if (smem > kSmemMax) return cudaErrorInvalidValue;
     static SmemLimit limit;
     const cudaError_t attr_err =
-        raise_smem_limit(limit, (const void *)gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES>, (int)kSmemMax);
+        raise_smem_limit(limit, (const void *)gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES, EP>, (int)kSmemMax);
     if (attr_err != cudaSuccess) return attr_err;
     int grid = tp.tiles < num_sms() ? tp.tiles : num_sms();
-    // a multiple of tiles_n: every CTA keeps one n block of W (WRES: always; else where that costs no round)
+    // a multiple of tiles_n: every CTA keeps one n block of W (WRES: always; else where that costs no round, and, for
+    // raw accumulators, which have no parameters to keep, where no CTA is left with the narrower last column block:
+    // 134400 x 320 x 320 of int8 A 98 us against 108)
     const int tiles_m = tp.tiles / tp.tiles_n;
     int per_n = num_sms() / tp.tiles_n;
     per_n = per_n < 1 ? 1 : (per_n > tiles_m ? tiles_m : per_n);
     const int whole = per_n * tp.tiles_n;
-    if (WRES || (whole <= grid && (tp.tiles + whole - 1) / whole == (tp.tiles + grid - 1) / grid)) grid = whole;
-    launch_after(gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES>, grid, tc_threads<BN, AF16>(), smem, s, tp);
+    if (WRES || (whole <= grid && (KIND != KIND_RAW32 || tp.N % BN == 0) && (tp.tiles + whole - 1) / whole == (tp.tiles + grid - 1) / grid)) grid = whole;
+    launch_after(gemm_tc_kernel<BN, STAGES, KIND, NB, AF16, WRES, EP>, grid, tc_threads<BN, AF16, EP>(), smem, s, tp);
     return cudaGetLastError();
 }
 
@@ -1365,7 +1372,7 @@ cudaError_t run(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s) {
     }
     // an int16 residual under int16 outputs by TMA, if its rows allow a map and no box wraps around
     tp.res_tma = 0;
-    if (tp.tma_store && ep.out_bits == 16 && ep.res && BN == 32 * epi_parts<BN, AF16>() && ((uintptr_t)ep.res % 16) == 0 && ep.ldr % 8 == 0 &&
+    if (tp.tma_store && ep.out_bits == 16 && ep.res && BN == 32 * epi_parts<BN, AF16, 0>() && ((uintptr_t)ep.res % 16) == 0 && ep.ldr % 8 == 0 &&
         ep.res_rows < (1ll << 31) && (ep.res_rows >= gp.M || ep.res_rows % 32 == 0))
         tp.res_tma = gemm_make_map(&tp.rmap, ep.res, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, ep.res_rows, gp.N, ep.ldr, 32, 32,
                                    CU_TENSOR_MAP_SWIZZLE_64B)
@@ -1391,9 +1398,14 @@ cudaError_t run(const GemmProblem &gp, const EpiParams &ep, cudaStream_t s) {
             if constexpr (NB == 1) return launch_tc<BN, STAGES, KIND_F16OUT, NB, AF16, WRES>(tp, s);
             else return cudaErrorInvalidValue;
         }
+        if constexpr (BN == 128 && NB == 1 && AF16 && !WRES) {  // two column parts: see epi_parts
+            if (nseg > 2) tp.res_tma = 0;
+            if (ep.out_bits == 8 && (ep.res || nseg > 2)) return launch_tc<BN, STAGES, KIND_RQ8, NB, AF16, WRES, 2>(tp, s);
+            if (ep.out_bits == 16 && !tp.res_tma) return launch_tc<BN, STAGES, KIND_RQ16, NB, AF16, WRES, 2>(tp, s);
+        }
         if (ep.out_bits == 8) return launch_tc<BN, STAGES, KIND_RQ8, NB, AF16, WRES>(tp, s);
         if (ep.out_bits == 16) return launch_tc<BN, STAGES, KIND_RQ16, NB, AF16, WRES>(tp, s);
-        return launch_tc<BN, STAGES, KIND_RAW32, NB, AF16, WRES>(tp, s);
+        return launch_tc<BN, STAGES, KIND_RAW32, NB, AF16, WRES, BN == 128 && NB == 1 && AF16 ? 2 : 0>(tp, s);  // (two column parts: see epi_parts)
     }
 }
 

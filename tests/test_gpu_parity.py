@@ -551,6 +551,33 @@ def test_gemm_store_boxes_over_tiles(ilw, orc, M, N, K, a_f16, out_bits):
     ilw.device_status()
 
 
+@pytest.mark.parametrize("M,N,K,out_bits,res", [
+    (5000, 200, 768, 16, ""), (5000, 200, 768, 8, "r"), (5000, 200, 768, 16, "r"), (5000, 200, 768, 16, "odd"), (4900, 136, 1104, 16, ""),
+    (9700, 136, 2112, 16, "r"), (9700, 136, 2112, 8, ""), (5000, 200, 768, 32, ""), (5000, 200, 128, 32, ""), (9700, 72, 2112, 32, "")])
+@pytest.mark.parametrize("spread", [False, True])
+def test_gemm_column_parts(ilw, orc, M, N, K, out_bits, res, spread):
+    """128-wide tiles of fp16 rows with two column parts (raw accumulators; streamed weights without a residual box,
+    with int8 residuals, with three accumulators) and with four (residual by TMA), one shift or (spread) one for every
+    column, columns past the last tile, residual rows that TMA takes and (odd) does not."""
+    n = 400
+    A = synth.uniform_int(25, f"cp{K}", (n, K), -127, 127, np.int8)
+    W, b, m, s = synth.gemm_params(25, f"cpW{N}{K}", N, K, 60.0, 30.0 if out_bits == 8 else 9000.0, "literal")
+    A[n // 2], W[N // 3] = 127, 127  # accumulators up to 127^2 K
+    s = (29 + np.arange(N) % 14).astype(s.dtype) if spread else np.full_like(s, s[0])
+    R = synth.uniform_int(25, f"cpr{N}", (n, N), -32768, 32767, np.int16) if res else None
+    want = dev(orc.gemm_requant(A, W, b, m, s, out_bits, R, 3 << 28, 30))
+    kw = {}
+    if res:
+        r_d = torch.zeros((M, N + 3 if res == "odd" else N), dtype=torch.int16, device="cuda")[:, :N]
+        r_d[:] = dev(R).repeat(M // n + 1, 1)[:M]
+        kw = dict(res=r_d, m_r=3 << 28, s_r=30)
+    A_d = dev(A.astype(np.float16)).repeat(M // n + 1, 1)[:M].contiguous()
+    got = ilw.gemm(A_d, ilw.pack_weight(dev(W)), N, dev(b), None if out_bits == 32 else dev(m), None if out_bits == 32 else dev(s),
+                   out_bits, **kw)
+    for r in range(0, M, n):
+        assert torch.equal(got[r:r + n].to(torch.int32), want[:min(n, M - r)].to(torch.int32)), r
+
+
 @pytest.mark.parametrize("s_r", [1, 16, 17, 46, 47, 48, 62])
 @pytest.mark.parametrize("M,N,a_f16", [(70, 200, False), (4000, 384, True)])  # 64-wide tiles, resident weights
 def test_gemm_residual_shifts(ilw, orc, M, N, a_f16, s_r):
