@@ -311,23 +311,21 @@ def test_attention_extreme_scores(ilw, orc):
 
 def test_int_layernorm_host_time_does_not_depend_on_steps(ilw):
     """The search for the roots that need no Newton steps (long at 10 steps, short at 20) is not part of a call: 200
-    calls of a short kernel take the host as long at either count (the best of 10; 14.5 and 10.2 us a call with
+    calls of a short kernel take the host as long at either count (the best of 20; 14.5 and 10.2 us a call with
     the search in each)."""
     x = torch.zeros((16, 192), dtype=torch.int16, device="cuda")
     out = torch.empty((16, 192), dtype=torch.int8, device="cuda")
     ln = [dev(a) for a in synth.ln_params(7, "lnhost", 192)]
 
-    def best(iters):
-        t = []
-        for _ in range(11):
-            torch.cuda.synchronize()
-            t0 = time.perf_counter()
-            for _ in range(200):
-                ilw.int_layernorm(x, *ln, iters, 8, out=out)
-            t.append(time.perf_counter() - t0)
-        return min(t[1:])
+    def calls(iters):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        for _ in range(200):
+            ilw.int_layernorm(x, *ln, iters, 8, out=out)
+        return time.perf_counter() - t0
 
-    assert best(10) < 1.2 * best(20)
+    t = [(calls(10), calls(20)) for _ in range(21)][1:]  # in turn: a busy host slows both
+    assert min(a for a, _ in t) < 1.2 * min(b for _, b in t)
 
 
 def attention_ctas(ilw, B, T, H, dh, win, form, smx):
@@ -387,13 +385,16 @@ def test_attention_resident_shapes(ilw, orc, B, T, H, dh, win, form, ctas):
     (100, 63, 2, 64, 0, "f16", False), (200, 1, 2, 64, 0, "i8", False), (4, 1600, 3, 64, 10, "f16", False),  # one key tile
     (1, 64, 3, 32, 0, "i8", False), (1, 128, 3, 32, 0, "i8", False), (300, 65, 2, 64, 0, "f16", True),
     (100, 100, 6, 64, 0, "f16", True), (100, 192, 6, 32, 0, "f16", False), (8, 300, 8, 32, 0, "i8", True),
-    (16, 2300, 6, 64, 0, "f16", False), (16, 1600, 6, 64, 0, "f16", True)])
+    (16, 2300, 6, 64, 0, "f16", False), (16, 1600, 6, 64, 0, "f16", True),
+    (1, 33, 2, 32, 0, "f16", False), (1, 448, 1, 64, 0, "f16", True), (1, 897, 1, 64, 0, "f16", True),
+    (90, 40, 2, 32, 0, "i8", False), (41, 130, 2, 64, 0, "f16", True), (1, 5329, 1, 64, 1, "f16", False),
+    (1, 441, 2, 64, 21, "f16", False)])
 def test_attention_choice(ilw, orc, B, T, H, dh, win, form, resident):
     """The kernel that was faster where all were timed, and the result of the short groups, whose kernel depends on the number
     of groups and on the form of q|k|v."""
     smx = {"I0": 4000, "k_inter": 16, "k_out": 8, "s_d": -1, "m_p": 4, "M_hw": 31}
     assert (attention_ctas(ilw, B, T, H, dh, win, form, smx) > 0) == (resident and TENSOR_MEMORY)
-    if T <= 300 or win:
+    if B * T < 10000 or T <= 300 or win:
         check_attention_images(ilw, orc, B, T, H, dh, win, form, smx)
 
 
